@@ -24,8 +24,8 @@
  *    is row-major [ny][nx] (x fastest).
  *  - Grid (§6.1): x_j = j Lx/nx; spectral derivatives D = F^{-1}(iK)F with
  *    k_j = 2 pi j/L, j = -n/2+1..n/2-1, and the n/2 wavenumber set to 0.
- *    Sizes: a power of two (1d 8 <= nx <= 16384, where nx = 16384 runs each solve and
- *    right-hand side on a thread-block cluster of two CTAs; 2d 8 <= nx, ny <= 1024), or
+ *    Sizes: a power of two (1d 8 <= nx <= 16384, where from nx = 256 a solve or right-hand
+ *    side may run on a thread-block cluster of up to eight CTAs; 2d 8 <= nx, ny <= 1024), or
  *    n = 2^a 3^b 5^c with a >= 1 (1d 6 <= nx <= 16384; 2d 6 <= nx, ny <= 1024) on generic
  *    kernels (see sgn_layout_create for what they serve).
  */
@@ -132,12 +132,14 @@ void sgn_layout_destroy(sgn_layout* lay);
 /* Total packed points P (per component). */
 long long sgn_layout_points(const sgn_layout* lay);
 /* Kernel forms of a 1d layout's size classes.  The solve and the right-hand side of the
- * instances of n = 2^log2n run on one CTA per instance (ctas = 1, n <= 8192) or on a
- * thread-block cluster of two CTAs per instance that splits the instance's points and
- * modes between them (ctas = 2, n = 4096, 8192 and 16384; the only form of n = 16384).
- * The two forms agree up to rounding (their dot products add in another order).  A batch
- * that fills the GPU runs fastest on one CTA per instance; a few large instances run with
- * less latency on clusters.  Default: 1 below n = 16384.  set_form: SGN_ERR_INVALID_ARG on
+ * instances of n = 2^log2n run in the library's own form (ctas = 1, n <= 8192): up to n = 128
+ * one CTA per instance, above it a cluster of up to eight CTAs that splits the instance's
+ * points and modes, as many as the layout's other instances leave SMs for, with bitwise the
+ * same result for every number; or on a cluster of exactly two CTAs that splits them by
+ * halves and by parity (ctas = 2, n = 4096 and 8192).  The two forms agree up to rounding
+ * (their dot products add in another order).  n = 16384 has the library's own form only, which
+ * set_form and get_form name ctas = 2, as it always takes a cluster.  Default: 1 below
+ * n = 16384.  set_form: SGN_ERR_INVALID_ARG on
  * a 2d layout or bad arguments, SGN_ERR_UNSUPPORTED_SIZE for a form the size lacks.
  * States step with the new forms from their next step. */
 sgn_status sgn_layout_set_form(sgn_layout* lay, int log2n, int ctas);
@@ -362,7 +364,7 @@ sgn_status sgn_state_set_dealias(sgn_state* st, int on);
  * problem: for every combination of forms of the n = 4096 and 8192 classes (solve and
  * right-hand side chosen separately: up to 16 combinations), one untimed and three timed
  * RK4 steps with these dt (HOST [count]) and options, each from the same state, in two
- * passes keeping each combination's faster one.  The default (one CTA per instance) stays
+ * passes keeping each combination's faster one.  The default (the library's own form) stays
  * unless another combination is at least 3% faster; the choice stays set on the layout.
  * The state (eta, U, u, time, counters) is restored afterwards, so tuning leaves no trace
  * on the solution.  Allocates and frees 3 P doubles; synchronises `stream`; best_ms

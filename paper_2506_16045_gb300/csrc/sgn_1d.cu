@@ -527,13 +527,14 @@ cudaError_t launch_linimp_step1d(const Layout1d& lay, const void* tw64, const vo
                         : tw64;
   return for_each_class(lay, s, [&](auto NTc, auto MBc, int l, int first, int num, cudaStream_t s) {
     constexpr int NT = decltype(NTc)::value, MB = decltype(MBc)::value;
-    const bool gl = l > kSmemLog1d;                // transform buffer in global scratch
-    const size_t sm = gl ? 0 : (size_t)16 << l;    // cplx<double> and cplx<df>: 16 bytes
-    cplx<double>* big = gl ? static_cast<cplx<double>*>(lay.big) : nullptr;
+    if (l >= kSplitLog1d)
+      return launch_linimp_split(lay, l, first, num, tw64, tw32, precision, A, eta, hx, u, U,
+                                 res0_hat, res1_hat, c1, c0, solve, u_out ? u_out : u, ux_out, s);
+    const size_t sm = (size_t)16 << l;             // cplx<double> and cplx<df>: 16 bytes
     auto run = [&](auto kern, auto twp) -> cudaError_t {
       cudaError_t e = set_smem(kern, sm);
       if (e) return e;
-      kern<<<num, NT, sm, s>>>(lay.d_inst, lay.d_ids + first, big, twp, A, eta, hx, u, U,
+      kern<<<num, NT, sm, s>>>(lay.d_inst, lay.d_ids + first, nullptr, twp, A, eta, hx, u, U,
                                static_cast<const cplx<double>*>(res0_hat),
                                static_cast<cplx<double>*>(res1_hat), c1, c0,
                                static_cast<cplx<double>*>(ws), u_out ? u_out : u, ux_out);

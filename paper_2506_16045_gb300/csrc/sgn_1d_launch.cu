@@ -1,8 +1,9 @@
 // Launchers of the register-FFT 1d kernels: one launch per size class.  The kernels
-// (sgn_1d_pcg.cuh: a5/a6 solve, sgn_1d_rhs.cuh: a7 right-hand side) are instantiated per
-// size in the sgn_1d_l*.cu translation units, which compile in parallel.
+// (sgn_1d_pcg.cuh: a5/a6 solve, sgn_1d_rhs.cuh: a7 right-hand side; sgn_split_1d.cuh from
+// n = 256) are instantiated per size in the sgn_1d_*.cu and sgn_split_*.cu translation units, which compile in parallel.
 #include "sgn_1d_pcg.cuh"
 #include "sgn_1d_rhs.cuh"
+#include "sgn_split_1d.cuh"
 
 namespace sgn {
 
@@ -11,40 +12,85 @@ extern template cudaError_t pcg1d_launch<4, 1>(const PcgArgs&, int, int, cudaStr
 extern template cudaError_t pcg1d_launch<5, 1>(const PcgArgs&, int, int, cudaStream_t);
 extern template cudaError_t pcg1d_launch<6, 1>(const PcgArgs&, int, int, cudaStream_t);
 extern template cudaError_t pcg1d_launch<7, 1>(const PcgArgs&, int, int, cudaStream_t);
-extern template cudaError_t pcg1d_launch<8, 1>(const PcgArgs&, int, int, cudaStream_t);
-extern template cudaError_t pcg1d_launch<9, 1>(const PcgArgs&, int, int, cudaStream_t);
-extern template cudaError_t pcg1d_launch<10, 1>(const PcgArgs&, int, int, cudaStream_t);
-extern template cudaError_t pcg1d_launch<11, 1>(const PcgArgs&, int, int, cudaStream_t);
-extern template cudaError_t pcg1d_launch<12, 1>(const PcgArgs&, int, int, cudaStream_t);
-extern template cudaError_t pcg1d_launch<13, 1>(const PcgArgs&, int, int, cudaStream_t);
 extern template cudaError_t pcg1d_launch<12, 2>(const PcgArgs&, int, int, cudaStream_t);
 extern template cudaError_t pcg1d_launch<13, 2>(const PcgArgs&, int, int, cudaStream_t);
-extern template cudaError_t pcg1d_launch<14, 2>(const PcgArgs&, int, int, cudaStream_t);
 extern template cudaError_t rhs1d_launch<3, 1>(const RhsArgs&, int, int, cudaStream_t);
 extern template cudaError_t rhs1d_launch<4, 1>(const RhsArgs&, int, int, cudaStream_t);
 extern template cudaError_t rhs1d_launch<5, 1>(const RhsArgs&, int, int, cudaStream_t);
 extern template cudaError_t rhs1d_launch<6, 1>(const RhsArgs&, int, int, cudaStream_t);
 extern template cudaError_t rhs1d_launch<7, 1>(const RhsArgs&, int, int, cudaStream_t);
-extern template cudaError_t rhs1d_launch<8, 1>(const RhsArgs&, int, int, cudaStream_t);
-extern template cudaError_t rhs1d_launch<9, 1>(const RhsArgs&, int, int, cudaStream_t);
-extern template cudaError_t rhs1d_launch<10, 1>(const RhsArgs&, int, int, cudaStream_t);
-extern template cudaError_t rhs1d_launch<11, 1>(const RhsArgs&, int, int, cudaStream_t);
-extern template cudaError_t rhs1d_launch<12, 1>(const RhsArgs&, int, int, cudaStream_t);
-extern template cudaError_t rhs1d_launch<13, 1>(const RhsArgs&, int, int, cudaStream_t);
 extern template cudaError_t rhs1d_launch<12, 2>(const RhsArgs&, int, int, cudaStream_t);
 extern template cudaError_t rhs1d_launch<13, 2>(const RhsArgs&, int, int, cudaStream_t);
-extern template cudaError_t rhs1d_launch<14, 2>(const RhsArgs&, int, int, cudaStream_t);
+extern template cudaError_t split_pcg_launch<8>(const PcgArgs&, int, int, int, cudaStream_t);
+extern template cudaError_t split_rhs_launch<8>(const RhsArgs&, int, int, int, cudaStream_t);
+extern template cudaError_t split_linimp_launch<8>(const sp::LinArgs&, int, int, int,
+                                                     cudaStream_t);
+extern template cudaError_t split_pcg_launch<9>(const PcgArgs&, int, int, int, cudaStream_t);
+extern template cudaError_t split_rhs_launch<9>(const RhsArgs&, int, int, int, cudaStream_t);
+extern template cudaError_t split_linimp_launch<9>(const sp::LinArgs&, int, int, int,
+                                                     cudaStream_t);
+extern template cudaError_t split_pcg_launch<10>(const PcgArgs&, int, int, int, cudaStream_t);
+extern template cudaError_t split_rhs_launch<10>(const RhsArgs&, int, int, int, cudaStream_t);
+extern template cudaError_t split_linimp_launch<10>(const sp::LinArgs&, int, int, int,
+                                                     cudaStream_t);
+extern template cudaError_t split_pcg_launch<11>(const PcgArgs&, int, int, int, cudaStream_t);
+extern template cudaError_t split_rhs_launch<11>(const RhsArgs&, int, int, int, cudaStream_t);
+extern template cudaError_t split_linimp_launch<11>(const sp::LinArgs&, int, int, int,
+                                                     cudaStream_t);
+extern template cudaError_t split_pcg_launch<12>(const PcgArgs&, int, int, int, cudaStream_t);
+extern template cudaError_t split_rhs_launch<12>(const RhsArgs&, int, int, int, cudaStream_t);
+extern template cudaError_t split_linimp_launch<12>(const sp::LinArgs&, int, int, int,
+                                                     cudaStream_t);
+extern template cudaError_t split_pcg_launch<13>(const PcgArgs&, int, int, int, cudaStream_t);
+extern template cudaError_t split_rhs_launch<13>(const RhsArgs&, int, int, int, cudaStream_t);
+extern template cudaError_t split_linimp_launch<13>(const sp::LinArgs&, int, int, int,
+                                                     cudaStream_t);
+extern template cudaError_t split_pcg_launch<14>(const PcgArgs&, int, int, int, cudaStream_t);
+extern template cudaError_t split_rhs_launch<14>(const RhsArgs&, int, int, int, cudaStream_t);
+extern template cudaError_t split_linimp_launch<14>(const sp::LinArgs&, int, int, int,
+                                                     cudaStream_t);
+
+// log2 of the CTAs per instance of class l.  At least 2048 points per CTA stay together; from
+// there the classes are halved, the one with the largest share per CTA first, while every CTA
+// still has an SM of its own (one instance: up to 8 CTAs).  Splitting further than the SMs
+// would only add exchanges: two CTAs on an SM share its issue slots and its float64 pipe.
+int split_lcl(const Layout1d& lay, int l) {
+  int lcl[16], total = 0;
+  for (int c = 0; c < 16; ++c) {
+    const int num = lay.class_end[c] - lay.class_begin[c];
+    lcl[c] = c > 11 ? c - 11 : 0;
+    total += num << lcl[c];
+  }
+  for (;;) {
+    int best = -1;
+    for (int c = kSplitLog1d; c <= kMaxLog1d; ++c)
+      if (lay.class_end[c] > lay.class_begin[c] && lcl[c] < 3 &&
+          (best < 0 || c - lcl[c] >= best - lcl[best]))
+        best = c;
+    if (best < 0) break;
+    const int num = lay.class_end[best] - lay.class_begin[best];
+    if (total + (num << lcl[best]) > kSMs) break;
+    total += num << lcl[best];
+    lcl[best] += 1;
+  }
+  return lcl[l];
+}
 
 namespace {
 
-// The form of size class LG in this layout: one CTA per instance, or a two-CTA cluster
-// (n = 4096 and 8192 by choice, for the solve and the right-hand side separately;
-// n = 16384 always).  The solve's u_x hand-off is stored in natural point order by either
-// form, so the two kernels may take different forms.
+// The form of size class LG in this layout: up to n = 128 one CTA per instance; above, the
+// split kernels with the CTAs per instance that split_lcl chooses, or, where set_form(s) asked
+// for two CTAs (n = 4096 and 8192, solve and right-hand side separately), the two-CTA
+// clusters of sgn_1d_pcg.cuh and sgn_1d_rhs.cuh.  The solve's u_x hand-off is stored in natural
+// point order by every form, so the two kernels may take different forms.
 struct PcgKernels {
   template <int LG, int CL>
   static cudaError_t go(const PcgArgs& a, int first, int num, cudaStream_t s) {
     return pcg1d_launch<LG, CL>(a, first, num, s);
+  }
+  template <int LG>
+  static cudaError_t split(const PcgArgs& a, int first, int num, int lcl, cudaStream_t s) {
+    return split_pcg_launch<LG>(a, first, num, lcl, s);
   }
   static int ctas(const Layout1d& lay, int l) { return lay.ctas(l); }
 };
@@ -53,17 +99,20 @@ struct RhsKernels {
   static cudaError_t go(const RhsArgs& a, int first, int num, cudaStream_t s) {
     return rhs1d_launch<LG, CL>(a, first, num, s);
   }
+  template <int LG>
+  static cudaError_t split(const RhsArgs& a, int first, int num, int lcl, cudaStream_t s) {
+    return split_rhs_launch<LG>(a, first, num, lcl, s);
+  }
   static int ctas(const Layout1d& lay, int l) { return lay.rhs_ctas(l); }
 };
 
 template <int LG, typename K, typename Args>
 cudaError_t launch_form(const Layout1d& lay, const Args& a, int first, int num, cudaStream_t s,
                         K) {
-  if constexpr (LG > kSmemLog1d) {
-    return K::template go<LG, 2>(a, first, num, s);
-  } else if constexpr (LG >= kClusterLog1d) {
-    return K::ctas(lay, LG) == 2 ? K::template go<LG, 2>(a, first, num, s)
-                             : K::template go<LG, 1>(a, first, num, s);
+  if constexpr (LG >= kSplitLog1d) {
+    if constexpr (LG >= kClusterLog1d && LG <= kSmemLog1d)
+      if (K::ctas(lay, LG) == 2) return K::template go<LG, 2>(a, first, num, s);
+    return K::template split<LG>(a, first, num, split_lcl(lay, LG), s);
   } else {
     return K::template go<LG, 1>(a, first, num, s);
   }
@@ -175,6 +224,43 @@ cudaError_t launch_rhs1d_ux(const Layout1d& lay, const void* tw64, const void* t
   }, [&](int first, int num, cudaStream_t cs) {
     return mr_launch_rhs(lay, first, num, precision, g, eta, u, h, hx, f_eta, f_U, scratch, cs);
   });
+}
+
+cudaError_t launch_linimp_split(const Layout1d& lay, int l, int first, int num, const void* tw64,
+                                const void* tw32, int precision, const SolveRec* A,
+                                const double* eta, const double* hx, const double* u,
+                                const double* U, const void* res0_hat, void* res1_hat, double c1,
+                                double c0, bool solve, double* u_out, void* ux_out,
+                                cudaStream_t s) {
+  sp::LinArgs a;
+  a.insts = lay.d_inst;
+  a.ids = lay.d_ids;
+  a.tw64 = static_cast<const cplx<double>*>(tw64);
+  a.twdf = reinterpret_cast<const cplx<df>*>(static_cast<const char*>(tw32) + kTw32Bytes);
+  a.A = A;
+  a.eta = eta;
+  a.hx = hx;
+  a.u = u;
+  a.U = U;
+  a.res0 = static_cast<const cplx<double>*>(res0_hat);
+  a.res1 = static_cast<cplx<double>*>(res1_hat);
+  a.c1 = c1;
+  a.c0 = c0;
+  a.u_out = u_out;
+  a.ux = ux_out;
+  a.precision = precision;
+  a.solve = solve;
+  const int lcl = split_lcl(lay, l);
+  switch (l) {
+    case 8: return split_linimp_launch<8>(a, first, num, lcl, s);
+    case 9: return split_linimp_launch<9>(a, first, num, lcl, s);
+    case 10: return split_linimp_launch<10>(a, first, num, lcl, s);
+    case 11: return split_linimp_launch<11>(a, first, num, lcl, s);
+    case 12: return split_linimp_launch<12>(a, first, num, lcl, s);
+    case 13: return split_linimp_launch<13>(a, first, num, lcl, s);
+    case 14: return split_linimp_launch<14>(a, first, num, lcl, s);
+    default: return cudaErrorInvalidValue;
+  }
 }
 
 }  // namespace sgn

@@ -478,9 +478,11 @@ __device__ __forceinline__ double block_min(double v, double* scratch) {
 // shared-memory writes before it are visible to the partner CTA after it), the CTA's rank,
 // and the partner CTA's copy of a shared-memory object in a cluster of two.
 // -------------------------------------------------------------------------------------
+// The intrinsics, not inline PTX: they are convergent operations to the compiler, which may
+// otherwise duplicate a barrier into the branches around it.
 __device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;"
-               ::: "memory");
+  __cluster_barrier_arrive();
+  __cluster_barrier_wait();
 }
 __device__ __forceinline__ unsigned cluster_rank() { return __clusterRelativeBlockRank(); }
 template <typename P>

@@ -43,6 +43,8 @@ constexpr int kWsVectors = 6;          // half-spectrum vectors per instance in 
 constexpr int kMaxLog1d = 14;          // 1d n <= 16384 (n = 16384: two-CTA clusters)
 constexpr int kSmemLog1d = 13;         // largest 1d n whose float64 transform fits in one CTA
 constexpr int kClusterLog1d = 12;      // smallest 1d log2 n with a two-CTA cluster form
+constexpr int kSplitLog1d = 8;         // smallest 1d log2 n of the split kernels
+constexpr int kSMs = 152;              // streaming multiprocessors of a GB300
 constexpr int kGenericClass = 0;       // size class of the 1d n that are not powers of two
 // The size classes in launch order: the largest power of two first, the generic class last.
 constexpr int kNumClassSlots = kMaxLog1d - 3 + 2;
@@ -81,6 +83,9 @@ struct Layout1d {
   cudaEvent_t fork = nullptr;
   cudaEvent_t join[16] = {nullptr};
 };
+
+// log2 of the CTAs per instance that class l's split kernels take (sgn_1d_launch.cu)
+int split_lcl(const Layout1d& lay, int l);
 
 // Launchers (all asynchronous on `stream`; return cudaError_t of the launch).
 cudaError_t twiddles_init(void* tw64, void* tw32, cudaStream_t s);
@@ -143,6 +148,13 @@ cudaError_t launch_linimp_step1d(const Layout1d& lay, const void* tw64, const vo
                                  const void* res0_hat, void* res1_hat, double c1, double c0,
                                  bool solve, void* ws, double* u_out, void* ux_out,
                                  cudaStream_t s);
+// the same for the instances ids[first, first + num) of class l >= kSplitLog1d
+cudaError_t launch_linimp_split(const Layout1d& lay, int l, int first, int num, const void* tw64,
+                                const void* tw32, int precision, const SolveRec* A,
+                                const double* eta, const double* hx, const double* u,
+                                const double* U, const void* res0_hat, void* res1_hat, double c1,
+                                double c0, bool solve, double* u_out, void* ux_out,
+                                cudaStream_t s);
 
 // Sizes n = 2^a 3^b 5^c (a >= 1) that are not powers of two, 6 <= n <= 16384: one CTA per
 // instance with a mixed-radix transform in shared memory (n <= 6144; above, in global
