@@ -23,16 +23,20 @@ using d1::kPi;
 using mr::MrPlan;
 using mr::mr_plan;
 using mr::k_mr_twiddles;
-constexpr int kMrNT = 256;
+constexpr int kMrNT = 512;
 constexpr int kMrMaxN = 16384;       // largest generic n
 constexpr int kMrSmemN = 6144;       // largest n whose two transform buffers (192 KB) are in
                                      // shared memory; above it they are in global memory
 
-// wavenumber of mode m (Nyquist 0), in T
+// wavenumber of mode m (Nyquist 0), in T: ku = 2 pi / L in T.  No float64 in the float32 and
+// double-float forms (a float64 operation costs 62 float32 ones here, and a wavenumber is
+// formed for every mode of every transform).
 template <typename T>
-__device__ __forceinline__ T mr_k(int m, int n, double kunit) {
-  return num<T>(kunit * (double)wave_index(m, n));
+__device__ __forceinline__ T mr_k(int m, int n, T ku) {
+  return ku * from_int<T>(wave_index(m, n));
 }
+// the mirror n - m of mode m
+__device__ __forceinline__ int mr_mirror(int m, int n) { return m == 0 ? 0 : n - m; }
 
 struct MrTw {            // the instance's twiddle tables (n - 1 entries each)
   const cplx<double>* d;
@@ -77,8 +81,8 @@ __device__ __forceinline__ cplx<T>* mr_deriv_pair(cplx<T>* A, cplx<T>* B, const 
                                                   double kunit, const cplx<T>* tw) {
   const int n = P.n;
   cplx<T>* F = mr::mr_fft<T, kMrNT>(A, B, P, false, tw);
-  const double inv_n = 1.0 / n;
-  for (int m = threadIdx.x; m < n; m += kMrNT) F[m] = mul_pi(F[m]) * num<T>(kunit * wave_index(m, n) * inv_n);
+  const T kn = num<T>(kunit / n);
+  for (int m = threadIdx.x; m < n; m += kMrNT) F[m] = mul_pi(F[m]) * mr_k<T>(m, n, kn);
   __syncthreads();
   return mr::mr_fft<T, kMrNT>(F, F == A ? B : A, P, true, tw);
 }
@@ -103,11 +107,11 @@ __global__ void __launch_bounds__(kMrNT) k_mr_deriv(const MrArgs A, const double
 // w - q_x).  Writes the half spectrum m = 0..n/2 of G v into out (T arithmetic).  c: the
 // coefficients c1, c2, c3 at point j.
 template <typename T, typename Coef>
-__device__ void mr_matvec(cplx<T>* a, cplx<T>* b, const MrPlan& P, double kunit,
+__device__ void mr_matvec(cplx<T>* a, cplx<T>* b, const MrPlan& P, T ku,
                           const cplx<T>* tw, Coef coef, cplx<T>* out) {
   const int n = P.n, h = n / 2;
   // a holds V (full spectrum); form (1 - k) V in place
-  for (int m = threadIdx.x; m < n; m += kMrNT) a[m] = a[m] * (num<T>(1.0) - mr_k<T>(m, n, kunit));
+  for (int m = threadIdx.x; m < n; m += kMrNT) a[m] = a[m] * (num<T>(1.0) - mr_k<T>(m, n, ku));
   __syncthreads();
   cplx<T>* z = mr::mr_fft<T, kMrNT>(a, b, P, true, tw);
   const T inv_n = num<T>(1.0 / n);
@@ -120,8 +124,8 @@ __device__ void mr_matvec(cplx<T>* a, cplx<T>* b, const MrPlan& P, double kunit,
   __syncthreads();
   cplx<T>* Y = mr::mr_fft<T, kMrNT>(z, z == a ? b : a, P, false, tw);
   for (int m = threadIdx.x; m <= h; m += kMrNT) {
-    const T k = mr_k<T>(m, n, kunit);
-    const cplx<T> y = Y[m], ym = conj(Y[(n - m) % n]);
+    const T k = mr_k<T>(m, n, ku);
+    const cplx<T> y = Y[m], ym = conj(Y[mr_mirror(m, n)]);
     const cplx<T> s = y * (num<T>(1.0) - k) + ym * (num<T>(1.0) + k);
     out[m] = mk(half(s.x), half(s.y));
   }
@@ -213,14 +217,14 @@ struct CoefDf {
     const df e2 = e * e;
     c1 = e + e * g * g;
     c2 = half(e2 * g);
-    c3 = e2 * e * df(1.0 / 3.0);
+    c3 = e2 * e * df(0.3333333432674408f, -9.934107758624577e-09f);   // 1/3
   }
 };
-struct Coef32 {
-  const double* eta;
-  const double* hx;
+struct Coef32 {            // from float32 copies of eta and h_x
+  const float2* eh;
   __device__ void operator()(int j, float& c1, float& c2, float& c3) const {
-    const float e = (float)eta[j], g = (float)hx[j];
+    const float2 v = eh[j];
+    const float e = v.x, g = v.y;
     c1 = e * (1.0f + g * g);
     c2 = 0.5f * e * e * g;
     c3 = e * e * e * (1.0f / 3.0f);
@@ -242,9 +246,53 @@ __device__ __forceinline__ void mr_full(cplx<T>* V, const cplx<T>* H, int n) {
   __syncthreads();
 }
 
+// A sum kept in double-float (48 bits; its terms are float32 or double-float): no float64 in
+// the loops of the mixed path.
+struct DfSum {
+  df s{0.0f, 0.0f};
+  __device__ __forceinline__ void add(float v) {
+    const float h = __fadd_rn(s.hi, v), bb = __fsub_rn(h, s.hi);
+    const float e = __fadd_rn(__fsub_rn(s.hi, __fsub_rn(h, bb)), __fsub_rn(v, bb));
+    s = df(h, __fadd_rn(s.lo, e));
+  }
+};
+// over the CTA (fixed tree), in float64 at the end; red as block_sum's
+__device__ __forceinline__ double mr_sum(df v, df* slot, double* out) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+    v = v + df(__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o));
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+  __syncthreads();                                 // slot and out may still be read
+  if (l == 0) slot[w] = v;
+  __syncthreads();
+  if (w == 0) {
+    df r = l < kMrNT / 32 ? slot[l] : df(0.0f, 0.0f);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+      r = r + df(__shfl_xor_sync(0xffffffffu, r.hi, o), __shfl_xor_sync(0xffffffffu, r.lo, o));
+    if (l == 0) *out = (double)r.hi + (double)r.lo;
+  }
+  __syncthreads();
+  return *out;
+}
+// 1/a in double-float: a float32 reciprocal and one residual
+__device__ __forceinline__ df mr_recip(df a) {
+  const float r = __frcp_rn(a.hi);
+  const float e = fmaf(-a.lo, r, fmaf(-a.hi, r, 1.0f));
+  const float c = __fmul_rn(r, e), h = __fadd_rn(r, c);
+  return df(h, __fsub_rn(c, __fsub_rn(h, r)));
+}
+
+// One CTA per instance.  Bound by its SM: transforms through shared memory (n = 6144: 192 KB,
+// one CTA per SM) with a barrier per stage.  The mixed form had wavenumbers, 1/(sigma + alpha
+// k^2), Parseval weights, dot products and the float32 coefficients in float64 inside the
+// float32 loop; they are float32 and double-float now (the two norms of a refinement pass stay
+// float64).
 template <bool MIXED>
 __global__ void __launch_bounds__(kMrNT) k_mr_pcg(const MrArgs A, const MrPcgArgs a) {
   __shared__ double red[kMrNT / 32 + 1];
+  __shared__ df slot[kMrNT / 32];
+  __shared__ double dsum;
   const int id = A.ids[blockIdx.x];
   const Inst1d I = A.insts[id];
   MrPlan P;
@@ -271,42 +319,53 @@ __global__ void __launch_bounds__(kMrNT) k_mr_pcg(const MrArgs A, const MrPcgArg
     return;
   }
   const double sigma = R.sigma, alpha = R.alpha;
-  auto dinv = [&](int m) {
-    const double k = kunit * wave_index(m, n);
-    return 1.0 / (sigma + alpha * k * k);
-  };
-  auto wgt = [&](int m) { return (m == 0 || m == h) ? 1.0 : 2.0; };
+  using TH = typename std::conditional<MIXED, df, double>::type;
+  const TH kuh = num<TH>(kunit);
   cplx<double>* ws = a.ws + I.ws;
-  // ---- b^ and x0^ from one transform of b + i x0 (float64)
-  cplx<double>* d0 = tbuf<double>(A, I, 0);
-  cplx<double>* d1 = tbuf<double>(A, I, 1);
-  for (int j = threadIdx.x; j < n; j += kMrNT) d0[j] = mk(a.b[I.off + j], a.x[I.off + j]);
+  // ---- b^ and x0^ (slots 0 and 1) from one transform of b + i x0, and b.A^{-1}b
+  cplx<TH>* d0 = tbuf<TH>(A, I, 0);
+  cplx<TH>* d1 = tbuf<TH>(A, I, 1);
+  for (int j = threadIdx.x; j < n; j += kMrNT)
+    d0[j] = mk(num<TH>(a.b[I.off + j]), num<TH>(a.x[I.off + j]));
   __syncthreads();
-  cplx<double>* Y = mr::mr_fft<double, kMrNT>(d0, d1, P, false, tws.d);
-  cplx<double>* Bh = ws;            // float64 path: b^, x^, r^, p^, (G p)^ in slots 0..4
-  cplx<double>* Xh = ws + S;
-  double bb = 0.0;
-  for (int m = threadIdx.x; m <= h; m += kMrNT) {
-    const cplx<double> y = Y[m], ym = conj(Y[(n - m) % n]);
-    const cplx<double> sb = y + ym, sx = mul_mi(y - ym);
-    const cplx<double> bh = mk(0.5 * sb.x, 0.5 * sb.y), xh = mk(0.5 * sx.x, 0.5 * sx.y);
-    Bh[m] = bh;
-    Xh[m] = xh;
-    bb += wgt(m) * (bh.x * bh.x + bh.y * bh.y) * dinv(m);
-  }
-  bb = block_sum<kMrNT>(bb, red);
-  const double bnorm = sqrt(bb);
-  if (!(bnorm > 0.0)) {
+  cplx<TH>* Y = mr::mr_fft<TH, kMrNT>(d0, d1, P, false, tw_of<TH>(tws));
+  cplx<TH>* Bh = reinterpret_cast<cplx<TH>*>(ws);
+  cplx<TH>* Xh = reinterpret_cast<cplx<TH>*>(ws + S);
+  auto half_of = [&](int m, cplx<TH>& bh, cplx<TH>& xh) {
+    const cplx<TH> y = Y[m], ym = conj(Y[mr_mirror(m, n)]);
+    const cplx<TH> sb = y + ym, sx = mul_mi(y - ym);
+    bh = mk(half(sb.x), half(sb.y));
+    xh = mk(half(sx.x), half(sx.y));
+  };
+  int iters = 0, status = SGN_OK;
+  auto no_rhs = [&](double bb) {                   // b = 0 solves exactly, else a breakdown
     for (int j = threadIdx.x; j < n; j += kMrNT) a.x[I.off + j] = 0.0;
     R.status = (bb == 0.0) ? SGN_OK : SGN_ERR_BREAKDOWN;
     if (threadIdx.x == 0) a.rec[id] = R;
-    return;
-  }
-  int iters = 0, status = SGN_OK;
+  };
   if constexpr (!MIXED) {
+    // float64: b^, x^, r^, p^, (G p)^ in slots 0..4, 1/(sigma + alpha k^2) in slot 5
     cplx<double>* Rh = ws + 2 * S;
     cplx<double>* Ph = ws + 3 * S;
     cplx<double>* Gh = ws + 4 * S;
+    double* Dv = reinterpret_cast<double*>(ws + 5 * S);
+    auto wgt = [&](int m) { return (m == 0 || m == h) ? 1.0 : 2.0; };
+    double bb = 0.0;
+    for (int m = threadIdx.x; m <= h; m += kMrNT) {
+      const double k = kunit * wave_index(m, n), di = 1.0 / (sigma + alpha * k * k);
+      Dv[m] = di;
+      cplx<double> bh, xh;
+      half_of(m, bh, xh);
+      Bh[m] = bh;
+      Xh[m] = xh;
+      bb += wgt(m) * (bh.x * bh.x + bh.y * bh.y) * di;
+    }
+    bb = block_sum<kMrNT>(bb, red);
+    const double bnorm = sqrt(bb);
+    if (!(bnorm > 0.0)) {
+      no_rhs(bb);
+      return;
+    }
     const Coef64 coef{eta, hx};
     auto matvec = [&](const cplx<double>* Vh) {     // Gh = (G v)^
       mr_full<double>(d0, Vh, n);
@@ -316,9 +375,10 @@ __global__ void __launch_bounds__(kMrNT) k_mr_pcg(const MrArgs A, const MrPcgArg
     double rz = 0.0;
     for (int m = threadIdx.x; m <= h; m += kMrNT) {
       const cplx<double> r = Bh[m] - Gh[m];
+      const double di = Dv[m];
       Rh[m] = r;
-      Ph[m] = r * dinv(m);
-      rz += wgt(m) * (r.x * r.x + r.y * r.y) * dinv(m);
+      Ph[m] = r * di;
+      rz += wgt(m) * (r.x * r.x + r.y * r.y) * di;
     }
     rz = block_sum<kMrNT>(rz, red);
     const double tol = a.rtol * bnorm;
@@ -343,7 +403,7 @@ __global__ void __launch_bounds__(kMrNT) k_mr_pcg(const MrArgs A, const MrPcgArg
         Xh[m] = Xh[m] + Ph[m] * al;
         const cplx<double> r = Rh[m] - Gh[m] * al;
         Rh[m] = r;
-        rzn += wgt(m) * (r.x * r.x + r.y * r.y) * dinv(m);
+        rzn += wgt(m) * (r.x * r.x + r.y * r.y) * Dv[m];
       }
       rzn = block_sum<kMrNT>(rzn, red);
       ++iters;
@@ -353,57 +413,72 @@ __global__ void __launch_bounds__(kMrNT) k_mr_pcg(const MrArgs A, const MrPcgArg
       }
       const double be = rzn / rz;
       rz = rzn;
-      for (int m = threadIdx.x; m <= h; m += kMrNT) Ph[m] = Rh[m] * dinv(m) + Ph[m] * be;
+      for (int m = threadIdx.x; m <= h; m += kMrNT) Ph[m] = Rh[m] * Dv[m] + Ph[m] * be;
     }
     R.ratio = sqrt(rz) / bnorm;
     __syncthreads();
     mr_full<double>(d0, Xh, n);
     const cplx<double>* x = mr::mr_fft<double, kMrNT>(d0, d1, P, true, tws.d);
-    for (int j = threadIdx.x; j < n; j += kMrNT) a.x[I.off + j] = x[j].x / n;
+    const double inv_n = 1.0 / n;
+    for (int j = threadIdx.x; j < n; j += kMrNT) a.x[I.off + j] = x[j].x * inv_n;
   } else {
     // double-float refinement: b^ and x^ (slots 0, 1) and the residual (slot 4) in
     // double-float; the float32 inner solve's r, p (slot 2) and d, G p (slot 3), two
-    // float32 vectors per slot
-    cplx<df>* Bd = reinterpret_cast<cplx<df>*>(ws);
-    cplx<df>* Xd = reinterpret_cast<cplx<df>*>(ws + S);
+    // float32 vectors per slot; float32 eta, h_x in slot 5
     cplx<df>* Gd = reinterpret_cast<cplx<df>*>(ws + 4 * S);
     cplx<float>* Rf = reinterpret_cast<cplx<float>*>(ws + 2 * S);
     cplx<float>* Pf = Rf + S;
     cplx<float>* Df = reinterpret_cast<cplx<float>*>(ws + 3 * S);
     cplx<float>* Gf = Df + S;
-    // the float64 b^, x^ become double-float (each thread rewrites its own modes in place)
+    float2* eh = reinterpret_cast<float2*>(ws + 5 * S);
+    const float sigf = (float)sigma, alf = (float)alpha, kf = (float)kunit;
+    const df sigh(sigma), alh(alpha);
+    auto dinvf = [&](int m) {
+      const float k = kf * (float)wave_index(m, n);
+      return recip(fmaf(alf * k, k, sigf));
+    };
+    auto wf = [&](int m) { return (m == 0 || m == h) ? 1.0f : 2.0f; };
+    // w_m |v|^2 / (sigma + alpha k^2) in float64 (|v|^2 may leave the float32 range), the
+    // symbol's reciprocal by double-float
+    auto term = [&](int m, cplx<df> v) {
+      const df k = mr_k<df>(m, n, kuh);
+      const double x = to_f64(v.x), y = to_f64(v.y);
+      const double q = (x * x + y * y) * to_f64(mr_recip(sigh + alh * (k * k)));
+      return (m == 0 || m == h) ? q : q + q;
+    };
+    double bb = 0.0;
     for (int m = threadIdx.x; m <= h; m += kMrNT) {
-      const cplx<double> bh = Bh[m], xh = Xh[m];
-      Bd[m] = mk(df(bh.x), df(bh.y));
-      Xd[m] = mk(df(xh.x), df(xh.y));
+      cplx<df> bh, xh;
+      half_of(m, bh, xh);
+      Bh[m] = bh;
+      Xh[m] = xh;
+      bb += term(m, bh);
     }
-    __syncthreads();
-    cplx<df>* h0 = tbuf<df>(A, I, 0);
-    cplx<df>* h1 = tbuf<df>(A, I, 1);
+    for (int j = threadIdx.x; j < n; j += kMrNT)
+      eh[j] = make_float2(df(eta[j]).hi, df(hx[j]).hi);
+    bb = block_sum<kMrNT>(bb, red);
+    const double bnorm = sqrt(bb);
+    if (!(bnorm > 0.0)) {
+      no_rhs(bb);
+      return;
+    }
     cplx<float>* f0 = tbuf<float>(A, I, 0);
     cplx<float>* f1 = tbuf<float>(A, I, 1);
     const CoefDf cdf{eta, hx};
-    const Coef32 c32{eta, hx};
-    const float sigf = (float)sigma, alf = (float)alpha, kf = (float)kunit;
-    auto dinvf = [&](int m) {
-      const float k = kf * (float)wave_index(m, n);
-      return 1.0f / (sigf + alf * k * k);
-    };
+    const Coef32 c32{eh};
     int refinements = 0;
     double ratio = 0.0;
     for (;;) {
       // r^ = b^ - (G x)^ in double-float, and r.A^{-1}r
-      mr_full<df>(h0, Xd, n);
-      mr_matvec<df>(h0, h1, P, kunit, tws.h, cdf, Gd);
-      double rz64 = 0.0;
+      mr_full<df>(d0, Xh, n);
+      mr_matvec<df>(d0, d1, P, kuh, tws.h, cdf, Gd);
+      double rs = 0.0;
       for (int m = threadIdx.x; m <= h; m += kMrNT) {
-        const cplx<df> r = Bd[m] - Gd[m];
+        const cplx<df> r = Bh[m] - Gd[m];
         Gd[m] = r;
-        const double rx = to_f64(r.x), ry = to_f64(r.y);
-        rz64 += wgt(m) * (rx * rx + ry * ry) * dinv(m);
+        rs += term(m, r);
       }
-      rz64 = block_sum<kMrNT>(rz64, red);
-      const double nr = sqrt(rz64);
+      const double nr = sqrt(block_sum<kMrNT>(rs, red));
       ratio = nr / bnorm;
       if (ratio <= a.rtol) {
         status = SGN_OK;
@@ -416,51 +491,52 @@ __global__ void __launch_bounds__(kMrNT) k_mr_pcg(const MrArgs A, const MrPcgArg
       }
       const double tin = a.rtol_inner > 0.0 ? a.rtol_inner
                                             : fmin(0.1, fmax(1e-6, 0.3 * a.rtol / ratio));
-      const float sc = (float)(1.0 / nr);
+      const float sc = (float)(1.0 / nr), tin2 = (float)(tin * tin);
       // float32 PCG for G d = r / ||r||
-      double rz = 0.0;
+      DfSum z0;
       for (int m = threadIdx.x; m <= h; m += kMrNT) {
-        const cplx<float> r = mk((float)to_f64(Gd[m].x) * sc, (float)to_f64(Gd[m].y) * sc);
+        const cplx<df> g = Gd[m];
+        const cplx<float> r = mk((g.x.hi + g.x.lo) * sc, (g.y.hi + g.y.lo) * sc);
         Rf[m] = r;
         Df[m] = mk(0.0f, 0.0f);
         const cplx<float> z = r * dinvf(m);
         Pf[m] = z;
-        rz += wgt(m) * (double)(r.x * z.x + r.y * z.y);
+        z0.add(wf(m) * (r.x * z.x + r.y * z.y));
       }
-      rz = block_sum<kMrNT>(rz, red);
+      float rz = (float)mr_sum(z0.s, slot, &dsum);
       const int it0 = iters;
       int st_in = SGN_OK;
-      while (sqrt(rz) > tin) {
+      while (rz > tin2) {
         if (iters >= a.maxit) {
           st_in = SGN_ERR_NOT_CONVERGED;
           break;
         }
         __syncthreads();
         mr_full<float>(f0, Pf, n);
-        mr_matvec<float>(f0, f1, P, kunit, tws.f, c32, Gf);
-        double pq = 0.0;
+        mr_matvec<float>(f0, f1, P, kf, tws.f, c32, Gf);
+        DfSum ps;
         for (int m = threadIdx.x; m <= h; m += kMrNT)
-          pq += wgt(m) * (double)(Pf[m].x * Gf[m].x + Pf[m].y * Gf[m].y);
-        pq = block_sum<kMrNT>(pq, red);
-        if (!(pq > 0.0) || !isfinite(pq)) {
+          ps.add(wf(m) * (Pf[m].x * Gf[m].x + Pf[m].y * Gf[m].y));
+        const float pq = (float)mr_sum(ps.s, slot, &dsum);
+        if (!(pq > 0.0f) || !isfinite(pq)) {
           st_in = SGN_ERR_BREAKDOWN;
           break;
         }
-        const float al = (float)(rz / pq);
-        double rzn = 0.0;
+        const float al = rz / pq;
+        DfSum zs;
         for (int m = threadIdx.x; m <= h; m += kMrNT) {
           Df[m] = Df[m] + Pf[m] * al;
           const cplx<float> r = Rf[m] - Gf[m] * al;
           Rf[m] = r;
-          rzn += wgt(m) * (double)((r.x * r.x + r.y * r.y) * dinvf(m));
+          zs.add(wf(m) * ((r.x * r.x + r.y * r.y) * dinvf(m)));
         }
-        rzn = block_sum<kMrNT>(rzn, red);
+        const float rzn = (float)mr_sum(zs.s, slot, &dsum);
         ++iters;
         if (!isfinite(rzn)) {
           st_in = SGN_ERR_BREAKDOWN;
           break;
         }
-        const float be = (float)(rzn / rz);
+        const float be = rzn / rz;
         rz = rzn;
         for (int m = threadIdx.x; m <= h; m += kMrNT) Pf[m] = Rf[m] * dinvf(m) + Pf[m] * be;
       }
@@ -470,15 +546,15 @@ __global__ void __launch_bounds__(kMrNT) k_mr_pcg(const MrArgs A, const MrPcgArg
       const df un(nr);
       __syncthreads();
       for (int m = threadIdx.x; m <= h; m += kMrNT)
-        Xd[m] = mk(Xd[m].x + df(Df[m].x, 0.0f) * un, Xd[m].y + df(Df[m].y, 0.0f) * un);
+        Xh[m] = mk(Xh[m].x + df(Df[m].x, 0.0f) * un, Xh[m].y + df(Df[m].y, 0.0f) * un);
       ++refinements;
       __syncthreads();
     }
     R.refinements = refinements;
     R.ratio = ratio;
     __syncthreads();
-    mr_full<df>(h0, Xd, n);
-    const cplx<df>* x = mr::mr_fft<df, kMrNT>(h0, h1, P, true, tws.h);
+    mr_full<df>(d0, Xh, n);
+    const cplx<df>* x = mr::mr_fft<df, kMrNT>(d0, d1, P, true, tws.h);
     const df inv_n(1.0 / n);
     for (int j = threadIdx.x; j < n; j += kMrNT) a.x[I.off + j] = to_f64(x[j].x * inv_n);
   }
