@@ -180,7 +180,7 @@ cudaError_t launch_pcg1d(const Layout1d& lay, const void* tw64, const void* tw32
     return launch_form<decltype(Lc)::value>(lay, a, first, num, cs, PcgKernels{});
   }, [&](int first, int num, cudaStream_t cs) {
     return mr_launch_pcg(lay, first, num, precision, eta, hx, b, x, given, kind, rtol,
-                         rtol_inner, maxit, max_refine, rec, ws, cs);
+                         rtol_inner, maxit, max_refine, rec, ws, nullptr, cs);
   });
 }
 
@@ -192,12 +192,11 @@ cudaError_t launch_pcg1d_ux(const Layout1d& lay, const void* tw64, const void* t
   PcgArgs a = pcg_args(lay, tw64, tw32, precision, eta, hx, b, x, nullptr, kind, rtol,
                        rtol_inner, maxit, max_refine, rec, ws, coef_df);
   a.ux = scratch;
-  // the generic kernels take no u_x hand-off: their right-hand side derives u itself
   return d1::for_each_size(lay, s, [&](auto Lc, int first, int num, cudaStream_t cs) {
     return launch_form<decltype(Lc)::value>(lay, a, first, num, cs, PcgKernels{});
   }, [&](int first, int num, cudaStream_t cs) {
     return mr_launch_pcg(lay, first, num, precision, eta, hx, b, x, nullptr, kind, rtol,
-                         rtol_inner, maxit, max_refine, rec, ws, cs);
+                         rtol_inner, maxit, max_refine, rec, ws, scratch, cs);
   });
 }
 
@@ -209,7 +208,7 @@ cudaError_t launch_rhs1d(const Layout1d& lay, const void* tw64, const void* tw32
   return d1::for_each_size(lay, s, [&](auto Lc, int first, int num, cudaStream_t cs) {
     return launch_form<decltype(Lc)::value>(lay, a, first, num, cs, RhsKernels{});
   }, [&](int first, int num, cudaStream_t cs) {
-    return mr_launch_rhs(lay, first, num, precision, g, eta, u, h, hx, f_eta, f_U, scratch, cs);
+    return mr_launch_rhs(lay, first, num, precision, g, eta, u, h, hx, f_eta, f_U, scratch, false, cs);
   });
 }
 
@@ -222,7 +221,7 @@ cudaError_t launch_rhs1d_ux(const Layout1d& lay, const void* tw64, const void* t
   return d1::for_each_size(lay, s, [&](auto Lc, int first, int num, cudaStream_t cs) {
     return launch_form<decltype(Lc)::value>(lay, a, first, num, cs, RhsKernels{});
   }, [&](int first, int num, cudaStream_t cs) {
-    return mr_launch_rhs(lay, first, num, precision, g, eta, u, h, hx, f_eta, f_U, scratch, cs);
+    return mr_launch_rhs(lay, first, num, precision, g, eta, u, h, hx, f_eta, f_U, scratch, true, cs);
   });
 }
 

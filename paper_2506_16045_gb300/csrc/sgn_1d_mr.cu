@@ -101,35 +101,56 @@ __global__ void __launch_bounds__(kMrNT) k_mr_deriv(const MrArgs A, const double
   for (int j = threadIdx.x; j < I.n; j += kMrNT) fx[I.off + j] = o[j].x;
 }
 
-// (G v)^ of a real field held as its full spectrum V (modes 0..n-1): the transform of
-// v + i v_x is (1 - k) V; pointwise w = c1 v + c2 v_x, q = c2 v + c3 v_x; (G v)^_m =
-// ((1 - k_m) Y_m + (1 + k_m) conj Y_{n-m}) / 2 with Y the transform of w + i q (Def:G as
-// w - q_x).  Writes the half spectrum m = 0..n/2 of G v into out (T arithmetic).  c: the
-// coefficients c1, c2, c3 at point j.
-template <typename T, typename Coef>
-__device__ void mr_matvec(cplx<T>* a, cplx<T>* b, const MrPlan& P, T ku,
-                          const cplx<T>* tw, Coef coef, cplx<T>* out) {
-  const int n = P.n, h = n / 2;
-  // a holds V (full spectrum); form (1 - k) V in place
-  for (int m = threadIdx.x; m < n; m += kMrNT) a[m] = a[m] * (num<T>(1.0) - mr_k<T>(m, n, ku));
+// The transform of v + i v_x from the half spectrum of the real field v: a_m = (1 - k) v_m and
+// a_{n-m} = (1 + k) conj v_m, the DC and Nyquist coefficients taken real (their imaginary
+// parts are rounding residue).  get(m): v_m, m = 0..n/2.  Ends with a barrier.
+template <typename T, typename Get>
+__device__ __forceinline__ void mr_fill(cplx<T>* a, int n, T ku, Get get) {
+  const int h = n / 2;
+  const T one = from_int<T>(1);
+  for (int m = threadIdx.x; m <= h; m += kMrNT) {
+    const cplx<T> v = get(m);
+    if (m == 0 || m == h) {
+      a[m] = mk(v.x, from_int<T>(0));
+    } else {
+      const T k = mr_k<T>(m, n, ku);
+      a[m] = v * (one - k);
+      a[n - m] = conj(v) * (one + k);
+    }
+  }
   __syncthreads();
+}
+
+// With Z = F(v + i v_x) in a (mr_fill): back to real space, pointwise w = c1 v + c2 v_x,
+// q = c2 v + c3 v_x, and the transform Y of w + i q, from which mr_gv takes (G v)^ (Def:G as
+// w - q_x).  point(j, v, v_x) may keep the field.  Returns Y, after a barrier.
+template <typename T, typename Coef, typename Point>
+__device__ __forceinline__ cplx<T>* mr_wq(cplx<T>* a, cplx<T>* b, const MrPlan& P, T inv_n,
+                                          const cplx<T>* tw, const Coef& coef, Point point) {
+  const int n = P.n;
   cplx<T>* z = mr::mr_fft<T, kMrNT>(a, b, P, true, tw);
-  const T inv_n = num<T>(1.0 / n);
   for (int j = threadIdx.x; j < n; j += kMrNT) {
     const T v = z[j].x * inv_n, vx = z[j].y * inv_n;
     T c1, c2, c3;
     coef(j, c1, c2, c3);
+    point(j, v, vx);
     z[j] = mk(c1 * v + c2 * vx, c2 * v + c3 * vx);
   }
   __syncthreads();
-  cplx<T>* Y = mr::mr_fft<T, kMrNT>(z, z == a ? b : a, P, false, tw);
-  for (int m = threadIdx.x; m <= h; m += kMrNT) {
-    const T k = mr_k<T>(m, n, ku);
-    const cplx<T> y = Y[m], ym = conj(Y[mr_mirror(m, n)]);
-    const cplx<T> s = y * (num<T>(1.0) - k) + ym * (num<T>(1.0) + k);
-    out[m] = mk(half(s.x), half(s.y));
-  }
-  __syncthreads();
+  return mr::mr_fft<T, kMrNT>(z, z == a ? b : a, P, false, tw);
+}
+struct NoPoint {
+  template <typename T>
+  __device__ __forceinline__ void operator()(int, T, T) const {}
+};
+
+// (G v)^_m = ((1 - k_m) Y_m + (1 + k_m) conj Y_{n-m}) / 2, m = 0..n/2
+template <typename T>
+__device__ __forceinline__ cplx<T> mr_gv(const cplx<T>* Y, int m, int n, T ku) {
+  const T one = from_int<T>(1), k = mr_k<T>(m, n, ku);
+  const cplx<T> y = Y[m], ym = conj(Y[mr_mirror(m, n)]);
+  const cplx<T> s = y * (one - k) + ym * (one + k);
+  return mk(half(s.x), half(s.y));
 }
 
 struct Coef64 {
@@ -157,16 +178,21 @@ __global__ void __launch_bounds__(kMrNT) k_mr_apply_G(const MrArgs A, const doub
   const double kunit = 2.0 * kPi / I.L;
   for (int j = threadIdx.x; j < n; j += kMrNT) a[j] = mk(u[I.off + j], 0.0);
   __syncthreads();
+  // (1 - k) times the spectrum of a real field is that of v + i v_x
   cplx<double>* V = mr::mr_fft<double, kMrNT>(a, b, P, false, tw);
   cplx<double>* o = V == a ? b : a;
-  // (G u)^ of modes 0..n/2 into V itself: mode m is read and written only by the thread
-  // that computes it (its mirror n - m is above n/2 and never written)
-  mr_matvec<double>(V, o, P, kunit, tw, Coef64{eta + I.off, hx + I.off}, V);
-  // V[0..h] = (G u)^; build the Hermitian full spectrum and invert
-  for (int m = threadIdx.x; m < h; m += kMrNT)
-    if (m > 0) V[n - m] = conj(V[m]);
+  for (int m = threadIdx.x; m < n; m += kMrNT) V[m] = V[m] * (1.0 - mr_k<double>(m, n, kunit));
   __syncthreads();
-  const cplx<double>* x = mr::mr_fft<double, kMrNT>(V, o, P, true, tw);
+  cplx<double>* Y = mr_wq<double>(V, o, P, 1.0 / n, tw, Coef64{eta + I.off, hx + I.off}, NoPoint());
+  o = Y == a ? b : a;
+  // the Hermitian full spectrum of G u into the other buffer, and back
+  for (int m = threadIdx.x; m <= h; m += kMrNT) {
+    const cplx<double> g = mr_gv<double>(Y, m, n, kunit);
+    o[m] = g;
+    if (m > 0 && m < h) o[n - m] = conj(g);
+  }
+  __syncthreads();
+  const cplx<double>* x = mr::mr_fft<double, kMrNT>(o, Y, P, true, tw);
   for (int j = threadIdx.x; j < n; j += kMrNT) Gu[I.off + j] = x[j].x / n;
 }
 
@@ -206,6 +232,7 @@ struct MrPcgArgs {
   int maxit, max_refine;
   SolveRec* rec;
   cplx<double>* ws;
+  void* ux;              // nullable: also store x_x here (double-float or float64)
 };
 
 // coefficients of Def:MatrixM in double-float and float32
@@ -231,21 +258,6 @@ struct Coef32 {            // from float32 copies of eta and h_x
   }
 };
 
-// the full spectrum V_m (m = 0..n-1) of a real field from its half spectrum H (m = 0..n/2),
-// the DC and Nyquist coefficients taken real (their imaginary parts are rounding residue)
-template <typename T>
-__device__ __forceinline__ void mr_full(cplx<T>* V, const cplx<T>* H, int n) {
-  const int h = n / 2;
-  for (int m = threadIdx.x; m < n; m += kMrNT) {
-    cplx<T> v;
-    if (m == 0 || m == h) v = mk(H[m].x, from_int<T>(0));
-    else if (m < h) v = H[m];
-    else v = conj(H[n - m]);
-    V[m] = v;
-  }
-  __syncthreads();
-}
-
 // A sum kept in double-float (48 bits; its terms are float32 or double-float): no float64 in
 // the loops of the mixed path.
 struct DfSum {
@@ -256,13 +268,16 @@ struct DfSum {
     s = df(h, __fadd_rn(s.lo, e));
   }
 };
-// over the CTA (fixed tree), in float64 at the end; red as block_sum's
-__device__ __forceinline__ double mr_sum(df v, df* slot, double* out) {
+// over the CTA (fixed tree); slot[2][warps] and out[2] are used in turn, so a half is written
+// again only after the barriers of the sum between
+__device__ __forceinline__ float mr_sum(df v, df* slots, float* outs, int& turn) {
+  df* slot = slots + turn * (kMrNT / 32);
+  float* out = outs + turn;
+  turn ^= 1;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1)
     v = v + df(__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o));
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  __syncthreads();                                 // slot and out may still be read
   if (l == 0) slot[w] = v;
   __syncthreads();
   if (w == 0) {
@@ -270,7 +285,7 @@ __device__ __forceinline__ double mr_sum(df v, df* slot, double* out) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1)
       r = r + df(__shfl_xor_sync(0xffffffffu, r.hi, o), __shfl_xor_sync(0xffffffffu, r.lo, o));
-    if (l == 0) *out = (double)r.hi + (double)r.lo;
+    if (l == 0) *out = r.hi + r.lo;
   }
   __syncthreads();
   return *out;
@@ -291,8 +306,9 @@ __device__ __forceinline__ df mr_recip(df a) {
 template <bool MIXED>
 __global__ void __launch_bounds__(kMrNT) k_mr_pcg(const MrArgs A, const MrPcgArgs a) {
   __shared__ double red[kMrNT / 32 + 1];
-  __shared__ df slot[kMrNT / 32];
-  __shared__ double dsum;
+  __shared__ df slot[2 * (kMrNT / 32)];
+  __shared__ float sums[2];
+  int turn = 0;
   const int id = A.ids[blockIdx.x];
   const Inst1d I = A.insts[id];
   MrPlan P;
@@ -367,9 +383,12 @@ __global__ void __launch_bounds__(kMrNT) k_mr_pcg(const MrArgs A, const MrPcgArg
       return;
     }
     const Coef64 coef{eta, hx};
+    const double inv_n = 1.0 / n;
     auto matvec = [&](const cplx<double>* Vh) {     // Gh = (G v)^
-      mr_full<double>(d0, Vh, n);
-      mr_matvec<double>(d0, d1, P, kunit, tws.d, coef, Gh);
+      mr_fill<double>(d0, n, kunit, [&](int m) { return Vh[m]; });
+      const cplx<double>* W = mr_wq<double>(d0, d1, P, inv_n, tws.d, coef, NoPoint());
+      for (int m = threadIdx.x; m <= h; m += kMrNT) Gh[m] = mr_gv<double>(W, m, n, kunit);
+      __syncthreads();
     };
     matvec(Xh);
     double rz = 0.0;
@@ -417,22 +436,32 @@ __global__ void __launch_bounds__(kMrNT) k_mr_pcg(const MrArgs A, const MrPcgArg
     }
     R.ratio = sqrt(rz) / bnorm;
     __syncthreads();
-    mr_full<double>(d0, Xh, n);
+    // x + i x_x from one transform
+    mr_fill<double>(d0, n, kunit, [&](int m) { return Xh[m]; });
     const cplx<double>* x = mr::mr_fft<double, kMrNT>(d0, d1, P, true, tws.d);
-    const double inv_n = 1.0 / n;
-    for (int j = threadIdx.x; j < n; j += kMrNT) a.x[I.off + j] = x[j].x * inv_n;
+    double* ux = a.ux ? static_cast<double*>(a.ux) + I.off : nullptr;
+    for (int j = threadIdx.x; j < n; j += kMrNT) {
+      a.x[I.off + j] = x[j].x * inv_n;
+      if (ux) ux[j] = x[j].y * inv_n;
+    }
   } else {
     // double-float refinement: b^ and x^ (slots 0, 1) and the residual (slot 4) in
-    // double-float; the float32 inner solve's r, p (slot 2) and d, G p (slot 3), two
-    // float32 vectors per slot; float32 eta, h_x in slot 5
+    // double-float, float32 eta, h_x in slot 5.  The float32 inner solve lives in the two
+    // transform buffers' 32 n bytes: its two transform buffers (16 n), then p, r and the
+    // correction d (half spectra, 12 n + 24).  x and x_x come from the residual's own
+    // transform; until the solve ends x holds double-float bits.
     cplx<df>* Gd = reinterpret_cast<cplx<df>*>(ws + 4 * S);
-    cplx<float>* Rf = reinterpret_cast<cplx<float>*>(ws + 2 * S);
-    cplx<float>* Pf = Rf + S;
-    cplx<float>* Df = reinterpret_cast<cplx<float>*>(ws + 3 * S);
-    cplx<float>* Gf = Df + S;
     float2* eh = reinterpret_cast<float2*>(ws + 5 * S);
+    cplx<float>* f0 = tbuf<float>(A, I, 0);
+    cplx<float>* f1 = f0 + n;
+    cplx<float>* Pf = f1 + n;
+    cplx<float>* Rf = Pf + S;
+    cplx<float>* Df = Rf + S;
+    double* xo = a.x + I.off;
+    df* ux = a.ux ? static_cast<df*>(a.ux) + I.off : nullptr;
     const float sigf = (float)sigma, alf = (float)alpha, kf = (float)kunit;
-    const df sigh(sigma), alh(alpha);
+    const float inv_nf = recip((float)n);
+    const df sigh(sigma), alh(alpha), inv_n = mr_recip(df(n));
     auto dinvf = [&](int m) {
       const float k = kf * (float)wave_index(m, n);
       return recip(fmaf(alf * k, k, sigf));
@@ -462,19 +491,20 @@ __global__ void __launch_bounds__(kMrNT) k_mr_pcg(const MrArgs A, const MrPcgArg
       no_rhs(bb);
       return;
     }
-    cplx<float>* f0 = tbuf<float>(A, I, 0);
-    cplx<float>* f1 = tbuf<float>(A, I, 1);
     const CoefDf cdf{eta, hx};
     const Coef32 c32{eh};
     int refinements = 0;
     double ratio = 0.0;
     for (;;) {
-      // r^ = b^ - (G x)^ in double-float, and r.A^{-1}r
-      mr_full<df>(d0, Xh, n);
-      mr_matvec<df>(d0, d1, P, kuh, tws.h, cdf, Gd);
+      // r^ = b^ - (G x)^ in double-float, and r.A^{-1}r; the real-space x on the way
+      mr_fill<df>(d0, n, kuh, [&](int m) { return Xh[m]; });
+      const cplx<df>* W = mr_wq<df>(d0, d1, P, inv_n, tws.h, cdf, [&](int j, df v, df vx) {
+        xo[j] = __hiloint2double(__float_as_int(v.lo), __float_as_int(v.hi));
+        if (ux) ux[j] = vx;
+      });
       double rs = 0.0;
       for (int m = threadIdx.x; m <= h; m += kMrNT) {
-        const cplx<df> r = Bh[m] - Gd[m];
+        const cplx<df> r = Bh[m] - mr_gv<df>(W, m, n, kuh);
         Gd[m] = r;
         rs += term(m, r);
       }
@@ -492,18 +522,17 @@ __global__ void __launch_bounds__(kMrNT) k_mr_pcg(const MrArgs A, const MrPcgArg
       const double tin = a.rtol_inner > 0.0 ? a.rtol_inner
                                             : fmin(0.1, fmax(1e-6, 0.3 * a.rtol / ratio));
       const float sc = (float)(1.0 / nr), tin2 = (float)(tin * tin);
-      // float32 PCG for G d = r / ||r||
+      // float32 PCG for G d = r / ||r||; p = A^{-1} r + beta p is formed with its transform's
+      // input (beta = 0 first), and (G p)^ is taken from Y twice instead of being kept
       DfSum z0;
       for (int m = threadIdx.x; m <= h; m += kMrNT) {
         const cplx<df> g = Gd[m];
         const cplx<float> r = mk((g.x.hi + g.x.lo) * sc, (g.y.hi + g.y.lo) * sc);
         Rf[m] = r;
-        Df[m] = mk(0.0f, 0.0f);
-        const cplx<float> z = r * dinvf(m);
-        Pf[m] = z;
-        z0.add(wf(m) * (r.x * z.x + r.y * z.y));
+        Df[m] = Pf[m] = mk(0.0f, 0.0f);
+        z0.add(wf(m) * ((r.x * r.x + r.y * r.y) * dinvf(m)));
       }
-      float rz = (float)mr_sum(z0.s, slot, &dsum);
+      float rz = mr_sum(z0.s, slot, sums, turn), beta = 0.0f;
       const int it0 = iters;
       int st_in = SGN_OK;
       while (rz > tin2) {
@@ -511,13 +540,18 @@ __global__ void __launch_bounds__(kMrNT) k_mr_pcg(const MrArgs A, const MrPcgArg
           st_in = SGN_ERR_NOT_CONVERGED;
           break;
         }
-        __syncthreads();
-        mr_full<float>(f0, Pf, n);
-        mr_matvec<float>(f0, f1, P, kf, tws.f, c32, Gf);
+        mr_fill<float>(f0, n, kf, [&](int m) {
+          const cplx<float> p = Rf[m] * dinvf(m) + Pf[m] * beta;
+          Pf[m] = p;
+          return p;
+        });
+        const cplx<float>* Yf = mr_wq<float>(f0, f1, P, inv_nf, tws.f, c32, NoPoint());
         DfSum ps;
-        for (int m = threadIdx.x; m <= h; m += kMrNT)
-          ps.add(wf(m) * (Pf[m].x * Gf[m].x + Pf[m].y * Gf[m].y));
-        const float pq = (float)mr_sum(ps.s, slot, &dsum);
+        for (int m = threadIdx.x; m <= h; m += kMrNT) {
+          const cplx<float> p = Pf[m], g = mr_gv<float>(Yf, m, n, kf);
+          ps.add(wf(m) * (p.x * g.x + p.y * g.y));
+        }
+        const float pq = mr_sum(ps.s, slot, sums, turn);
         if (!(pq > 0.0f) || !isfinite(pq)) {
           st_in = SGN_ERR_BREAKDOWN;
           break;
@@ -526,37 +560,34 @@ __global__ void __launch_bounds__(kMrNT) k_mr_pcg(const MrArgs A, const MrPcgArg
         DfSum zs;
         for (int m = threadIdx.x; m <= h; m += kMrNT) {
           Df[m] = Df[m] + Pf[m] * al;
-          const cplx<float> r = Rf[m] - Gf[m] * al;
+          const cplx<float> r = Rf[m] - mr_gv<float>(Yf, m, n, kf) * al;
           Rf[m] = r;
           zs.add(wf(m) * ((r.x * r.x + r.y * r.y) * dinvf(m)));
         }
-        const float rzn = (float)mr_sum(zs.s, slot, &dsum);
+        const float rzn = mr_sum(zs.s, slot, sums, turn);
         ++iters;
         if (!isfinite(rzn)) {
           st_in = SGN_ERR_BREAKDOWN;
           break;
         }
-        const float be = rzn / rz;
+        beta = rzn / rz;
         rz = rzn;
-        for (int m = threadIdx.x; m <= h; m += kMrNT) Pf[m] = Rf[m] * dinvf(m) + Pf[m] * be;
       }
       // a float32 breakdown after some progress keeps the correction (the next residual
       // decides); the iteration cap is reported by the refinement loop
       if (st_in == SGN_ERR_BREAKDOWN && iters == it0) status = SGN_ERR_BREAKDOWN;
       const df un(nr);
-      __syncthreads();
       for (int m = threadIdx.x; m <= h; m += kMrNT)
         Xh[m] = mk(Xh[m].x + df(Df[m].x, 0.0f) * un, Xh[m].y + df(Df[m].y, 0.0f) * un);
       ++refinements;
-      __syncthreads();
+      __syncthreads();                             // d has been read; d0 is filled next
     }
     R.refinements = refinements;
     R.ratio = ratio;
-    __syncthreads();
-    mr_full<df>(d0, Xh, n);
-    const cplx<df>* x = mr::mr_fft<df, kMrNT>(d0, d1, P, true, tws.h);
-    const df inv_n(1.0 / n);
-    for (int j = threadIdx.x; j < n; j += kMrNT) a.x[I.off + j] = to_f64(x[j].x * inv_n);
+    for (int j = threadIdx.x; j < n; j += kMrNT) {
+      const double v = xo[j];
+      xo[j] = to_f64(df(__int_as_float(__double2loint(v)), __int_as_float(__double2hiint(v))));
+    }
   }
   R.iters = iters;
   R.status = status;
@@ -568,7 +599,10 @@ __global__ void __launch_bounds__(kMrNT) k_mr_pcg(const MrArgs A, const MrPcgArg
 // with Phi' = eta^3 Q/3 + eta^2 m d + eta^2 S/2 + eta m s - eta u^2 (the flux folded in),
 // Q = u d_x - d^2, S = u s_x; f_eta = -m, f_U = -g eta zeta_x + Phi'_x - h_x Psi,
 // Psi = eta^2 Q/2 + eta m d + eta S + m s.  Intermediates in scratch planes (T per point).
-template <typename T>
+// UXG: d = u_x is already in the first scratch plane (from the solve that produced u), so the
+// pairs are (eta u, zeta) -> (m, zeta_x), (s, d) -> (s_x, d_x) and Phi': six transforms
+// instead of eight.
+template <typename T, bool UXG>
 __global__ void __launch_bounds__(kMrNT) k_mr_rhs(const MrArgs A, double g, const double* __restrict__ eta,
                                                  const double* __restrict__ u,
                                                  const double* __restrict__ hgt,
@@ -585,61 +619,67 @@ __global__ void __launch_bounds__(kMrNT) k_mr_rhs(const MrArgs A, double g, cons
   cplx<T>* b0 = tbuf<T>(A, I, 0);
   cplx<T>* b1 = tbuf<T>(A, I, 1);
   // planes of Ptot 8-byte values (float64 or double-float), indexed by point
-  T* D = reinterpret_cast<T*>(scr);                 // d, then Psi
-  T* M = reinterpret_cast<T*>(scr + Ptot);          // m
-  T* ZX = reinterpret_cast<T*>(scr + 2 * Ptot);     // zeta_x
-  T* SX = reinterpret_cast<T*>(scr + 3 * Ptot);     // s_x
-  T* DX = reinterpret_cast<T*>(scr + 4 * Ptot);     // d_x
+  T* D = reinterpret_cast<T*>(scr) + o;                 // d, then Psi
+  T* M = reinterpret_cast<T*>(scr + Ptot) + o;          // m
+  T* ZX = reinterpret_cast<T*>(scr + 2 * Ptot) + o;     // zeta_x
+  T* SX = reinterpret_cast<T*>(scr + 3 * Ptot) + o;     // s_x
   static_assert(sizeof(T) == sizeof(double), "8-byte plane elements");
-  // (u, eta u)
-  for (int j = threadIdx.x; j < n; j += kMrNT) {
-    const T uu = num<T>(u[o + j]), e = num<T>(eta[o + j]);
-    b0[j] = mk(uu, e * uu);
-  }
-  __syncthreads();
-  const cplx<T>* r = mr_deriv_pair<T>(b0, b1, P, kunit, tw);
-  for (int j = threadIdx.x; j < n; j += kMrNT) {
-    D[o + j] = r[j].x;
-    M[o + j] = r[j].y;
-  }
-  __syncthreads();
-  // (zeta, s)
-  for (int j = threadIdx.x; j < n; j += kMrNT) {
-    const T e = num<T>(eta[o + j]), hh = num<T>(hgt[o + j]), g1 = num<T>(hx[o + j]);
-    b0[j] = mk(e - hh, g1 * num<T>(u[o + j]));
-  }
-  __syncthreads();
-  r = mr_deriv_pair<T>(b0, b1, P, kunit, tw);
-  for (int j = threadIdx.x; j < n; j += kMrNT) {
-    ZX[o + j] = r[j].x;
-    SX[o + j] = r[j].y;
-  }
-  __syncthreads();
-  // d -> d_x
-  for (int j = threadIdx.x; j < n; j += kMrNT) b0[j] = mk(D[o + j], from_int<T>(0));
-  __syncthreads();
-  r = mr_deriv_pair<T>(b0, b1, P, kunit, tw);
-  for (int j = threadIdx.x; j < n; j += kMrNT) DX[o + j] = r[j].x;
-  __syncthreads();
-  // Phi' -> Phi'_x; f_eta, and Psi kept for f_U
-  const T third = num<T>(1.0 / 3.0);
-  for (int j = threadIdx.x; j < n; j += kMrNT) {
-    const T uu = num<T>(u[o + j]), e = num<T>(eta[o + j]), g1 = num<T>(hx[o + j]);
-    const T d = D[o + j], m = M[o + j], s = g1 * uu;
-    const T Q = uu * DX[o + j] - d * d, Sv = uu * SX[o + j];
-    const T e2 = e * e;
-    const T phi = e2 * e * Q * third + e2 * m * d + half(e2 * Sv) + e * m * s - e * uu * uu;
-    const T psi = half(e2 * Q) + e * m * d + e * Sv + m * s;
-    b0[j] = mk(phi, from_int<T>(0));
-    D[o + j] = psi;                       // d is no longer needed
-    f_eta[o + j] = -to_f64(m);
-  }
-  __syncthreads();
-  r = mr_deriv_pair<T>(b0, b1, P, kunit, tw);
-  const T gT = num<T>(g);
-  for (int j = threadIdx.x; j < n; j += kMrNT) {
-    const T e = num<T>(eta[o + j]), g1 = num<T>(hx[o + j]);
-    f_U[o + j] = to_f64(r[j].x - gT * e * ZX[o + j] - g1 * D[o + j]);
+  const T third = num<T>(1.0 / 3.0), gT = num<T>(g);
+  constexpr int passes = UXG ? 3 : 4;
+#pragma unroll 1
+  for (int pass = 0; pass < passes; ++pass) {
+    // 0: (eta u, zeta), 1: (s, d); or 2: (u, eta u), 3: (zeta, s), 4: d; then 5: Phi'
+    const int what = UXG ? (pass == 0 ? 0 : pass == 1 ? 1 : 5) : (pass < 3 ? 2 + pass : 5);
+    if (what != 5) {
+      for (int j = threadIdx.x; j < n; j += kMrNT) {
+        if (what == 4) {
+          b0[j] = mk(D[j], from_int<T>(0));
+          continue;
+        }
+        const T uu = num<T>(u[o + j]), e = num<T>(eta[o + j]);
+        if (what == 0) b0[j] = mk(e * uu, e - num<T>(hgt[o + j]));
+        else if (what == 1) b0[j] = mk(num<T>(hx[o + j]) * uu, D[j]);
+        else if (what == 2) b0[j] = mk(uu, e * uu);
+        else b0[j] = mk(e - num<T>(hgt[o + j]), num<T>(hx[o + j]) * uu);
+      }
+      __syncthreads();
+    }
+    const cplx<T>* r = mr_deriv_pair<T>(b0, b1, P, kunit, tw);
+    if (what == 5) {
+      for (int j = threadIdx.x; j < n; j += kMrNT) {
+        const T e = num<T>(eta[o + j]), g1 = num<T>(hx[o + j]);
+        f_U[o + j] = to_f64(r[j].x - gT * e * ZX[j] - g1 * D[j]);
+      }
+    } else if (pass == passes - 2) {
+      // all derivatives are there: Phi' (the next input), Psi (kept for f_U) and f_eta; the
+      // result r may be b0 itself, each point read before it is written
+      for (int j = threadIdx.x; j < n; j += kMrNT) {
+        const T uu = num<T>(u[o + j]), e = num<T>(eta[o + j]), g1 = num<T>(hx[o + j]);
+        const T d = D[j], m = M[j], s = g1 * uu;
+        const T dx = UXG ? r[j].y : r[j].x, sx = UXG ? r[j].x : SX[j];
+        const T Q = uu * dx - d * d, Sv = uu * sx;
+        const T e2 = e * e;
+        const T phi = e2 * e * Q * third + e2 * m * d + half(e2 * Sv) + e * m * s - e * uu * uu;
+        D[j] = half(e2 * Q) + e * m * d + e * Sv + m * s;     // d is no longer needed
+        b0[j] = mk(phi, from_int<T>(0));
+        f_eta[o + j] = -to_f64(m);
+      }
+      __syncthreads();
+    } else {
+      for (int j = threadIdx.x; j < n; j += kMrNT) {
+        if (what == 0) {
+          M[j] = r[j].x;
+          ZX[j] = r[j].y;
+        } else if (what == 2) {
+          D[j] = r[j].x;
+          M[j] = r[j].y;
+        } else {
+          ZX[j] = r[j].x;
+          SX[j] = r[j].y;
+        }
+      }
+      __syncthreads();
+    }
   }
 }
 
@@ -716,8 +756,10 @@ cudaError_t mr_launch_precond(const Layout1d& lay, int first, int num, const Sol
 cudaError_t mr_launch_pcg(const Layout1d& lay, int first, int num, int precision,
                           const double* eta, const double* hx, const double* b, double* x,
                           const SolveRec* given, int kind, double rtol, double rtol_inner,
-                          int maxit, int max_refine, SolveRec* rec, void* ws, cudaStream_t s) {
+                          int maxit, int max_refine, SolveRec* rec, void* ws, void* ux,
+                          cudaStream_t s) {
   MrPcgArgs a;
+  a.ux = ux;
   a.eta = eta;
   a.hx = hx;
   a.b = b;
@@ -745,19 +787,17 @@ cudaError_t mr_launch_pcg(const Layout1d& lay, int first, int num, int precision
 cudaError_t mr_launch_rhs(const Layout1d& lay, int first, int num, int precision, double g,
                           const double* eta, const double* u, const double* h,
                           const double* hx, double* f_eta, double* f_U, double* scratch,
-                          cudaStream_t s) {
+                          bool ux_given, cudaStream_t s) {
   const size_t sm = mr_smem(lay);
-  cudaError_t e;
-  if (precision == SGN_PREC_MIXED) {
-    if ((e = mr_attr(k_mr_rhs<df>, sm))) return e;
-    k_mr_rhs<df><<<num, kMrNT, sm, s>>>(mr_args(lay, first), g, eta, u, h, hx, f_eta, f_U,
-                                       scratch, lay.points);
-  } else {
-    if ((e = mr_attr(k_mr_rhs<double>, sm))) return e;
-    k_mr_rhs<double><<<num, kMrNT, sm, s>>>(mr_args(lay, first), g, eta, u, h, hx, f_eta, f_U,
-                                           scratch, lay.points);
-  }
-  return cudaGetLastError();
+  auto go = [&](auto k) -> cudaError_t {
+    const cudaError_t e = mr_attr(k, sm);
+    if (e) return e;
+    k<<<num, kMrNT, sm, s>>>(mr_args(lay, first), g, eta, u, h, hx, f_eta, f_U, scratch,
+                             lay.points);
+    return cudaGetLastError();
+  };
+  if (precision == SGN_PREC_MIXED) return ux_given ? go(k_mr_rhs<df, true>) : go(k_mr_rhs<df, false>);
+  return ux_given ? go(k_mr_rhs<double, true>) : go(k_mr_rhs<double, false>);
 }
 
 }  // namespace sgn

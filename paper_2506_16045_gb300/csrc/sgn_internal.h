@@ -173,11 +173,12 @@ cudaError_t mr_launch_precond(const Layout1d& lay, int first, int num, const Sol
 cudaError_t mr_launch_pcg(const Layout1d& lay, int first, int num, int precision,
                           const double* eta, const double* hx, const double* b, double* x,
                           const SolveRec* given, int kind, double rtol, double rtol_inner,
-                          int maxit, int max_refine, SolveRec* rec, void* ws, cudaStream_t s);
+                          int maxit, int max_refine, SolveRec* rec, void* ws, void* ux,
+                          cudaStream_t s);
 cudaError_t mr_launch_rhs(const Layout1d& lay, int first, int num, int precision, double g,
                           const double* eta, const double* u, const double* h,
                           const double* hx, double* f_eta, double* f_U, double* scratch,
-                          cudaStream_t s);
+                          bool ux_given, cudaStream_t s);
 
 struct Layout2d;
 
