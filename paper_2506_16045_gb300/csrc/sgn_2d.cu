@@ -1136,7 +1136,7 @@ cudaError_t layout2d_create(Layout2d& L, const sgn_grid& g) {
 namespace {
 
 PersistArgs2d persist_args(const Layout2d& L, const void* tw32) {
-  PersistArgs2d a;
+  PersistArgs2d a = {};
   a.inst = static_cast<const PInst2d*>(L.pinst);
   a.B = 1;
   a.nx = L.nx;
@@ -1999,7 +1999,7 @@ cudaError_t launch_pcg2d_batch(Layout2d& first, Batch2d& Bt, const void* tw64, c
     }
   }
   const PersistArgs2d pa = [&] {
-    PersistArgs2d a;
+    PersistArgs2d a = {};
     a.inst = static_cast<const PInst2d*>(Bt.pinst);
     a.B = B;
     a.nx = first.nx;

@@ -238,13 +238,17 @@ struct PersistArgs2d {
   unsigned* bar;          // arrival counter of the grid barriers
   int* err;               // set when a barrier wait gives up
   const void* tw32;       // float32 twiddle table
+  // grids whose nx or ny is not a power of two: the sides' float32 stage tables (mr_fft.cuh)
+  bool mr;
+  const void* mr_twx;
+  const void* mr_twy;
 };
 
 }  // namespace d2
 
 // Launchers of the persistent inner solve (sgn_2d_pcg.cu).
 // CTAs of the cooperative grid: every SM's resident CTAs, at most the largest phase's units
-cudaError_t persist2d_grid(int nx, int ny, int B, int* grid);
+cudaError_t persist2d_grid(int nx, int ny, int B, int* grid, bool mr = false);
 // Zeroes the barrier words, then runs the inner solves of args.inst[0..B) to completion.
 cudaError_t launch_pcg2d_persist(const d2::PersistArgs2d& args, int grid, cudaStream_t s);
 

@@ -17,7 +17,8 @@
 //                          float64, or float32 inner solves inside float64 refinement)
 //   right-hand side       (Eq:DAE_DSWE with Def:bigF in 2d, float64)
 // A solve runs as one cached graph whose loops are while nodes driven by device-side
-// decisions (build_mr_graph); under stream capture the same steps run host-driven.
+// decisions (build_mr_graph), the float32 inner solves as one persistent launch each; under
+// stream capture the method runs host-driven, a kernel at a time.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -401,26 +402,6 @@ __global__ void k2m_decide(MrScal* S, cudaGraphConditionalHandle h) {
   cudaGraphSetConditional(h, go);
 }
 
-// mixed: the inner solve starts from d = 0 with r.z in rz
-__global__ void k2m_inner_init(MrScal* S, cudaGraphConditionalHandle h) {
-  S->it0 = S->iters;
-  S->st_in = SGN_OK;
-  S->skip = 0;
-  unsigned go = 0u;
-  if (sqrt(fmax(S->rz, 0.0)) > S->tol) {
-    if (S->iters >= S->maxit) S->st_in = SGN_ERR_NOT_CONVERGED;
-    else go = 1u;
-  }
-  cudaGraphSetConditional(h, go);
-}
-
-// mixed: after an inner solve; a float32 breakdown without progress ends the solve
-__global__ void k2m_after_inner(MrScal* S) {
-  if (S->st_in == SGN_ERR_BREAKDOWN && S->iters == S->it0) S->status = SGN_ERR_BREAKDOWN;
-  S->refinements += 1;
-  S->skip = 0;
-}
-
 // y += sign alpha x, p = z + beta p, x += nr d, out = scale r: the loop's vector updates with
 // their scalars read on the device (skipped after a breakdown in the same iteration)
 template <typename Sv>
@@ -443,20 +424,129 @@ __global__ void k2m_xpby_s(long long n, const MrScal* S, const Sv* __restrict__ 
     p[i] = (Sv)((double)z[i] + b * (double)p[i]);
 }
 
-__global__ void k2m_correct_s(long long n, const MrScal* S, const float* __restrict__ d,
-                              double* __restrict__ x) {
-  const double s = S->nr;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-       i += (long long)gridDim.x * blockDim.x)
-    x[i] += s * (double)d[i];
-}
-
 __global__ void k2m_scale_s(long long n, const MrScal* S, const double* __restrict__ r,
                             float* __restrict__ out) {
   const double s = S->scale;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x)
     out[i] = (float)(s * r[i]);
+}
+
+// ---- the float32 inner solve on half spectra (the persistent kernel of sgn_2d_pcg.cu) ---------
+// Its vectors and transform planes are half spectra [nx/2 + 1][ny], column-major.
+using d2::PInst2d;
+using d2::PersistArgs2d;
+
+// float32 eta, h_x, h_y
+__global__ void k2m_ehh(long long P, const double* __restrict__ eta, const double* __restrict__ gh,
+                        float* __restrict__ ehh) {
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < P;
+       i += (long long)gridDim.x * blockDim.x) {
+    ehh[i] = (float)eta[i];
+    ehh[P + i] = (float)gh[i];
+    ehh[2 * P + i] = (float)gh[P + i];
+  }
+}
+
+// From the packed spectrum Z of the two components of the scaled residual: r, x = 0, p = 0,
+// and the partial sums of r.A^{-1}r (Parseval weights of the half spectrum).
+__global__ void __launch_bounds__(256) k2m_to_half(Grid2 G, const cplx<float>* __restrict__ Z,
+                                                  const PInst2d* __restrict__ I,
+                                                  const SolveRec* __restrict__ rec,
+                                                  double* __restrict__ part) {
+  __shared__ double red[256 / 32 + 1];
+  const int h = G.nx / 2;
+  const long long HP = (long long)(h + 1) * G.ny;
+  const float sig = (float)rec->sigma, al = (float)rec->alpha, is = recip(sig);
+  const float kxu = (float)G.kx, kyu = (float)G.ky;
+  const cplx<float> zero = mk(0.0f, 0.0f);
+  double acc = 0.0;
+  for (long long i = blockIdx.x * 256LL + threadIdx.x; i < HP; i += 256LL * gridDim.x) {
+    const int c = (int)(i / G.ny), y = (int)(i - (long long)c * G.ny);
+    const int my = y == 0 ? 0 : G.ny - y, mx = c == 0 ? 0 : G.nx - c;
+    const cplx<float> z = Z[(long long)y * G.nx + c], zm = conj(Z[(long long)my * G.nx + mx]);
+    const cplx<float> U = mk((z.x + zm.x) * 0.5f, (z.y + zm.y) * 0.5f);
+    const cplx<float> V = mk((z.y - zm.y) * 0.5f, (zm.x - z.x) * 0.5f);
+    I->r[0][i] = U;
+    I->r[1][i] = V;
+    I->x[0][i] = zero;
+    I->x[1][i] = zero;
+    I->p[0][i] = zero;
+    I->p[1][i] = zero;
+    const float kx = c == h ? 0.0f : kxu * (float)c, ky = kyu * (float)wave_index(y, G.ny);
+    const float f = al * recip(fmaf(al, kx * kx + ky * ky, sig));
+    const cplx<float> kr = mk(kx * U.x + ky * V.x, kx * U.y + ky * V.y);
+    const float q = U.x * (U.x - f * kx * kr.x) + U.y * (U.y - f * kx * kr.y) +
+                    V.x * (V.x - f * ky * kr.x) + V.y * (V.y - f * ky * kr.y);
+    acc += (double)((c == 0 || c == h) ? q * is : 2.0f * q * is);
+  }
+  acc = block_sum<256>(acc, red);
+  if (threadIdx.x == 0) part[blockIdx.x] = acc;
+}
+
+// The inner solve's scalars: r.z, the tolerance in the spectrum's units (P times the real
+// sums), A's symbol; done at once when r.z is below it or no iteration is left.
+__global__ void __launch_bounds__(256) k2m_half_begin(MrScal* S, const SolveRec* rec, Scal2d* sc,
+                                                      const double* __restrict__ part, int nparts,
+                                                      double P) {
+  __shared__ double red[256 / 32 + 1];
+  double v = 0.0;
+  for (int i = threadIdx.x; i < nparts; i += 256) v += part[i];
+  v = block_sum<256>(v, red);
+  if (threadIdx.x != 0) return;
+  S->it0 = S->iters;
+  S->skip = 0;
+  sc->rz = v;
+  sc->tol = S->tol * sqrt(P);
+  sc->sigf = (float)rec->sigma;
+  sc->alphaAf = (float)rec->alpha;
+  sc->isigf = (float)(1.0 / rec->sigma);
+  sc->iters = S->iters;
+  sc->cap = S->maxit;
+  const bool go = sqrt(fmax(v, 0.0)) > sc->tol;
+  sc->status = go && S->iters >= S->maxit ? SGN_ERR_NOT_CONVERGED : SGN_OK;
+  sc->done = !go || S->iters >= S->maxit;
+}
+
+// After it: a float32 breakdown without progress ends the solve, and so does a barrier of the
+// persistent kernel that gave up.
+__global__ void k2m_half_end(MrScal* S, const Scal2d* sc) {
+  S->iters = sc->iters;
+  S->st_in = sc->status;
+  if (S->st_in == SGN_ERR_BREAKDOWN && S->iters == S->it0) S->status = SGN_ERR_BREAKDOWN;
+  if (S->st_in == SGN_ERR_TIMEOUT) S->status = SGN_ERR_TIMEOUT;
+  S->refinements += 1;
+}
+
+// The packed spectrum of the correction's two components from their half spectra
+__global__ void k2m_from_half(Grid2 G, const PInst2d* __restrict__ I, cplx<float>* __restrict__ Z) {
+  const int h = G.nx / 2;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < G.P;
+       i += (long long)gridDim.x * blockDim.x) {
+    const int y = (int)(i / G.nx), c = (int)(i - (long long)y * G.nx);
+    cplx<float> D1, D2;
+    if (c <= h) {
+      D1 = I->x[0][(long long)c * G.ny + y];
+      D2 = I->x[1][(long long)c * G.ny + y];
+    } else {
+      const long long o = (long long)(G.nx - c) * G.ny + (y == 0 ? 0 : G.ny - y);
+      D1 = conj(I->x[0][o]);
+      D2 = conj(I->x[1][o]);
+    }
+    Z[i] = mk(D1.x - D2.y, D1.y + D2.x);
+  }
+}
+
+// x += (nr / P) (Re, Im) Z
+__global__ void k2m_correct_half(long long P, const MrScal* S, const cplx<float>* __restrict__ Z,
+                                 double* __restrict__ x) {
+  const double s = S->nr / (double)P;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < P;
+       i += (long long)gridDim.x * blockDim.x) {
+    const cplx<float> z = Z[i];
+    x[i] += s * (double)z.x;
+    x[P + i] += s * (double)z.y;
+  }
 }
 
 // the report into rec (coefficients kept); x = 0 when b was zero (or not finite)
@@ -602,6 +692,42 @@ cudaError_t smem_attr(K kernel, size_t bytes) {
   return raise_smem(kernel, bytes);
 }
 
+// The inner solve's vectors and planes: nine half planes of (nx/2 + 1) ny complex float32 in
+// the real planes 11 .. 19 (8 P bytes each), beside rf in plane 10.
+PInst2d mr_pinst(const Mr& M) {
+  PInst2d I = {};
+  auto half = [&](int j) { return reinterpret_cast<cplx<float>*>(M.rp(11 + j)); };
+  for (int c = 0; c < 2; ++c) {
+    I.r[c] = half(c);
+    I.x[c] = half(2 + c);
+    I.p[c] = half(4 + c);
+  }
+  for (int q = 0; q < 3; ++q) I.t[q] = half(6 + q);
+  I.ehh = M.L.ehh;
+  I.sc = M.L.sc;
+  I.kxu = M.G.kx;
+  I.kyu = M.G.ky;
+  return I;
+}
+PersistArgs2d mr_persist_args(const Mr& M) {
+  PersistArgs2d a = {};
+  a.inst = static_cast<const PInst2d*>(M.L.pinst);
+  a.B = 1;
+  a.nx = M.G.nx;
+  a.ny = M.G.ny;
+  a.H = M.L.H;
+  a.tw = 1;
+  a.col_units = M.L.H;
+  a.row_units = M.G.ny / 2;
+  a.parts = M.L.pparts;
+  a.bar = M.L.pbar;
+  a.err = reinterpret_cast<int*>(M.L.pbar + 1);
+  a.mr = true;
+  a.mr_twx = M.twx<float>();
+  a.mr_twy = M.twy<float>();
+  return a;
+}
+
 // 2d transform of K planes at Z (stride P); the inverse without the 1/P
 template <typename T>
 cudaError_t fft2(const Mr& M, cplx<T>* Z, int K, bool inv, cudaStream_t s) {
@@ -731,6 +857,14 @@ cudaError_t mr2d_create(Layout2d& L) {
   if ((e = cudaMalloc(&L.mr_sc, sizeof(MrScal)))) return e;
   if ((e = cudaMalloc(&L.stage, sizeof(double) * 7 * L.P))) return e;
   if ((e = cudaMalloc(&L.stage_rec, sizeof(SolveRec) * 2))) return e;
+  // the persistent inner solve of the mixed path
+  if ((e = persist2d_grid(L.nx, L.ny, 1, &L.p_grid, true))) return e;
+  if ((e = cudaMalloc(&L.ehh, sizeof(float) * 3 * L.P))) return e;
+  if ((e = cudaMalloc(&L.pinst, sizeof(PInst2d)))) return e;
+  if ((e = cudaMalloc(&L.pparts, sizeof(double) * (L.H + L.ny / 2)))) return e;
+  if ((e = cudaMalloc(&L.pbar, 2 * sizeof(unsigned)))) return e;
+  const PInst2d pi = mr_pinst(Mr(L));
+  if ((e = cudaMemcpy(L.pinst, &pi, sizeof(pi), cudaMemcpyHostToDevice))) return e;
   return cudaStreamSynchronize(nullptr);          // the tables (legacy stream)
 }
 
@@ -766,8 +900,9 @@ cudaError_t mr2d_precond(const Layout2d& L, const SolveRec* rec, const double* r
 namespace {
 
 // The solve as one graph (inputs from L.stage, options from the scalars, the report to
-// L.stage_rec[1]): the float64 PCG loop, or the refinement loop around the float32 inner
-// loop, as while nodes whose conditions the decision kernels set.
+// L.stage_rec[1]): the float64 PCG loop, or the refinement loop around the persistent float32
+// inner solve, as while nodes whose conditions the decision kernels set.  As a loop of kernels
+// an inner iteration took 29 launches of 3-4 us each on full spectra (384 x 240: 115 us).
 cudaError_t build_mr_graph(const Layout2d& L, bool mixed, bool given, cudaGraphExec_t* out,
                            cudaGraph_t* src) {
   const Mr M(L);
@@ -785,12 +920,7 @@ cudaError_t build_mr_graph(const Layout2d& L, bool mixed, bool given, cudaGraphE
   double* q = M.rp(6);
   double* l = M.rp(8);
   float* rf = M.fp(10);
-  float* pf = M.fp(11);
-  float* zf = M.fp(12);
-  float* qf = M.fp(13);
-  float* df_ = M.fp(14);
-  float* lf = M.fp(15);
-  cudaStream_t cs[3] = {nullptr, nullptr, nullptr};
+  cudaStream_t cs[2] = {nullptr, nullptr};
   cudaGraph_t g = nullptr;
   cudaError_t e = cudaSuccess;
   int capturing = 0;
@@ -865,8 +995,12 @@ cudaError_t build_mr_graph(const Layout2d& L, bool mixed, bool given, cudaGraphE
     }
     if (!e) e = end(1);
   } else {
-    cudaGraphConditionalHandle hout, hin;
-    cudaGraph_t body = nullptr, ibody = nullptr;
+    cudaGraphConditionalHandle hout;
+    cudaGraph_t body = nullptr;
+    if (!e) {
+      k2m_ehh<<<blocks_for(P), 256, 0, cs[0]>>>(P, eta, gh, L.ehh);
+      e = last();
+    }
     if (!e) e = residual64(cs[0]);
     if (!e) e = cudaGraphConditionalHandleCreate(&hout, g, 0, 0);
     if (!e) {
@@ -875,44 +1009,29 @@ cudaError_t build_mr_graph(const Layout2d& L, bool mixed, bool given, cudaGraphE
     }
     if (!e) e = capture_add_while(cs[0], hout, &body);
     if (!e) e = begin(1, body);
-    // the inner solve of G d = r / ||r|| from d = 0
+    // the inner solve of G d = r / ||r|| from d = 0: one persistent launch on half spectra
     if (!e) {
       k2m_scale_s<<<nb, 256, 0, cs[1]>>>(V, S, r, rf);
+      k2m_pack<float, float><<<blocks_for(P), 256, 0, cs[1]>>>(P, rf, rf + P, M.za<float>());
       e = last();
     }
-    if (!e) e = cudaMemsetAsync(df_, 0, sizeof(float) * V, cs[1]);
-    if (!e) e = ainv<float, float>(M, rec, rf, zf, cs[1]);
-    if (!e) e = cudaMemcpyAsync(pf, zf, sizeof(float) * V, cudaMemcpyDeviceToDevice, cs[1]);
-    if (!e) e = cudaGraphConditionalHandleCreate(&hin, body, 0, 0);
+    if (!e) e = fft2<float>(M, M.za<float>(), 1, false, cs[1]);
     if (!e) {
-      k2m_dot1<float><<<kRedBlocks, 256, 0, cs[1]>>>(V, rf, zf, L.mr_dev);
-      k2m_dot2<<<1, 256, 0, cs[1]>>>(L.mr_dev, &S->rz);
-      k2m_inner_init<<<1, 1, 0, cs[1]>>>(S, hin);
+      const PInst2d* I = static_cast<const PInst2d*>(L.pinst);
+      k2m_to_half<<<kRedBlocks, 256, 0, cs[1]>>>(M.G, M.za<float>(), I, rec, L.mr_dev);
+      k2m_half_begin<<<1, 256, 0, cs[1]>>>(S, rec, L.sc, L.mr_dev, kRedBlocks, (double)P);
       e = last();
     }
-    if (!e) e = capture_add_while(cs[1], hin, &ibody);
-    if (!e) e = begin(2, ibody);
-    if (!e) e = applyG<float, float>(M, eta, gh, pf, qf, lf, cs[2]);
+    if (!e) e = launch_pcg2d_persist(mr_persist_args(M), L.p_grid, cs[1]);
     if (!e) {
-      k2m_dot1<float><<<kRedBlocks, 256, 0, cs[2]>>>(V, pf, qf, L.mr_dev);
-      k2m_dot2<<<1, 256, 0, cs[2]>>>(L.mr_dev, &S->pq);
-      k2m_alpha<<<1, 1, 0, cs[2]>>>(S, 1);
-      k2m_axpy_s<float><<<nb, 256, 0, cs[2]>>>(V, S, 1.0, pf, df_);
-      k2m_axpy_s<float><<<nb, 256, 0, cs[2]>>>(V, S, -1.0, qf, rf);
+      k2m_half_end<<<1, 1, 0, cs[1]>>>(S, L.sc);
+      k2m_from_half<<<blocks_for(P), 256, 0, cs[1]>>>(
+          M.G, static_cast<const PInst2d*>(L.pinst), M.za<float>());
       e = last();
     }
-    if (!e) e = ainv<float, float>(M, rec, rf, zf, cs[2]);
+    if (!e) e = fft2<float>(M, M.za<float>(), 1, true, cs[1]);
     if (!e) {
-      k2m_dot1<float><<<kRedBlocks, 256, 0, cs[2]>>>(V, rf, zf, L.mr_dev);
-      k2m_dot2<<<1, 256, 0, cs[2]>>>(L.mr_dev, &S->rzn);
-      k2m_beta<<<1, 1, 0, cs[2]>>>(S, 1, hin);
-      k2m_xpby_s<float><<<nb, 256, 0, cs[2]>>>(V, S, zf, pf);
-      e = last();
-    }
-    if (!e) e = end(2);
-    if (!e) {
-      k2m_after_inner<<<1, 1, 0, cs[1]>>>(S);
-      k2m_correct_s<<<nb, 256, 0, cs[1]>>>(V, S, df_, x);
+      k2m_correct_half<<<blocks_for(P), 256, 0, cs[1]>>>(P, S, M.za<float>(), x);
       e = last();
     }
     if (!e) e = residual64(cs[1]);
@@ -927,7 +1046,7 @@ cudaError_t build_mr_graph(const Layout2d& L, bool mixed, bool given, cudaGraphE
     e = last();
   }
   if (!e) e = end(0);
-  for (int i = 2; i >= 0; --i)
+  for (int i = 1; i >= 0; --i)
     if (capturing & (1 << i)) end(i);          // a failed build: close its captures
   if (!e) e = cudaGraphInstantiate(out, g, 0);
   for (auto& c : cs)

@@ -32,6 +32,7 @@
 #include <cstdio>
 
 #include "sgn_2d_dev.cuh"
+#include "sgn_mr_fft.cuh"
 
 namespace sgn {
 
@@ -199,10 +200,69 @@ __device__ __forceinline__ void pstage(const cplx<float>* __restrict__ src,
 // up to 2^maxb (maxb = 4: radix 16, 3: radix 8), split as evenly as possible.
 __device__ __forceinline__ int pfft_stages(int log2n, int maxb) { return (log2n + maxb - 1) / maxb; }
 
-template <int GT>
-__device__ __forceinline__ cplx<float>* pfft(cplx<float>* a, cplx<float>* b, int log2n, int nb, int S,
-                                          bool inv, const cplx<float>* tws, int t, int g,
-                                          int maxb) {
+// A transform length: its logarithm and stage radices (powers of two), or its mixed-radix
+// stages (MR: radices 8, then 4 or 2, then 5, then 3, tables as mr_fft.cuh lays them out).
+constexpr int kMrStages = 12;
+struct MrStages {
+  int n, ns;
+  int R[kMrStages], p[kMrStages], q[kMrStages];     // radix, sub-length, butterflies n / R
+  unsigned mp[kMrStages];                           // ceil(2^32 / p): i div p by one product
+};
+struct PLen {
+  int log2n, maxb;
+  const MrStages* mr;
+};
+
+// A mixed-radix stage: as pstage, with general indices (three transforms at most).
+template <int R, int GT>
+__device__ __forceinline__ void pstage_mr(const cplx<float>* __restrict__ src,
+                                          cplx<float>* __restrict__ dst, const MrStages& P, int st,
+                                          int nb, int S, bool inv,
+                                          const cplx<float>* __restrict__ tws, int t, int g) {
+  const int q = P.q[st], p = P.p[st];
+  const unsigned mp = P.mp[st];
+#pragma unroll 1
+  for (int gi = t; gi < nb * q; gi += GT) {
+    const int j = (gi >= q) + (gi >= 2 * q), i = gi - j * q;
+    const int k = p > 1 ? i - p * (int)__umulhi((unsigned)i, mp) : 0;
+    cplx<float> x[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) x[r] = src[j * S + pad(i + r * q)];
+    if (p > 1) {
+      const cplx<float>* tb = tws + p - 1 + k;
+#pragma unroll
+      for (int r = 1; r < R; ++r) x[r] = cmul_tw(x[r], tb[(r - 1) * p], inv);
+    }
+    if constexpr (R == 3 || R == 5) mr::mr_dft<float, R>(x, inv);
+    else dft_reg<R>(x, inv);
+    const int o = (i - k) * R + k;
+#pragma unroll
+    for (int s = 0; s < R; ++s) dst[j * S + pad(o + s * p)] = x[s];
+  }
+  gsync<GT>(g);
+}
+
+template <int GT, bool MR>
+__device__ __forceinline__ cplx<float>* pfft(cplx<float>* a, cplx<float>* b, const PLen& len, int nb,
+                                          int S, bool inv, const cplx<float>* tws, int t, int g) {
+  if constexpr (MR) {
+    const MrStages& P = *len.mr;
+    cplx<float>* src = a;
+    cplx<float>* dst = b;
+    for (int st = 0; st < P.ns; ++st) {
+      const int R = P.R[st];
+      if (R == 8) pstage_mr<8, GT>(src, dst, P, st, nb, S, inv, tws, t, g);
+      else if (R == 4) pstage_mr<4, GT>(src, dst, P, st, nb, S, inv, tws, t, g);
+      else if (R == 2) pstage_mr<2, GT>(src, dst, P, st, nb, S, inv, tws, t, g);
+      else if (R == 5) pstage_mr<5, GT>(src, dst, P, st, nb, S, inv, tws, t, g);
+      else pstage_mr<3, GT>(src, dst, P, st, nb, S, inv, tws, t, g);
+      cplx<float>* tmp = src;
+      src = dst;
+      dst = tmp;
+    }
+    return src;
+  }
+  const int log2n = len.log2n, maxb = len.maxb;
   const int ns = pfft_stages(log2n, maxb);
   const int base = log2n / ns, extra = log2n - base * ns;
   int lp = 0;
@@ -343,7 +403,14 @@ struct PSmem {
   cplx<float>* A;       // this group's buffers
   cplx<float>* B;
   cplx<float>* C;       // staged form only
+  PLen lx, ly;          // the transform lengths nx and ny
 };
+
+// the index of -k for a mode index of a length-n transform
+template <bool MR>
+__device__ __forceinline__ int neg_mode(int m, int n) {
+  return MR ? (m == 0 ? 0 : n - m) : (n - m) & (n - 1);
+}
 
 // Sizes in complex float32 entries, both even (16-byte aligned buffers).  A and B each hold
 // three padded transforms; staged, B also takes the raw row pairs of a row unit (6 (nx/2 + 1)
@@ -361,7 +428,7 @@ __host__ __device__ inline int persist_bc(int nx, int ny, bool stg) {
 
 // ---- C1: p update, projection, divergence, column iFFT (column c, group g) -------------
 // The solve's vectors and transform planes are column-major, [H][ny]: a column is contiguous.
-template <bool STG, int GT>
+template <bool STG, int GT, bool MR>
 __device__ __forceinline__ void col_inverse(const PersistArgs2d& a, const PInst2d& I,
                                          const IScal& s, int c, const PSmem& sm, int t, int g) {
   const int ny = a.ny, S = pad_len(ny), nx = a.nx;
@@ -434,7 +501,7 @@ __device__ __forceinline__ void col_inverse(const PersistArgs2d& a, const PInst2
     for (int q = 0; q < 2; ++q) {
       cplx<float>* v = buf + q * S;
       for (int y = t; y <= (ny >> 1); y += GT) {
-        const int ym = (ny - y) & (ny - 1);
+        const int ym = neg_mode<MR>(y, ny);
         const cplx<float> sm2 = v[pad(y)] + conj(v[pad(ym)]);
         const cplx<float> hm = mk(0.5f * sm2.x, 0.5f * sm2.y);
         v[pad(y)] = hm;
@@ -450,7 +517,7 @@ __device__ __forceinline__ void col_inverse(const PersistArgs2d& a, const PInst2
     buf[2 * S + pad(y)] = mul_ik(p1, kx) + mul_ik(p2, ky_of(s, y, ny));
   }
   gsync<GT>(g);
-  const cplx<float>* o = pfft<GT>(sm.A, sm.B, a.logny, 3, S, true, sm.twy, t, g, a.maxb);
+  const cplx<float>* o = pfft<GT, MR>(sm.A, sm.B, sm.ly, 3, S, true, sm.twy, t, g);
   for (int y = t; y < ny; y += GT) {
 #pragma unroll
     for (int q = 0; q < 3; ++q) stcg(I.t[q] + cb + y, o[q * S + pad(y)]);
@@ -458,7 +525,7 @@ __device__ __forceinline__ void col_inverse(const PersistArgs2d& a, const PInst2
 }
 
 // ---- R: C2R, Def:MatrixM pointwise with the p.Gp partial, R2C (row pair y0, group g) -----
-template <bool STG, int GT>
+template <bool STG, int GT, bool MR>
 __device__ __forceinline__ float row_matvec(const PersistArgs2d& a, const PInst2d& I, int y0,
                                             const PSmem& sm, int t, int g) {
   const int nx = a.nx, h = nx >> 1, S = pad_len(nx);
@@ -529,8 +596,9 @@ __device__ __forceinline__ float row_matvec(const PersistArgs2d& a, const PInst2
     }
   }
   gsync<GT>(g);
-  cplx<float>* w = pfft<GT>(sm.A, sm.B, a.lognx, 3, S, true, sm.twx, t, g, a.maxb);
-  const float inv = __int_as_float((127 - a.lognx - a.logny) << 23);   // 1 / (nx ny), exact
+  cplx<float>* w = pfft<GT, MR>(sm.A, sm.B, sm.lx, 3, S, true, sm.twx, t, g);
+  // 1 / (nx ny): exact for powers of two
+  const float inv = MR ? recip((float)(nx * a.ny)) : __int_as_float((127 - a.lognx - a.logny) << 23);
   const float third = 1.0f / 3.0f;
   float part = 0.0f;
   for (int x0 = 0; x0 < nx; x0 += kRows * GT) {
@@ -580,14 +648,14 @@ __device__ __forceinline__ float row_matvec(const PersistArgs2d& a, const PInst2
   }
   gsync<GT>(g);
   cplx<float>* other = w == sm.A ? sm.B : sm.A;
-  const cplx<float>* Y = pfft<GT>(w, other, a.lognx, 3, S, false, sm.twx, t, g, a.maxb);
+  const cplx<float>* Y = pfft<GT, MR>(w, other, sm.lx, 3, S, false, sm.twx, t, g);
   // R2C split of the three packed rows, A = (Y_m + conj Y_{n-m})/2, B = (Y_m - conj Y_{n-m})/(2i),
   // stored back as row pairs of columns m: t0 = (A_0, A_1), t1 = (B_0, B_1), t2 = (A_2, B_2)
   for (int m = t; m <= h; m += GT) {
     cplx<float> A_[3], B_[3];
 #pragma unroll
     for (int r = 0; r < 3; ++r) {
-      const cplx<float> yv = Y[r * S + pad(m)], yc = conj(Y[r * S + pad((nx - m) & (nx - 1))]);
+      const cplx<float> yv = Y[r * S + pad(m)], yc = conj(Y[r * S + pad(neg_mode<MR>(m, nx))]);
       const cplx<float> sm2 = yv + yc, dm = mul_mi(yv - yc);
       A_[r] = mk(0.5f * sm2.x, 0.5f * sm2.y);
       B_[r] = mk(0.5f * dm.x, 0.5f * dm.y);
@@ -601,7 +669,7 @@ __device__ __forceinline__ float row_matvec(const PersistArgs2d& a, const PInst2
 }
 
 // ---- C2: column FFT, G p, x and r updates, r.z partial (column c, group g) ---------------
-template <bool STG, int GT>
+template <bool STG, int GT, bool MR>
 __device__ __forceinline__ float col_forward_update(const PersistArgs2d& a, const PInst2d& I,
                                                     const IScal& s, int c, const PSmem& sm,
                                                     int t, int g) {
@@ -652,7 +720,7 @@ __device__ __forceinline__ float col_forward_update(const PersistArgs2d& a, cons
     }
   }
   gsync<GT>(g);
-  const cplx<float>* o = pfft<GT>(sm.A, sm.B, a.logny, 3, S, false, sm.twy, t, g, a.maxb);
+  const cplx<float>* o = pfft<GT, MR>(sm.A, sm.B, sm.ly, 3, S, false, sm.twy, t, g);
   float part = 0.0f;
   const float al = s.alpha;
   const float kx = kx_of(s, c, nx);
@@ -711,12 +779,14 @@ __device__ __forceinline__ float col_forward_update(const PersistArgs2d& a, cons
 
 // STG: the staged form (a third shared buffer per group takes each unit's global inputs
 // by asynchronous copies, all in flight at once); otherwise loads go through registers.
-template <bool STG, int GT>
+// MR: grids with a side that is not a power of two (mixed-radix transforms, not staged).
+template <bool STG, int GT, bool MR>
 __global__ void __launch_bounds__(kPNT, 1) k2_pcg_persist(const __grid_constant__ PersistArgs2d a) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ IScal S[kMaxBatch2d];
   __shared__ df slot[kPNT / 32];        // the groups' warp totals
   __shared__ int s_stop;
+  __shared__ MrStages mst[MR ? 2 : 1];
   // thread t of group g; the group's buffers after the twiddle table
   const int g = threadIdx.x / GT, t = threadIdx.x - g * GT;
   const int be = persist_be(a.nx, a.ny, STG), bc = persist_bc(a.nx, a.ny, STG);
@@ -727,7 +797,32 @@ __global__ void __launch_bounds__(kPNT, 1) k2_pcg_persist(const __grid_constant_
   sm.A = sm.twx + ntw + (2 * be + bc) * g;
   sm.B = sm.A + be;
   sm.C = sm.B + be;
-  {
+  sm.lx = PLen{a.lognx, a.maxb, &mst[0]};
+  sm.ly = PLen{a.logny, a.maxb, &mst[MR ? 1 : 0]};
+  if constexpr (MR) {
+    const cplx<float>* gx = static_cast<const cplx<float>*>(a.mr_twx);
+    const cplx<float>* gy = static_cast<const cplx<float>*>(a.mr_twy);
+    for (int m = threadIdx.x; m < a.nx - 1; m += kPNT) sm.twx[m] = gx[m];
+    if (a.ny != a.nx)
+      for (int m = threadIdx.x; m < a.ny - 1; m += kPNT) sm.twy[m] = gy[m];
+    if (threadIdx.x < 2) {
+      mr::MrPlan P;
+      const int n = threadIdx.x ? a.ny : a.nx;
+      mr::mr_plan(n, P);
+      MrStages& M = mst[MR ? threadIdx.x : 0];
+      M.n = n;
+      M.ns = P.ns;
+      int p = 1;
+      for (int st = 0; st < P.ns; ++st) {
+        const int R = P.radix(st);
+        M.R[st] = R;
+        M.p[st] = p;
+        M.q[st] = n / R;
+        M.mp[st] = p > 1 ? (unsigned)((0x100000000ull + p - 1) / p) : 0u;
+        p *= R;
+      }
+    }
+  } else {
     // the stage tables of both lengths from the 16384-entry float32 table e^{-2 pi i m / 16384}
     const cplx<float>* tg = static_cast<const cplx<float>*>(a.tw32);
     for (int which = 0; which < (a.ny == a.nx ? 1 : 2); ++which) {
@@ -782,7 +877,7 @@ __global__ void __launch_bounds__(kPNT, 1) k2_pcg_persist(const __grid_constant_
     for (int u = slot0; u < B * CU; u += nslots) {
       const int b = u / CU, c = u - b * CU;
       if (S[b].done) continue;
-      col_inverse<STG, GT>(a, a.inst[b], S[b], c, sm, t, g);
+      col_inverse<STG, GT, MR>(a, a.inst[b], S[b], c, sm, t, g);
       gsync<GT>(g);
     }
     if ((stop = grid_barrier(a.bar, a.err, target, &s_stop))) break;
@@ -790,7 +885,7 @@ __global__ void __launch_bounds__(kPNT, 1) k2_pcg_persist(const __grid_constant_
     for (int u = slot0; u < B * RU; u += nslots) {
       const int b = u / RU, pr = u - b * RU;
       if (S[b].done) continue;
-      const float part = row_matvec<STG, GT>(a, a.inst[b], 2 * pr, sm, t, g);
+      const float part = row_matvec<STG, GT, MR>(a, a.inst[b], 2 * pr, sm, t, g);
       group_part<GT>(part, slot, a.parts + (long long)b * RU + pr, t, g);
     }
     if ((stop = grid_barrier(a.bar, a.err, target, &s_stop))) break;
@@ -810,7 +905,7 @@ __global__ void __launch_bounds__(kPNT, 1) k2_pcg_persist(const __grid_constant_
     for (int u = slot0; u < B * CU; u += nslots) {
       const int b = u / CU, c = u - b * CU;
       if (S[b].done) continue;
-      const float part = col_forward_update<STG, GT>(a, a.inst[b], S[b], c, sm, t, g);
+      const float part = col_forward_update<STG, GT, MR>(a, a.inst[b], S[b], c, sm, t, g);
       group_part<GT>(part, slot, parts2 + (long long)b * CU + c, t, g);
     }
     if ((stop = grid_barrier(a.bar, a.err, target, &s_stop))) break;
@@ -863,21 +958,24 @@ static size_t persist_smem(int nx, int ny, bool stg, int gt) {
 }
 
 using PersistKernel = void (*)(PersistArgs2d);
-static PersistKernel persist_kernel(bool stg, int gt) {
-  if (gt == 256) return stg ? k2_pcg_persist<true, 256> : k2_pcg_persist<false, 256>;
-  return stg ? k2_pcg_persist<true, 128> : k2_pcg_persist<false, 128>;
+static PersistKernel persist_kernel(bool stg, int gt, bool mr) {
+  if (mr) return gt == 256 ? k2_pcg_persist<false, 256, true> : k2_pcg_persist<false, 128, true>;
+  if (gt == 256) return stg ? k2_pcg_persist<true, 256, false> : k2_pcg_persist<false, 256, false>;
+  return stg ? k2_pcg_persist<true, 128, false> : k2_pcg_persist<false, 128, false>;
 }
 
 // The staged form runs where its shared memory (with the kernel's static part) fits one
 // CTA on this device: with 128-thread groups sides up to 512, with 256-thread groups up to
 // 1024, on a 227 KB part.
-static cudaError_t persist_staged(int nx, int ny, int gt, bool* stg) {
+static cudaError_t persist_staged(int nx, int ny, int gt, bool mr, bool* stg) {
+  *stg = false;
+  if (mr) return cudaSuccess;         // rows of nx floats need not start on 16 bytes
   int dev = 0, optin = 0;
   cudaError_t e;
   if ((e = cudaGetDevice(&dev))) return e;
   if ((e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev))) return e;
   cudaFuncAttributes fa;
-  if ((e = cudaFuncGetAttributes(&fa, persist_kernel(true, gt)))) return e;
+  if ((e = cudaFuncGetAttributes(&fa, persist_kernel(true, gt, false)))) return e;
   *stg = fa.sharedSizeBytes + persist_smem(nx, ny, true, gt) <= (size_t)optin;
   return cudaSuccess;
 }
@@ -908,17 +1006,17 @@ bool persist2d_tile_ok(int nx, int ny, int tw) {
 
 // Resident CTAs of the persistent kernel on this device (one per SM: 512 threads of up to
 // 128 registers), at most the largest phase's unit count.
-cudaError_t persist2d_grid(int nx, int ny, int B, int* grid) {
+cudaError_t persist2d_grid(int nx, int ny, int B, int* grid, bool mr) {
   cudaError_t e;
   PersistKernel k128 = nullptr;
   size_t smem128 = 0;
   for (int gt : {128, 256}) {
     bool stg = false;
-    if ((e = persist_staged(nx, ny, gt, &stg))) return e;
+    if ((e = persist_staged(nx, ny, gt, mr, &stg))) return e;
     const size_t smem = persist_smem(nx, ny, stg, gt);
-    if ((e = raise_smem(persist_kernel(stg, gt), smem))) return e;
+    if ((e = raise_smem(persist_kernel(stg, gt, mr), smem))) return e;
     if (gt == 128) {
-      k128 = persist_kernel(stg, gt);
+      k128 = persist_kernel(stg, gt, mr);
       smem128 = smem;
     }
   }
@@ -942,7 +1040,7 @@ cudaError_t launch_pcg2d_persist(const PersistArgs2d& args, int grid, cudaStream
   if (e) return e;
   const int gt = persist_gt(args, grid);
   bool stg = false;
-  if ((e = persist_staged(args.nx, args.ny, gt, &stg))) return e;
+  if ((e = persist_staged(args.nx, args.ny, gt, args.mr, &stg))) return e;
   const size_t smem = persist_smem(args.nx, args.ny, stg, gt);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
@@ -954,7 +1052,7 @@ cudaError_t launch_pcg2d_persist(const PersistArgs2d& args, int grid, cudaStream
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, persist_kernel(stg, gt), args);
+  return cudaLaunchKernelEx(&cfg, persist_kernel(stg, gt, args.mr), args);
 }
 
 }  // namespace sgn
