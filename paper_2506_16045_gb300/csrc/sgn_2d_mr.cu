@@ -36,9 +36,9 @@ using mr::MrPlan;
 using mr::mr_plan;
 
 constexpr int kRowNT = 128;            // threads of a row-pass CTA
-constexpr int kRowElems = 2048;        // complex entries per row-pass CTA (whole rows)
+constexpr int kRowElems = 2048;        // complex entries per row-pass CTA at most (whole rows)
 constexpr int kColNT = 256;            // threads of a column-pass CTA
-constexpr int kColTile = 4;            // columns per column-pass CTA
+constexpr int kColTile = 4;            // columns per column-pass CTA at most
 constexpr int kRedBlocks = 256;        // first-stage blocks of a dot product
 constexpr int kMaxSide = 1024;
 constexpr double kPi2 = 6.283185307179586476925286766559;
@@ -86,16 +86,16 @@ __global__ void __launch_bounds__(kRowNT) k2m_rows(cplx<T>* __restrict__ Z, int 
   for (int i = threadIdx.x; i < cnt; i += kRowNT) base[i] = r[i];
 }
 
-// columns x0 .. x0 + kColTile - 1 of every plane, gathered as kColTile sequences of ny
+// columns x0 .. x0 + tile - 1 of every plane, gathered as tile sequences of ny
 template <typename T>
 __global__ void __launch_bounds__(kColNT) k2m_cols(cplx<T>* __restrict__ Z, int nx, int ny,
-                                                  long long P, bool inv,
+                                                  long long P, int tile, bool inv,
                                                   const cplx<T>* __restrict__ tw) {
   extern __shared__ __align__(16) unsigned char smem[];
   cplx<T>* a = reinterpret_cast<cplx<T>*>(smem);
-  cplx<T>* b = a + (size_t)kColTile * ny;
-  const int x0 = blockIdx.x * kColTile;
-  const int cols = min(kColTile, nx - x0);
+  cplx<T>* b = a + (size_t)tile * ny;
+  const int x0 = blockIdx.x * tile;
+  const int cols = min(tile, nx - x0);
   cplx<T>* base = Z + (long long)blockIdx.y * P + x0;
   const int cnt = ny * cols;
   for (int i = threadIdx.x; i < cnt; i += kColNT) {
@@ -728,21 +728,25 @@ PersistArgs2d mr_persist_args(const Mr& M) {
   return a;
 }
 
-// 2d transform of K planes at Z (stride P); the inverse without the 1/P
+// 2d transform of K planes at Z (stride P); the inverse without the 1/P.  Rows and columns per
+// CTA: as many as give every SM two CTAs (a float64 pass of one 384 x 240 plane ran on 48 and
+// 96 of the 152 SMs with 2048 entries and four columns per CTA, 31 and 18 us), at most
+// kRowElems entries and kColTile columns.
 template <typename T>
 cudaError_t fft2(const Mr& M, cplx<T>* Z, int K, bool inv, cudaStream_t s) {
   const int nx = M.G.nx, ny = M.G.ny;
-  const int nb = max(1, kRowElems / nx);
+  const int nb = max(1, min(kRowElems / nx, ny * K / (2 * kSMs)));
   size_t sm = (size_t)2 * nb * nx * sizeof(cplx<T>);
   cudaError_t e = smem_attr(k2m_rows<T>, sm);
   if (e) return e;
   k2m_rows<T><<<dim3((ny + nb - 1) / nb, K), kRowNT, sm, s>>>(Z, nx, ny, M.G.P, nb, inv,
                                                              M.twx<T>());
   if ((e = cudaGetLastError())) return e;
-  sm = (size_t)2 * kColTile * ny * sizeof(cplx<T>);
+  const int tile = max(1, min(kColTile, nx * K / (2 * kSMs)));
+  sm = (size_t)2 * tile * ny * sizeof(cplx<T>);
   if ((e = smem_attr(k2m_cols<T>, sm))) return e;
-  k2m_cols<T><<<dim3((nx + kColTile - 1) / kColTile, K), kColNT, sm, s>>>(Z, nx, ny, M.G.P, inv,
-                                                                         M.twy<T>());
+  k2m_cols<T><<<dim3((nx + tile - 1) / tile, K), kColNT, sm, s>>>(Z, nx, ny, M.G.P, tile, inv,
+                                                                 M.twy<T>());
   return cudaGetLastError();
 }
 
