@@ -26,7 +26,7 @@
 // groups, up to 1024 with 256-thread groups), the staged form gives each group a third
 // buffer and issues all of a unit's input copies at once, so a unit waits for memory once
 // instead of once per batch of rows.  Each barrier waits at most
-// kBarrierTimeoutNs; a CTA that gives up sets the error word, every CTA then leaves the
+// kBarrierTimeoutNs; a CTA that gives up sets the counter's top bit, every CTA then leaves the
 // loop at its next barrier, and the solve reports SGN_ERR_TIMEOUT.  The launch is
 // cooperative, so every CTA of the grid is resident at once.
 #include <cstdio>
@@ -46,9 +46,14 @@ constexpr int kPNT = 512;                 // threads per CTA
 constexpr int kRows = 1;                  // rows a thread loads per batch: with every phase
                                           // inlined, more would spill past 128 registers
 constexpr unsigned long long kBarrierTimeoutNs = 2000000000ull;   // 2 s
+constexpr unsigned kStopBit = 0x80000000u;      // of the arrival counter: leave the kernel
 
-struct IScal {            // per-instance scalars, identical in every CTA
-  double rz, tol, pq;
+// Per-instance scalars, identical in every CTA.  Double-float, not float64: one warp of every
+// CTA adds the partials and one lane forms alpha and beta between two barriers, where a float64
+// add is 64 clocks and a division or square root 700-1000 (the two sums took 7200 of 60000
+// clocks per iteration at 512^2; with the barrier below, 4 RK4 steps: 16.8 -> 16.2 ms).
+struct IScal {
+  df rz, tol2;
   float alpha, beta, sigf, alAf, isigf, kxu, kyu;
   int iters, cap, done, status;
 };
@@ -309,51 +314,69 @@ __device__ __forceinline__ void cp_wait_all() { asm volatile("cp.async.wait_all;
 
 // Grid-wide barrier on a monotone arrival counter: the k-th barrier of the launch waits for
 // k * gridDim.x arrivals.  Returns true when the launch must stop (a wait gave up here or
-// in another CTA).
+// in another CTA: the counter's top bit).  One release add and one acquire load that sees
+// the last arrival are the whole round trip; the timer is read, and the poll slowed down,
+// only every 64 polls, and the stop bit travels with the count (a second fence and a load
+// of the error word were another trip to the L2 in each of the three barriers).
 __device__ __forceinline__ bool grid_barrier(unsigned* bar, int* err, unsigned& target,
                                              int* s_stop) {
   target += gridDim.x;
   __syncthreads();
   if (threadIdx.x == 0) {
-    __threadfence();
-    atomicAdd(bar, 1u);
-    const unsigned long long t0 = global_ns();
-    int stop = 0;
-    while (ld_acquire(bar) < target) {
-      if (global_ns() - t0 > kBarrierTimeoutNs) {
-        atomicExch(err, 1);
-        stop = 1;
-        break;
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
+    unsigned long long t0 = 0;
+    unsigned v, polls = 0;
+    while ((v = ld_acquire(bar)) < target) {
+      if ((++polls & 63u) == 0) {
+        const unsigned long long t = global_ns();
+        if (t0 == 0) t0 = t;
+        if (t - t0 > kBarrierTimeoutNs) {
+          atomicExch(err, 1);
+          v = atomicOr(bar, kStopBit) | kStopBit;
+          break;
+        }
+        __nanosleep(64);
       }
-      __nanosleep(64);
     }
-    __threadfence();
-    *s_stop = stop | *reinterpret_cast<volatile int*>(err);
+    *s_stop = (v & kStopBit) ? 1 : 0;
   }
   __syncthreads();
   return *s_stop != 0;
 }
 
-// Sum of the per-unit partials of every live instance (units [b U, b U + U)), each summed by
-// one warp in a fixed order; fin(b, total) runs on one lane per instance.
+__device__ __forceinline__ df ld_part(const double* p) {
+  const float2 v = __ldcg(reinterpret_cast<const float2*>(p));
+  return df(v.x, v.y);
+}
+// a / b rounded to float32 (the float32 quotient corrected by its double-float remainder)
+__device__ __forceinline__ float quot(df a, df b) {
+  const float q = a.hi / b.hi;
+  const df r = a - b * df(q, 0.0f);
+  return q + r.hi / b.hi;
+}
+
+// Sum of the per-unit partials (double-float) of every live instance (units [b U, b U + U)),
+// each summed by one warp in a fixed order; fin(b, total) runs on one lane per instance.
 template <typename Fin>
 __device__ __forceinline__ void sum_units(const double* parts, int U, IScal* S, int B, Fin fin) {
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
   for (int b = w; b < B; b += kPNT / 32) {
     if (S[b].done) continue;
-    double acc = 0.0;
+    df acc(0.0f, 0.0f);
     for (int i0 = 0; i0 < U; i0 += 8 * 32) {
-      double v[8];
+      df v[8];
 #pragma unroll
       for (int k = 0; k < 8; ++k) {
         const int i = i0 + l + 32 * k;
-        v[k] = i < U ? __ldcg(parts + (long long)b * U + i) : 0.0;
+        v[k] = i < U ? ld_part(parts + (long long)b * U + i) : df(0.0f, 0.0f);
       }
 #pragma unroll
-      for (int k = 0; k < 8; ++k) acc += v[k];
+      for (int k = 0; k < 8; ++k) acc = acc + v[k];
     }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    for (int o = 16; o > 0; o >>= 1)
+      acc = acc + df(__shfl_xor_sync(0xffffffffu, acc.hi, o),
+                     __shfl_xor_sync(0xffffffffu, acc.lo, o));
     if (l == 0) fin(b, acc);
   }
   __syncthreads();
@@ -373,8 +396,8 @@ __device__ __forceinline__ void ainv(const IScal& s, float kx, float ky, cplx<fl
   z2 = (r2 - kr * (f * ky)) * s.isigf;
 }
 
-// Sum of the float partials of group g in double-float, stored as a double to `out` by the
-// group's thread 0 (warp shuffles, then the group's four warp totals in order).
+// Sum of the float partials of group g in double-float, stored to `out` by the group's
+// thread 0 (warp shuffles, then the group's four warp totals in order).
 template <int GT>
 __device__ __forceinline__ void group_part(float v, df* slot, double* out, int t, int g) {
   df a(v, 0.0f);
@@ -389,7 +412,7 @@ __device__ __forceinline__ void group_part(float v, df* slot, double* out, int t
     df r = slot[g * (GT / 32)];
 #pragma unroll
     for (int w = 1; w < GT / 32; ++w) r = r + slot[g * (GT / 32) + w];
-    __stcg(out, (double)r.hi + (double)r.lo);
+    __stcg(reinterpret_cast<float2*>(out), make_float2(r.hi, r.lo));
   }
   gsync<GT>(g);
 }
@@ -841,13 +864,13 @@ __global__ void __launch_bounds__(kPNT, 1) k2_pcg_persist(const __grid_constant_
     }
   }
   const int B = a.B, CU = a.col_units, RU = a.row_units;
-  const long long P = (long long)a.nx * a.ny;
+  const float Pf = (float)(a.nx * a.ny), iPf = 1.0f / Pf;
+  const df inv_p(iPf, fmaf(-iPf, Pf, 1.0f) * iPf);    // 1/P to 48 bits
   for (int b = threadIdx.x; b < B; b += kPNT) {
     const Scal2d* sc = a.inst[b].sc;
     IScal s;
-    s.rz = sc->rz;
-    s.tol = sc->tol;
-    s.pq = 0.0;
+    s.rz = df(sc->rz);
+    s.tol2 = df(sc->tol * sc->tol);
     s.alpha = 0.0f;
     s.beta = 0.0f;
     s.sigf = sc->sigf;
@@ -890,14 +913,12 @@ __global__ void __launch_bounds__(kPNT, 1) k2_pcg_persist(const __grid_constant_
     }
     if ((stop = grid_barrier(a.bar, a.err, target, &s_stop))) break;
     // alpha = r.z / p.Gp (p.Gp in the half-spectrum units of r.z: P times the real sum)
-    sum_units(a.parts, RU, S, B, [&](int b, double tot) {
-      const double pq = tot * (double)P;
-      if (!(pq > 0.0) || !isfinite(pq)) {
+    sum_units(a.parts, RU, S, B, [&](int b, df tot) {
+      if (!(tot.hi > 0.0f) || !isfinite(tot.hi)) {
         S[b].status = SGN_ERR_BREAKDOWN;
         S[b].done = 1;
       } else {
-        S[b].pq = pq;
-        S[b].alpha = (float)(S[b].rz / pq);
+        S[b].alpha = quot(S[b].rz * inv_p, tot);
       }
     });
     // ---- C2
@@ -909,16 +930,16 @@ __global__ void __launch_bounds__(kPNT, 1) k2_pcg_persist(const __grid_constant_
       group_part<GT>(part, slot, parts2 + (long long)b * CU + c, t, g);
     }
     if ((stop = grid_barrier(a.bar, a.err, target, &s_stop))) break;
-    sum_units(parts2, CU, S, B, [&](int b, double rz) {
+    sum_units(parts2, CU, S, B, [&](int b, df rz) {
       IScal& s = S[b];
       s.iters += 1;
-      if (!isfinite(rz)) {
+      if (!isfinite(rz.hi)) {
         s.status = SGN_ERR_BREAKDOWN;
         s.done = 1;
       } else {
-        s.beta = (float)(rz / s.rz);
+        s.beta = quot(rz, s.rz);
         s.rz = rz;
-        if (sqrt(rz) <= s.tol) {
+        if ((rz - s.tol2).hi <= 0.0f) {
           s.done = 1;
         } else if (s.iters >= s.cap) {
           s.status = SGN_ERR_NOT_CONVERGED;
@@ -931,7 +952,7 @@ __global__ void __launch_bounds__(kPNT, 1) k2_pcg_persist(const __grid_constant_
   for (int b = threadIdx.x; b < B; b += kPNT) {
     Scal2d* sc = a.inst[b].sc;
     const IScal& s = S[b];
-    sc->rz = s.rz;
+    sc->rz = to_f64(s.rz);
     sc->iters = s.iters;
     sc->status = stop ? SGN_ERR_TIMEOUT : s.status;
     sc->done = 1;
