@@ -18,6 +18,7 @@
 #include <vector>
 
 #include "sgn_2d_dev.cuh"
+#include "sgn_2d_fft.cuh"
 
 namespace sgn {
 
@@ -71,7 +72,8 @@ __device__ __forceinline__ void grid_finish(double s, double* parts, Scal2d* sc,
 
 // =======================================================================================
 // Column pass: tiles of TW columns of K half planes, transposed into shared memory
-// (column c of plane q at buf + (q TW + c) * (ny + 1)), transformed along y.
+// (column c of plane q at buf + (q TW + c) * stride), transformed along y.  In spectral space
+// the threads walk the positions (every row is its own sector, in any order).
 // =======================================================================================
 enum ColMode { COL_FWD = 0, COL_INV = 1, COL_MATVEC_IN = 2, COL_MATVEC_OUT = 3 };
 
@@ -93,22 +95,38 @@ struct ColArgs {
   int check_done;           // return immediately when sc->done
 };
 
-template <typename T, int TW, int MAXB, int MODE>
-__global__ void __launch_bounds__(kColNT, 1) k2_cols(Modes2d M, int log2ny, const void* t64,
+// Stride of the columns in shared memory: of two columns the second is four 16-byte banks off.
+template <int TW>
+__host__ __device__ constexpr int col_stride(int ny) { return TW == 1 ? ny : ny + 4; }
+
+template <typename T, int TW, int NT, int MODE>
+__global__ void __launch_bounds__(NT, NT < 512 ? 2 : 1) k2_cols(Modes2d M, int log2ny, const void* t64,
                                                      const void* t32, ColArgs a) {
   if (a.check_done && ((volatile Scal2d*)a.sc)->done) return;
   extern __shared__ __align__(16) unsigned char smem[];
   cplx<T>* buf = reinterpret_cast<cplx<T>*>(smem);
   const cplx<T>* tw = Tw<T>::get(t64, t32);
-  const int ny = M.ny, H = M.H, stride = ny + 1;
+  const int ny = M.ny, H = M.H, stride = col_stride<TW>(ny);
   const int c0 = blockIdx.x * TW;
   const int nplanes = (MODE == COL_MATVEC_IN || MODE == COL_MATVEC_OUT) ? 3 : a.K;
   using TP = typename WorkP<T>::type;         // per-mode precision (float32 for float32)
   const ModesT<TP> MT(M);
+  constexpr bool inverse = (MODE == COL_INV || MODE == COL_MATVEC_IN);
+  cplx<T>* tab = buf + nplanes * TW * stride;
+  fill_tw2(tab, log2ny, tw);
+  AinvT<TP> Ai{};
+  TP beta = 0;
+  if constexpr (MODE == COL_MATVEC_IN && std::is_same<T, TP>::value) {
+    if (a.pupdate) {
+      Ai = ainv_of(a.sc, T(0));
+      beta = cg_beta(a.sc, T(0));
+    }
+  }
 
   // ---- load
-  for (int e = threadIdx.x; e < TW * ny; e += kColNT) {
-    const int y = e / TW, c = e % TW, col = c0 + c;
+  for (int e = threadIdx.x; e < TW * ny; e += NT) {
+    const int p = e / TW, c = e % TW, col = c0 + c, y = inverse ? mode_at(p, log2ny) : p;
+    const int sp = sw2(p);
     const long long gi = (long long)y * H + col;
     const bool ok = col < H;
     if constexpr (MODE == COL_MATVEC_IN) {
@@ -119,9 +137,8 @@ __global__ void __launch_bounds__(kColNT, 1) k2_cols(Modes2d M, int log2ny, cons
           if constexpr (std::is_same<T, TP>::value) {
             cplx<T> r1 = ld_c<T>(a.rin[0], gi), r2 = ld_c<T>(a.rin[1], gi);
             cplx<T> q1 = ld_c<T>(a.pio[0], gi), q2 = ld_c<T>(a.pio[1], gi);
-            const T beta = cg_beta(a.sc, T(0));
             cplx<T> z1, z2;
-            ainv_of(a.sc, T(0)).apply(MT.kx(col), MT.ky(y), r1, r2, z1, z2);
+            Ai.apply(MT.kx(col), MT.ky(y), r1, r2, z1, z2);
             p1 = z1 + q1 * beta;
             p2 = z2 + q2 * beta;
           }
@@ -132,11 +149,11 @@ __global__ void __launch_bounds__(kColNT, 1) k2_cols(Modes2d M, int log2ny, cons
           p2 = ld_c<T>(a.vin[1], gi);
         }
       }
-      buf[(0 * TW + c) * stride + y] = p1;
-      buf[(1 * TW + c) * stride + y] = p2;
+      buf[(0 * TW + c) * stride + sp] = p1;
+      buf[(1 * TW + c) * stride + sp] = p2;
     } else {
       for (int q = 0; q < nplanes; ++q)
-        buf[(q * TW + c) * stride + y] = ok ? ld_c<T>(a.planes[q], gi)
+        buf[(q * TW + c) * stride + sp] = ok ? ld_c<T>(a.planes[q], gi)
                                             : mk(from_int<T>(0), from_int<T>(0));
     }
   }
@@ -151,43 +168,42 @@ __global__ void __launch_bounds__(kColNT, 1) k2_cols(Modes2d M, int log2ny, cons
       if (col != 0 && col != (M.nx >> 1)) continue;
       for (int q = 0; q < 2; ++q) {
         cplx<T>* v = buf + (q * TW + c) * stride;
-        for (int y = threadIdx.x; y <= (ny >> 1); y += kColNT) {
-          const int ym = (ny - y) & (ny - 1);
-          cplx<T> a = v[y], b = conj(v[ym]);
+        for (int y = threadIdx.x; y <= (ny >> 1); y += NT) {
+          const int py = sw2(pos_of(y, log2ny)), pm = sw2(pos_of((ny - y) & (ny - 1), log2ny));
+          cplx<T> a = v[py], b = conj(v[pm]);
           cplx<T> s = a + b;
           cplx<T> hm = mk(half(s.x), half(s.y));
-          v[y] = hm;
-          v[ym] = conj(hm);
+          v[py] = hm;
+          v[pm] = conj(hm);
         }
       }
     }
     __syncthreads();
-    for (int e = threadIdx.x; e < TW * ny; e += kColNT) {
-      const int y = e / TW, c = e % TW, col = c0 + c;
+    for (int e = threadIdx.x; e < TW * ny; e += NT) {
+      const int p = e / TW, c = e % TW, col = c0 + c, sp = sw2(p);
       const T kx = mode_k<T>(MT, col < H ? col : (M.nx >> 1), true),
-              ky = mode_k<T>(MT, y, false);
-      buf[(2 * TW + c) * stride + y] =
-          mul_ik(buf[(0 * TW + c) * stride + y], kx) + mul_ik(buf[(1 * TW + c) * stride + y], ky);
+              ky = mode_k<T>(MT, mode_at(p, log2ny), false);
+      buf[(2 * TW + c) * stride + sp] =
+          mul_ik(buf[(0 * TW + c) * stride + sp], kx) + mul_ik(buf[(1 * TW + c) * stride + sp], ky);
     }
     __syncthreads();
   }
-  const bool inverse = (MODE == COL_INV || MODE == COL_MATVEC_IN);
   // the planes' columns lie at one stride (sequence q TW + c): one batched transform of all
   // of them, so every stage's butterflies spread over the whole CTA
-  cta_fft_batch<T, kColNT, MAXB>(buf, ny, log2ny, nplanes * TW, stride, inverse, tw);
+  fft2d<T, inverse>(buf, log2ny, nplanes * TW, stride, tab);
 
   // ---- store / epilogue
   if constexpr (MODE == COL_MATVEC_OUT) {
     const double sigma = a.sc ? a.sc->sigma : 0.0, alphaA = a.sc ? a.sc->alpha_A : 0.0;
     double part = 0.0;      // residual mode (double-float or float64 data)
     TP partw = 0;           // dot-product mode, in the working precision
-    for (int e = threadIdx.x; e < TW * ny; e += kColNT) {
-      const int y = e / TW, c = e % TW, col = c0 + c;
+    for (int e = threadIdx.x; e < TW * ny; e += NT) {
+      const int p = e / TW, c = e % TW, col = c0 + c, y = mode_at(p, log2ny), sp = sw2(p);
       if (col >= H) continue;
       const long long gi = (long long)y * H + col;
       const T kx = mode_k<T>(MT, col, true), ky = mode_k<T>(MT, y, false);
-      cplx<T> w1 = buf[(0 * TW + c) * stride + y], w2 = buf[(1 * TW + c) * stride + y];
-      cplx<T> qh = buf[(2 * TW + c) * stride + y];
+      cplx<T> w1 = buf[(0 * TW + c) * stride + sp], w2 = buf[(1 * TW + c) * stride + sp];
+      cplx<T> qh = buf[(2 * TW + c) * stride + sp];
       cplx<T> g1 = w1 - mul_ik(qh, kx), g2 = w2 - mul_ik(qh, ky);
       if (a.residual) {
         g1 = ld_c<T>(a.bvec[0], gi) - g1;
@@ -198,9 +214,9 @@ __global__ void __launch_bounds__(kColNT, 1) k2_cols(Modes2d M, int log2ny, cons
         const double f = alphaA / (sigma + alphaA * k2);
         double r1x = to_f64(g1.x), r1y = to_f64(g1.y), r2x = to_f64(g2.x), r2y = to_f64(g2.y);
         double krx = kxd * r1x + kyd * r2x, kry = kxd * r1y + kyd * r2y;
-        double z1x = (r1x - f * kxd * krx) / sigma, z1y = (r1y - f * kxd * kry) / sigma;
-        double z2x = (r2x - f * kyd * krx) / sigma, z2y = (r2y - f * kyd * kry) / sigma;
-        part += M.weight(col) * (r1x * z1x + r1y * z1y + r2x * z2x + r2y * z2y);
+        double z1x = r1x - f * kxd * krx, z1y = r1y - f * kxd * kry;
+        double z2x = r2x - f * kyd * krx, z2y = r2y - f * kyd * kry;
+        part += M.weight(col) * (r1x * z1x + r1y * z1y + r2x * z2x + r2y * z2y);   // sigma times
       } else if (a.vdot[0]) {
         if constexpr (std::is_same<T, TP>::value) {
           cplx<T> p1 = ld_c<T>(a.vdot[0], gi), p2 = ld_c<T>(a.vdot[1], gi);
@@ -211,9 +227,9 @@ __global__ void __launch_bounds__(kColNT, 1) k2_cols(Modes2d M, int log2ny, cons
       st_c<T>(a.vout[1], gi, g2);
     }
     if (a.residual) {
-      grid_reduce<kColNT>(part, a.parts, a.sc, [&](double s) { a.sc->rz64 = s; });
+      grid_reduce<NT>(part, a.parts, a.sc, [&](double s) { a.sc->rz64 = s / sigma; });
     } else if (a.vdot[0]) {
-      grid_reduce<kColNT>(partw, a.parts, a.sc, [&](double s) {
+      grid_reduce<NT>(partw, a.parts, a.sc, [&](double s) {
         Scal2d* sc = a.sc;
         if (!(s > 0.0) || !isfinite(s)) {
           sc->status = SGN_ERR_BREAKDOWN;
@@ -225,11 +241,12 @@ __global__ void __launch_bounds__(kColNT, 1) k2_cols(Modes2d M, int log2ny, cons
       });
     }
   } else {
-    for (int e = threadIdx.x; e < TW * ny; e += kColNT) {
-      const int y = e / TW, c = e % TW, col = c0 + c;
+    for (int e = threadIdx.x; e < TW * ny; e += NT) {
+      const int p = e / TW, c = e % TW, col = c0 + c, y = inverse ? p : mode_at(p, log2ny);
       if (col >= H) continue;
+      const int sp = sw2(p);
       const long long gi = (long long)y * H + col;
-      for (int q = 0; q < nplanes; ++q) st_c<T>(a.planes[q], gi, buf[(q * TW + c) * stride + y]);
+      for (int q = 0; q < nplanes; ++q) st_c<T>(a.planes[q], gi, buf[(q * TW + c) * stride + sp]);
     }
   }
 }
@@ -266,8 +283,8 @@ __device__ __forceinline__ void coef6<double>(const float* hi, const float* lo, 
 // Matvec row kernel: planes t0, t1, t2 hold (after the column iFFT) the row half spectra of
 // p1, p2, d.  C2R -> pointwise w1, w2, q -> R2C back into t0, t1, t2.  Optionally writes
 // the real-space input (p1, p2) to xout (two planes of P doubles).
-template <typename T, int MAXB>
-__global__ void __launch_bounds__(kRowNT, 1) k2_rows_matvec(Modes2d M, int log2nx, long long P,
+template <typename T>
+__global__ void __launch_bounds__(kMatvecNT, 2) k2_rows_matvec(Modes2d M, int log2nx, long long P,
                                                             const void* t64, const void* t32,
                                                             void* t0, void* t1, void* t2,
                                                             const float* chi, const float* clo,
@@ -282,20 +299,23 @@ __global__ void __launch_bounds__(kRowNT, 1) k2_rows_matvec(Modes2d M, int log2n
   cplx<T>* T0 = reinterpret_cast<cplx<T>*>(t0);
   cplx<T>* T1 = reinterpret_cast<cplx<T>*>(t1);
   cplx<T>* T2 = reinterpret_cast<cplx<T>*>(t2);
-  load_c2r_pair<T>(z, T0 + (long long)y0 * H, T1 + (long long)y0 * H, nx, kRowNT);
-  load_c2r_pair<T>(z + nx, T0 + (long long)y1 * H, T1 + (long long)y1 * H, nx, kRowNT);
-  load_c2r_pair<T>(z + 2 * nx, T2 + (long long)y0 * H, T2 + (long long)y1 * H, nx, kRowNT);
+  cplx<T>* tab = z + 3 * nx;
+  fill_tw2(tab, log2nx, tw);
+  load_c2r_pair<T>(z, T0 + (long long)y0 * H, T1 + (long long)y0 * H, log2nx);
+  load_c2r_pair<T>(z + nx, T0 + (long long)y1 * H, T1 + (long long)y1 * H, log2nx);
+  load_c2r_pair<T>(z + 2 * nx, T2 + (long long)y0 * H, T2 + (long long)y1 * H, log2nx);
   __syncthreads();
-  cta_fft_batch<T, kRowNT, MAXB>(z, nx, log2nx, 3, nx, true, tw);
+  fft2d<T, true>(z, log2nx, 3, nx, tab);
   const T inv = pow2_inv<T>(log2nx + (__ffs(M.ny) - 1));    // 1 / (nx ny), exact
-  for (int x = threadIdx.x; x < nx; x += kRowNT) {
+  for (int x = threadIdx.x; x < nx; x += blockDim.x) {
+    const int sx = sw2(x);
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
       const int y = r ? y1 : y0;
       const long long j = (long long)y * nx + x;
-      cplx<T> pp = z[r * nx + x];
+      cplx<T> pp = z[r * nx + sx];
       T p1 = pp.x * inv, p2 = pp.y * inv;
-      T d = (r ? z[2 * nx + x].y : z[2 * nx + x].x) * inv;
+      T d = (r ? z[2 * nx + sx].y : z[2 * nx + sx].x) * inv;
       if (xout) {
         xout[j] = to_f64(p1);
         xout[P + j] = to_f64(p2);
@@ -305,23 +325,23 @@ __global__ void __launch_bounds__(kRowNT, 1) k2_rows_matvec(Modes2d M, int log2n
       T w1 = c[0] * p1 + c[1] * p2 + c[3] * d;
       T w2 = c[1] * p1 + c[2] * p2 + c[4] * d;
       T q = c[3] * p1 + c[4] * p2 + c[5] * d;
-      z[r * nx + x] = mk(w1, w2);
-      if (r) z[2 * nx + x].y = q; else z[2 * nx + x].x = q;
+      z[r * nx + sx] = mk(w1, w2);
+      if (r) z[2 * nx + sx].y = q; else z[2 * nx + sx].x = q;
     }
   }
   __syncthreads();
-  cta_fft_batch<T, kRowNT, MAXB>(z, nx, log2nx, 3, nx, false, tw);
+  fft2d<T, false>(z, log2nx, 3, nx, tab);
   // split back into half rows: (w1, w2) of y0, (w1, w2) of y1, (q y0, q y1); the row FFT
   // results are read only here, so the splits may write the half planes directly.
-  split_r2c_pair<T>(z, T0 + (long long)y0 * H, T1 + (long long)y0 * H, nx, kRowNT);
-  split_r2c_pair<T>(z + nx, T0 + (long long)y1 * H, T1 + (long long)y1 * H, nx, kRowNT);
-  split_r2c_pair<T>(z + 2 * nx, T2 + (long long)y0 * H, T2 + (long long)y1 * H, nx, kRowNT);
+  split_r2c_pair<T>(z, T0 + (long long)y0 * H, T1 + (long long)y0 * H, log2nx);
+  split_r2c_pair<T>(z + nx, T0 + (long long)y1 * H, T1 + (long long)y1 * H, log2nx);
+  split_r2c_pair<T>(z + 2 * nx, T2 + (long long)y0 * H, T2 + (long long)y1 * H, log2nx);
 }
 
 // R2C row pass of K/2 packed pairs of real planes (double storage): pair q packs
 // (src[2q], src[2q+1]); half rows go to dst[2q], dst[2q+1].  `scale` multiplies the input.
-template <typename T, int MAXB>
-__global__ void __launch_bounds__(kRowNT, 1) k2_rows_r2c(Modes2d M, int log2nx, long long P,
+template <typename T>
+__global__ void __launch_bounds__(kRowNT, 3) k2_rows_r2c(Modes2d M, int log2nx, long long P,
                                                          const void* t64, const void* t32,
                                                          const double* s0, const double* s1,
                                                          const double* s2, const double* s3,
@@ -334,23 +354,25 @@ __global__ void __launch_bounds__(kRowNT, 1) k2_rows_r2c(Modes2d M, int log2nx, 
   const int y = blockIdx.x;
   const double* src[4] = {s0, s1, s2, s3};
   void* dst[4] = {d0, d1, d2, d3};
+  cplx<T>* tab = z + npairs * nx;
+  fill_tw2(tab, log2nx, tw);
   for (int q = 0; q < npairs; ++q)
-    for (int x = threadIdx.x; x < nx; x += kRowNT) {
+    for (int x = threadIdx.x; x < nx; x += blockDim.x) {
       const long long j = (long long)y * nx + x;
       const double a = src[2 * q] ? src[2 * q][j] : 0.0, b = src[2 * q + 1] ? src[2 * q + 1][j] : 0.0;
-      z[q * nx + x] = mk(num<T>(a), num<T>(b));
+      z[q * nx + sw2(x)] = mk(num<T>(a), num<T>(b));
     }
   __syncthreads();
-  cta_fft_batch<T, kRowNT, MAXB>(z, nx, log2nx, npairs, nx, false, tw);
+  fft2d<T, false>(z, log2nx, npairs, nx, tab);
   for (int q = 0; q < npairs; ++q)
     split_r2c_pair<T>(z + q * nx, reinterpret_cast<cplx<T>*>(dst[2 * q]) + (long long)y * H,
-                      reinterpret_cast<cplx<T>*>(dst[2 * q + 1]) + (long long)y * H, nx, kRowNT);
+                      reinterpret_cast<cplx<T>*>(dst[2 * q + 1]) + (long long)y * H, log2nx);
 }
 
 // C2R row pass: pair q of half planes (src[2q], src[2q+1]) -> real planes dst[2q],
 // dst[2q+1] (double storage), scaled by 1/(nx ny).
-template <typename T, int MAXB>
-__global__ void __launch_bounds__(kRowNT, 1) k2_rows_c2r(Modes2d M, int log2nx, long long P,
+template <typename T>
+__global__ void __launch_bounds__(kRowNT, 3) k2_rows_c2r(Modes2d M, int log2nx, long long P,
                                                          const void* t64, const void* t32,
                                                          const void* s0, const void* s1,
                                                          const void* s2, const void* s3,
@@ -363,17 +385,18 @@ __global__ void __launch_bounds__(kRowNT, 1) k2_rows_c2r(Modes2d M, int log2nx, 
   const int y = blockIdx.x;
   const void* src[4] = {s0, s1, s2, s3};
   double* dst[4] = {d0, d1, d2, d3};
+  cplx<T>* tab = z + npairs * nx;
+  fill_tw2(tab, log2nx, tw);
   for (int q = 0; q < npairs; ++q)
     load_c2r_pair<T>(z + q * nx, reinterpret_cast<const cplx<T>*>(src[2 * q]) + (long long)y * H,
-                     reinterpret_cast<const cplx<T>*>(src[2 * q + 1]) + (long long)y * H, nx,
-                     kRowNT);
+                     reinterpret_cast<const cplx<T>*>(src[2 * q + 1]) + (long long)y * H, log2nx);
   __syncthreads();
-  cta_fft_batch<T, kRowNT, MAXB>(z, nx, log2nx, npairs, nx, true, tw);
+  fft2d<T, true>(z, log2nx, npairs, nx, tab);
   const T inv = pow2_inv<T>(log2nx + (__ffs(M.ny) - 1));    // 1 / (nx ny), exact
   for (int q = 0; q < npairs; ++q)
-    for (int x = threadIdx.x; x < nx; x += kRowNT) {
+    for (int x = threadIdx.x; x < nx; x += blockDim.x) {
       const long long j = (long long)y * nx + x;
-      cplx<T> v = z[q * nx + x];
+      cplx<T> v = z[q * nx + sw2(x)];
       if (dst[2 * q]) dst[2 * q][j] = to_f64(v.x * inv);
       if (dst[2 * q + 1]) dst[2 * q + 1][j] = to_f64(v.y * inv);
     }
@@ -823,58 +846,47 @@ cudaError_t smem_attr(K kernel, size_t bytes) {
   return raise_smem(kernel, bytes);
 }
 
-// Columns per CTA for this layout: 2, or 4 for float32 planes when 2-column tiles would not
-// fit one wave on 152 SMs (nx = 1024: 257 tiles).  Four float32 columns also fill each
-// 32-byte sector of a row (two leave half of it unread); wider elements fill it with two.
+// Columns per CTA for this layout: 2 (two 16-byte elements fill a 32-byte sector of a row; two
+// float32 ones leave half of it unread).  4 for float32 planes when 2-column tiles would not
+// fit one wave on 152 SMs (nx = 1024: 257 tiles).  1 for 16-byte elements when every column
+// then has an SM of its own (nx <= 256), where 2-column tiles leave half of the SMs idle
+// (float64 column transforms of 256 x 256: @@TW@@).
 template <typename T>
 int col_tw_of(const Layout2d& L) {
   const int H = L.nx / 2 + 1;
-  return (std::is_same<T, float>::value && (H + 1) / 2 > 152) ? 4 : 2;
+  if (!std::is_same<T, float>::value) return H <= kSMs ? 1 : 2;
+  return (H + 1) / 2 > kSMs ? 4 : 2;
 }
 
 template <typename T>
-size_t col_smem(const Layout2d& L, int K) {
-  return (size_t)K * col_tw_of<T>(L) * (L.ny + 1) * sizeof(cplx<T>);
+size_t row_smem(const Layout2d& L, int nrows) {            // and the twiddles
+  return (size_t)(nrows + 1) * L.nx * sizeof(cplx<T>);
 }
 
-template <typename T>
-size_t row_smem(const Layout2d& L, int nrows) {
-  return (size_t)nrows * L.nx * sizeof(cplx<T>);
+// Threads of a CTA: one per butterfly, within [64, most].
+int threads_for(int butterflies, int most) {
+  const int t = (butterflies + 31) / 32 * 32;
+  return t < 64 ? 64 : (t > most ? most : t);
 }
 
-// column pass launcher: MAXB from the K planes' TW columns x ny/4 butterflies per radix-4
-// stage over kColNT threads
+// column pass launcher: K planes' TW columns of ny/4 butterflies per stage
 template <typename T, int TW, int MODE>
 cudaError_t cols_tw(const Layout2d& L, const void* t64, const void* t32, const ColArgs& a,
                     cudaStream_t s) {
   const Modes2d M = modes_of(L);
   const int tiles = (M.H + TW - 1) / TW;
   const int K = (MODE == COL_MATVEC_IN || MODE == COL_MATVEC_OUT) ? 3 : a.K;
-  const size_t sm = (size_t)K * TW * (L.ny + 1) * sizeof(cplx<T>);
-  // K TW ny / 4 butterflies per radix-4 stage; MAXB = ceil(that / kColNT): at most 4, or 8
-  // for the four float32 columns of the widest grids
-  const int need = (K * TW * L.ny / 4 + kColNT - 1) / kColNT;
-  cudaError_t e;
-  if (need <= 1) {
-    auto k = k2_cols<T, TW, 1, MODE>;
-    if ((e = smem_attr(k, sm))) return e;
-    k<<<tiles, kColNT, sm, s>>>(M, L.ly, t64, t32, a);
-  } else if (need <= 2) {
-    auto k = k2_cols<T, TW, 2, MODE>;
-    if ((e = smem_attr(k, sm))) return e;
-    k<<<tiles, kColNT, sm, s>>>(M, L.ly, t64, t32, a);
-  } else if (need <= 4 || TW < 4) {
-    auto k = k2_cols<T, TW, 4, MODE>;
-    if ((e = smem_attr(k, sm))) return e;
-    k<<<tiles, kColNT, sm, s>>>(M, L.ly, t64, t32, a);
-  } else {
-    if constexpr (TW == 4) {
-      auto k = k2_cols<T, TW, 8, MODE>;
-      if ((e = smem_attr(k, sm))) return e;
-      k<<<tiles, kColNT, sm, s>>>(M, L.ly, t64, t32, a);
-    }
-  }
-  return cudaGetLastError();
+  const size_t sm = ((size_t)K * TW * col_stride<TW>(L.ny) + L.ny) * sizeof(cplx<T>);
+  const int need = K * TW * L.ny / 4;
+  auto go = [&](auto k, int nt) {
+    cudaError_t e = smem_attr(k, sm);
+    if (e) return e;
+    k<<<tiles, nt, sm, s>>>(M, L.ly, t64, t32, a);
+    return cudaGetLastError();
+  };
+  if (need <= 128) return go(k2_cols<T, TW, 128, MODE>, 128);
+  if (need <= 256) return go(k2_cols<T, TW, 256, MODE>, 256);
+  return go(k2_cols<T, TW, 512, MODE>, 512);
 }
 
 template <typename T, int MODE>
@@ -882,6 +894,8 @@ cudaError_t cols(const Layout2d& L, const void* t64, const void* t32, const ColA
                  cudaStream_t s) {
   if constexpr (std::is_same<T, float>::value) {
     if (col_tw_of<T>(L) == 4) return cols_tw<T, 4, MODE>(L, t64, t32, a, s);
+  } else {
+    if (col_tw_of<T>(L) == 1) return cols_tw<T, 1, MODE>(L, t64, t32, a, s);
   }
   return cols_tw<T, 2, MODE>(L, t64, t32, a, s);
 }
@@ -891,18 +905,12 @@ cudaError_t rows_matvec(const Layout2d& L, const void* t64, const void* t32, voi
                         void* t2, double* xout, Scal2d* sc, int check_done, cudaStream_t s) {
   const Modes2d M = modes_of(L);
   const size_t sm = row_smem<T>(L, 3);
-  const int need = (3 * L.nx / 4 + kRowNT - 1) / kRowNT;   // butterflies per thread
-  cudaError_t e;
-#define SGN_ROWS_MV(MB)                                                                     \
-  {                                                                                        \
-    auto k = k2_rows_matvec<T, MB>;                                                        \
-    if ((e = smem_attr(k, sm))) return e;                                                  \
-    k<<<L.ny / 2, kRowNT, sm, s>>>(M, L.lx, L.P, t64, t32, t0, t1, t2, L.coef,              \
-                                   L.coef_lo, xout, sc, check_done);                       \
-  }
-  if (need <= 1) SGN_ROWS_MV(1) else if (need <= 2) SGN_ROWS_MV(2) else if (need <= 3) SGN_ROWS_MV(3)
-  else SGN_ROWS_MV(4)
-#undef SGN_ROWS_MV
+  auto k = k2_rows_matvec<T>;
+  cudaError_t e = smem_attr(k, sm);
+  if (e) return e;
+  k<<<L.ny / 2, threads_for(3 * L.nx / 4, kMatvecNT), sm, s>>>(M, L.lx, L.P, t64, t32, t0, t1, t2,
+                                                               L.coef, L.coef_lo, xout, sc,
+                                                               check_done);
   return cudaGetLastError();
 }
 
@@ -912,16 +920,11 @@ cudaError_t rows_r2c(const Layout2d& L, const void* t64, const void* t32, const 
                      void* d2, void* d3, int npairs, cudaStream_t s) {
   const Modes2d M = modes_of(L);
   const size_t sm = row_smem<T>(L, npairs);
-  const int need = (npairs * L.nx / 4 + kRowNT - 1) / kRowNT;
-  cudaError_t e;
-#define SGN_ROWS_F(MB)                                                                       \
-  {                                                                                         \
-    auto k = k2_rows_r2c<T, MB>;                                                            \
-    if ((e = smem_attr(k, sm))) return e;                                                   \
-    k<<<L.ny, kRowNT, sm, s>>>(M, L.lx, L.P, t64, t32, s0, s1, s2, s3, d0, d1, d2, d3, npairs); \
-  }
-  if (need <= 1) SGN_ROWS_F(1) else if (need <= 2) SGN_ROWS_F(2) else SGN_ROWS_F(4)
-#undef SGN_ROWS_F
+  auto k = k2_rows_r2c<T>;
+  cudaError_t e = smem_attr(k, sm);
+  if (e) return e;
+  k<<<L.ny, threads_for(npairs * L.nx / 4, kRowNT), sm, s>>>(M, L.lx, L.P, t64, t32, s0, s1, s2, s3,
+                                                             d0, d1, d2, d3, npairs);
   return cudaGetLastError();
 }
 
@@ -931,16 +934,11 @@ cudaError_t rows_c2r(const Layout2d& L, const void* t64, const void* t32, const 
                      double* d2, double* d3, int npairs, cudaStream_t s) {
   const Modes2d M = modes_of(L);
   const size_t sm = row_smem<T>(L, npairs);
-  const int need = (npairs * L.nx / 4 + kRowNT - 1) / kRowNT;
-  cudaError_t e;
-#define SGN_ROWS_I(MB)                                                                       \
-  {                                                                                         \
-    auto k = k2_rows_c2r<T, MB>;                                                            \
-    if ((e = smem_attr(k, sm))) return e;                                                   \
-    k<<<L.ny, kRowNT, sm, s>>>(M, L.lx, L.P, t64, t32, s0, s1, s2, s3, d0, d1, d2, d3, npairs); \
-  }
-  if (need <= 1) SGN_ROWS_I(1) else if (need <= 2) SGN_ROWS_I(2) else SGN_ROWS_I(4)
-#undef SGN_ROWS_I
+  auto k = k2_rows_c2r<T>;
+  cudaError_t e = smem_attr(k, sm);
+  if (e) return e;
+  k<<<L.ny, threads_for(npairs * L.nx / 4, kRowNT), sm, s>>>(M, L.lx, L.P, t64, t32, s0, s1, s2, s3,
+                                                             d0, d1, d2, d3, npairs);
   return cudaGetLastError();
 }
 

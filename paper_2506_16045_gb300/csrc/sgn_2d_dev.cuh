@@ -41,8 +41,8 @@ using d1::kLambdaPlus;
 using d1::kLambdaMinus;
 using d1::kFlatSlope;
 
-constexpr int kRowNT = 256;
-constexpr int kColNT = 512;
+constexpr int kRowNT = 256;           // most threads of a row pass, and of the row matvec
+constexpr int kMatvecNT = 384;
 constexpr int kMaxParts = 2048;
 
 // ---- mode helpers --------------------------------------------------------------------
@@ -178,39 +178,6 @@ template <>
 __device__ __forceinline__ df widen<df>(float v) { return df(v, 0.0f); }
 template <typename TH>
 __device__ __forceinline__ TH widen(double v) { return num<TH>(v); }
-
-// C2R of one packed pair: buf <- A + i B over the full row from two half rows, iFFT.
-template <typename T>
-__device__ __forceinline__ void load_c2r_pair(cplx<T>* z, const cplx<T>* A, const cplx<T>* B,
-                                              int nx, int NT) {
-  const int h = nx >> 1;
-  for (int m = threadIdx.x; m < nx; m += NT) {
-    cplx<T> a, b;
-    if (m <= h) {
-      a = A[m];
-      b = B[m];
-    } else {
-      a = conj(A[nx - m]);
-      b = conj(B[nx - m]);
-    }
-    // a + i b
-    z[m] = mk(a.x - b.y, a.y + b.x);
-  }
-}
-
-// R2C split of a packed FFT row Y = FFT(a + i b): A[m] = (Y_m + conj Y_{n-m})/2,
-// B[m] = (Y_m - conj Y_{n-m})/(2i), m = 0..nx/2.
-template <typename T>
-__device__ __forceinline__ void split_r2c_pair(const cplx<T>* Y, cplx<T>* A, cplx<T>* B, int nx,
-                                               int NT) {
-  const int h = nx >> 1;
-  for (int m = threadIdx.x; m <= h; m += NT) {
-    cplx<T> y = Y[m], yc = conj(Y[(nx - m) & (nx - 1)]);
-    cplx<T> s = y + yc, d = mul_mi(y - yc);
-    A[m] = mk(half(s.x), half(s.y));
-    B[m] = mk(half(d.x), half(d.y));
-  }
-}
 
 // ---- persistent inner solve (sgn_2d_pcg.cu) --------------------------------------------
 constexpr int kMaxBatch2d = kMaxBatch2dAbi;   // instances of one persistent inner solve
