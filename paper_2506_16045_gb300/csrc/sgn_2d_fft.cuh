@@ -7,9 +7,10 @@
 //
 // The passes are bound by latency (a stage is a shared load, a chain of dependent double-float
 // or float64 operations, a shared store and a barrier), then by the float64 pipe.  Against
-// Stockham stages with two barriers each, twiddles gathered from a table in global memory and
-// one thread per butterfly of a fixed block, at 512 x 512 (double-float, one GB300): two rows
-// passes 19.4 and 15.5 us, a column pass 20.0 us before; @@AFTER@@.
+// Stockham stages with two barriers each and twiddles gathered from a table in global memory,
+// double-float at 512 x 512 (one GB300): a column pass over two planes 20.0 -> 14.8 us, a row
+// pass over one pair 15.5 -> 12.7 us; 256 x 256 in float64, 2 RK4 steps: 14.1 -> 11.6 ms;
+// 512 x 512 mixed, 4 RK4 steps: 16.3 -> 15.1 ms.
 #pragma once
 #include "sgn_2d_dev.cuh"
 
