@@ -95,10 +95,6 @@ struct ColArgs {
   int check_done;           // return immediately when sc->done
 };
 
-// Stride of the columns in shared memory: of two columns the second is four 16-byte banks off.
-template <int TW>
-__host__ __device__ constexpr int col_stride(int ny) { return TW == 1 ? ny : ny + 4; }
-
 template <typename T, int TW, int NT, int MODE>
 __global__ void __launch_bounds__(NT, NT < 512 ? 2 : 1) k2_cols(Modes2d M, int log2ny, const void* t64,
                                                      const void* t32, ColArgs a) {
@@ -406,67 +402,23 @@ __global__ void __launch_bounds__(kRowNT, 3) k2_rows_c2r(Modes2d M, int log2nx, 
 // Per-mode kernels over half spectra
 // =======================================================================================
 
-// Spectral ops for derivatives and A^{-1}:
-//   OP_GRAD: out0 = i kx in0, out1 = i ky in0 (and out2, out3 from in1)
-//   OP_AINV: (out0, out1) = A^{-1} (in0, in1)
-//   OP_DIV : out0 = i kx in0 + i ky in1
-enum SpecOp { OP_GRAD = 0, OP_AINV = 1 };
-
-template <typename T, int OP>
-__global__ void k2_spec(Modes2d M, const void* in0, const void* in1, void* out0, void* out1,
-                        void* out2, void* out3, const Scal2d* sc, const SolveRec* A) {
+// (out0, out1) = A^{-1} (in0, in1)
+template <typename T>
+__global__ void k2_ainv(Modes2d M, const void* in0, const void* in1, void* out0, void* out1,
+                        const Scal2d* sc, const SolveRec* A) {
   const long long HP = (long long)M.ny * M.H;
+  const double sigma = A ? A->sigma : sc->sigma, alpha = A ? A->alpha : sc->alpha_A;
+  const T is = num<T>(1.0 / sigma);
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < HP;
        i += (long long)gridDim.x * blockDim.x) {
     const int y = (int)i / M.H, c = (int)i - y * M.H;   // half planes < 2^31 elements
     const double kx = M.kx(c), ky = M.ky(y);
-    if constexpr (OP == OP_GRAD) {
-      cplx<T> a = ld_c<T>(in0, i);
-      st_c<T>(out0, i, mul_ik(a, num<T>(kx)));
-      st_c<T>(out1, i, mul_ik(a, num<T>(ky)));
-      if (in1) {
-        cplx<T> b = ld_c<T>(in1, i);
-        st_c<T>(out2, i, mul_ik(b, num<T>(kx)));
-        st_c<T>(out3, i, mul_ik(b, num<T>(ky)));
-      }
-    } else {
-      const double sigma = A ? A->sigma : sc->sigma, alpha = A ? A->alpha : sc->alpha_A;
-      const double f = alpha / (sigma + alpha * (kx * kx + ky * ky));
-      const T kxT = num<T>(kx), kyT = num<T>(ky), fT = num<T>(f), is = num<T>(1.0 / sigma);
-      cplx<T> r1 = ld_c<T>(in0, i), r2 = ld_c<T>(in1, i);
-      cplx<T> kr = r1 * kxT + r2 * kyT;
-      st_c<T>(out0, i, (r1 - kr * (fT * kxT)) * is);
-      st_c<T>(out1, i, (r2 - kr * (fT * kyT)) * is);
-    }
-  }
-}
-
-// Spectral combinations of the 2d right-hand side (i k multiplies by the wavenumber, the
-// Nyquist wavenumbers being 0):
-//   RHS_DIVD: out0 = d^ = i kx in0 + i ky in1 (d = div u), out1 = i kx in2 + i ky in3
-//             (m = div(eta u)), out2 = i kx d^, out3 = i ky d^ (grad d);
-//   RHS_DIV2: out0 = i kx in0 + i ky in1, out1 = i kx in1 + i ky in2 (the two components of
-//             div(eta u (x) u) from eta u u, eta u v, eta v v).
-enum RhsSpec { RHS_DIVD = 0, RHS_DIV2 = 1 };
-template <typename T, int MODE>
-__global__ void k2_spec_rhs(Modes2d M, const void* in0, const void* in1, const void* in2,
-                            const void* in3, void* out0, void* out1, void* out2, void* out3) {
-  const long long HP = (long long)M.ny * M.H;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < HP;
-       i += (long long)gridDim.x * blockDim.x) {
-    const int y = (int)i / M.H, c = (int)i - y * M.H;   // half planes < 2^31 elements
-    const T kx = num<T>(M.kx(c)), ky = num<T>(M.ky(y));
-    const cplx<T> a = ld_c<T>(in0, i), b = ld_c<T>(in1, i), e = ld_c<T>(in2, i);
-    if constexpr (MODE == RHS_DIVD) {
-      const cplx<T> dh = mul_ik(a, kx) + mul_ik(b, ky);
-      st_c<T>(out0, i, dh);
-      st_c<T>(out1, i, mul_ik(e, kx) + mul_ik(ld_c<T>(in3, i), ky));
-      st_c<T>(out2, i, mul_ik(dh, kx));
-      st_c<T>(out3, i, mul_ik(dh, ky));
-    } else {
-      st_c<T>(out0, i, mul_ik(a, kx) + mul_ik(b, ky));
-      st_c<T>(out1, i, mul_ik(b, kx) + mul_ik(e, ky));
-    }
+    const double f = alpha / (sigma + alpha * (kx * kx + ky * ky));
+    const T kxT = num<T>(kx), kyT = num<T>(ky), fT = num<T>(f);
+    cplx<T> r1 = ld_c<T>(in0, i), r2 = ld_c<T>(in1, i);
+    cplx<T> kr = r1 * kxT + r2 * kyT;
+    st_c<T>(out0, i, (r1 - kr * (fT * kxT)) * is);
+    st_c<T>(out1, i, (r2 - kr * (fT * kyT)) * is);
   }
 }
 
@@ -757,53 +709,6 @@ __global__ void k2_lincomb(long long n, double* out, const double* x0, const dou
     for (int t = 0; t < nx; ++t) acc += A[t] * X[t][i];
     for (int t = 0; t < nf; ++t) accf += Cc[t] * F[t][i];
     out[i] = acc + d * accf;
-  }
-}
-
-// RHS pointwise stages (T arithmetic, double storage), see launch_rhs2d.
-template <typename T>
-__global__ void k2_rhs_stage(int stage, long long P, double g, const double* eta, const double* u,
-                             const double* hgt, const double* gh, double* w, double* f_eta,
-                             double* f_U) {
-  // w: scratch planes [0..]; see launch_rhs2d for the meaning of each index
-  for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < P;
-       j += (long long)gridDim.x * blockDim.x) {
-    const T e = num<T>(eta[j]), uu = num<T>(u[j]), vv = num<T>(u[P + j]);
-    const T hx = num<T>(gh[j]), hy = num<T>(gh[P + j]);
-    if (stage == 0) {
-      // inputs for the first derivative passes
-      w[0 * P + j] = to_f64(e * uu);                       // eta u
-      w[1 * P + j] = to_f64(e * vv);                       // eta v
-      w[2 * P + j] = eta[j] - hgt[j];                      // zeta
-      w[3 * P + j] = to_f64(hx * uu + hy * vv);            // s
-      w[4 * P + j] = to_f64(e * uu * uu);                  // eta u u
-      w[5 * P + j] = to_f64(e * uu * vv);                  // eta u v
-      w[6 * P + j] = to_f64(e * vv * vv);                  // eta v v
-    } else {
-      // 7 d = div u, 14 m = div(eta u), 18 zeta_x, 19 zeta_y, 20 s_x, 21 s_y, 22 d_x, 23 d_y,
-      // 24 and 26 the x and y components of div(eta u (x) u); Phi -> 8, Psi -> 9
-      const T d = num<T>(w[7 * P + j]);
-      const T m = num<T>(w[14 * P + j]);
-      const T s = hx * uu + hy * vv;
-      const T Sv = uu * num<T>(w[20 * P + j]) + vv * num<T>(w[21 * P + j]);
-      const T Q = uu * num<T>(w[22 * P + j]) + vv * num<T>(w[23 * P + j]) - d * d;
-      const T e2 = e * e, md = m * d;
-      if (stage == 2) {
-        w[8 * P + j] = to_f64(e2 * e * Q * num<T>(1.0 / 3.0) + e2 * md + half(e2 * Sv) + e * m * s);
-        w[9 * P + j] = to_f64(half(e2 * Q) + e * md + e * Sv + m * s);
-      } else {
-        // stage 3: Phi_x -> 30, Phi_y -> 31
-        const T Psi = num<T>(w[9 * P + j]);
-        const T gT = num<T>(g);
-        f_eta[j] = -to_f64(m);
-        const T fx = num<T>(w[30 * P + j]) - gT * e * num<T>(w[18 * P + j]) -
-                     num<T>(w[24 * P + j]) - hx * Psi;
-        const T fy = num<T>(w[31 * P + j]) - gT * e * num<T>(w[19 * P + j]) -
-                     num<T>(w[26 * P + j]) - hy * Psi;
-        f_U[j] = to_f64(fx);
-        f_U[P + j] = to_f64(fy);
-      }
-    }
   }
 }
 
@@ -1222,24 +1127,6 @@ size_t layout2d_res_bytes(const Layout2d& L) { return (size_t)16 * 2 * (L.HP > 0
 // Entry points
 // =======================================================================================
 
-cudaError_t launch_grad2d(const Layout2d& L, const void* tw64, const double* f, double* gradf,
-                          cudaStream_t s) {
-  if (L.mr) return mr2d_grad(L, f, gradf, s);
-  // forward transform of f (paired with zero), i k, inverse of both components
-  cudaError_t e = rows_r2c<double>(L, tw64, nullptr, f, nullptr, nullptr, nullptr,
-                                   tplane(L, 0), tplane(L, 3), nullptr, nullptr, 1, s);
-  if (e) return e;
-  ColArgs a{};
-  a.planes[0] = tplane(L, 0);
-  a.K = 1;
-  if ((e = cols<double, COL_FWD>(L, tw64, nullptr, a, s))) return e;
-  const Modes2d M = modes_of(L);
-  k2_spec<double, OP_GRAD><<<grid_for(L.HP, 256), 256, 0, s>>>(
-      M, tplane(L, 0), nullptr, tplane(L, 1), tplane(L, 2), nullptr, nullptr, nullptr, nullptr);
-  if ((e = cudaGetLastError())) return e;
-  return c2r_vec<double>(L, tw64, nullptr, tplane(L, 1), tplane(L, 2), gradf, s);
-}
-
 namespace {
 
 // Orszag's 2/3 rule on half planes: modes with |jx| > nx/3 or |jy| > ny/3 set to zero
@@ -1408,8 +1295,8 @@ cudaError_t launch_precond2d(const Layout2d& L, const void* tw64, const SolveRec
   cudaError_t e = r2c_vec<double>(L, tw64, nullptr, r, slot(L, 0), slot(L, 1), s);
   if (e) return e;
   const Modes2d M = modes_of(L);
-  k2_spec<double, OP_AINV><<<grid_for(L.HP, 256), 256, 0, s>>>(
-      M, slot(L, 0), slot(L, 1), slot(L, 2), slot(L, 3), nullptr, nullptr, nullptr, rec);
+  k2_ainv<double><<<grid_for(L.HP, 256), 256, 0, s>>>(
+      M, slot(L, 0), slot(L, 1), slot(L, 2), slot(L, 3), nullptr, rec);
   if ((e = cudaGetLastError())) return e;
   return c2r_vec<double>(L, tw64, nullptr, slot(L, 2), slot(L, 3), z, s);
 }
@@ -2091,108 +1978,6 @@ cudaError_t launch_pcg2d_batch(Layout2d& first, Batch2d& Bt, const void* tw64, c
   return cudaGetLastError();
 }
 
-namespace {
-
-// Right-hand side (Def:bigF) in four transform passes (see k2_rhs_stage for plane indices):
-// div u, div(eta u) and grad(div u) from one pass of (u, v, eta u, eta v); grad zeta and
-// grad s; the two components of div(eta u (x) u); grad Phi.  Sums of derivatives are formed
-// in spectral space, so only the twelve planes the pointwise stages read are transformed
-// back.  The transforms run in T (float64, or double-float for the mixed path); the
-// pointwise stages and the intermediate planes are float64.
-template <typename T>
-cudaError_t rhs2d(const Layout2d& L, const void* tw64, const void* tw32, double g,
-                  const double* eta, const double* u, const double* h, const double* gradh,
-                  double* f_eta, double* f_U, cudaStream_t s) {
-  double* w = L.rhs_w;
-  const long long P = L.P;
-  auto W = [&](int q) { return w + (long long)q * P; };
-  const int gb = grid_for(P, 256);
-  cudaError_t e;
-  auto grad_pair = [&](const double* a, const double* b, double* ax, double* ay, double* bx,
-                       double* by) -> cudaError_t {
-    cudaError_t r = rows_r2c<T>(L, tw64, tw32, a, b, nullptr, nullptr, tplane(L, 0),
-                                     tplane(L, 1), nullptr, nullptr, 1, s);
-    if (r) return r;
-    ColArgs c{};
-    c.planes[0] = tplane(L, 0);
-    c.planes[1] = tplane(L, 1);
-    c.K = 2;
-    if ((r = cols<T, COL_FWD>(L, tw64, tw32, c, s))) return r;
-    const Modes2d M = modes_of(L);
-    k2_spec<T, OP_GRAD><<<grid_for(L.HP, 256), 256, 0, s>>>(
-        M, tplane(L, 0), tplane(L, 1), slot(L, 0), slot(L, 1), slot(L, 2), slot(L, 3), nullptr,
-        nullptr);
-    if ((r = cudaGetLastError())) return r;
-    ColArgs ci{};
-    ci.planes[0] = slot(L, 0);
-    ci.planes[1] = slot(L, 1);
-    ci.planes[2] = slot(L, 2);
-    ci.planes[3] = slot(L, 3);
-    ci.K = 4;
-    if ((r = cols<T, COL_INV>(L, tw64, tw32, ci, s))) return r;
-    return rows_c2r<T>(L, tw64, tw32, slot(L, 0), slot(L, 1), slot(L, 2), slot(L, 3), ax,
-                            ay, bx, by, 2, s);
-  };
-  // Pass of four real fields through the forward transform, a spectral combination and the
-  // inverse transform of nout planes (written to out[0..nout) as real planes).
-  auto combo = [&](const double* a, const double* b, const double* c, const double* d, int K,
-                   int mode, int nout, double* const* out) -> cudaError_t {
-    cudaError_t r = rows_r2c<T>(L, tw64, tw32, a, b, c, d, tplane(L, 0), tplane(L, 1),
-                                tplane(L, 2), tplane(L, 3), (K + 1) / 2, s);
-    if (r) return r;
-    ColArgs cf{};
-    for (int q = 0; q < 4; ++q) cf.planes[q] = tplane(L, q);
-    cf.K = K;
-    if ((r = cols<T, COL_FWD>(L, tw64, tw32, cf, s))) return r;
-    const Modes2d M = modes_of(L);
-    if (mode == RHS_DIVD)
-      k2_spec_rhs<T, RHS_DIVD><<<grid_for(L.HP, 256), 256, 0, s>>>(
-          M, tplane(L, 0), tplane(L, 1), tplane(L, 2), tplane(L, 3), slot(L, 0), slot(L, 1),
-          slot(L, 2), slot(L, 3));
-    else
-      k2_spec_rhs<T, RHS_DIV2><<<grid_for(L.HP, 256), 256, 0, s>>>(
-          M, tplane(L, 0), tplane(L, 1), tplane(L, 2), nullptr, slot(L, 0), slot(L, 1), nullptr,
-          nullptr);
-    if ((r = cudaGetLastError())) return r;
-    ColArgs ci{};
-    for (int q = 0; q < 4; ++q) ci.planes[q] = slot(L, q);
-    ci.K = nout;
-    if ((r = cols<T, COL_INV>(L, tw64, tw32, ci, s))) return r;
-    return rows_c2r<T>(L, tw64, tw32, slot(L, 0), slot(L, 1), slot(L, 2), slot(L, 3), out[0],
-                       out[1], nout > 2 ? out[2] : nullptr, nout > 2 ? out[3] : nullptr,
-                       nout / 2, s);
-  };
-  k2_rhs_stage<double><<<gb, 256, 0, s>>>(0, P, g, eta, u, h, gradh, w, f_eta, f_U);
-  if ((e = cudaGetLastError())) return e;
-  // d = div u, m = div(eta u), grad d from one pass of (u, v, eta u, eta v)
-  {
-    double* out[4] = {W(7), W(14), W(22), W(23)};
-    if ((e = combo(u, u + P, W(0), W(1), 4, RHS_DIVD, 4, out))) return e;
-  }
-  if ((e = grad_pair(W(2), W(3), W(18), W(19), W(20), W(21)))) return e;   // grad zeta, grad s
-  // div(eta u (x) u) from (eta u u, eta u v, eta v v)
-  {
-    double* out[4] = {W(24), W(26), nullptr, nullptr};
-    if ((e = combo(W(4), W(5), W(6), nullptr, 3, RHS_DIV2, 2, out))) return e;
-  }
-  k2_rhs_stage<double><<<gb, 256, 0, s>>>(2, P, g, eta, u, h, gradh, w, f_eta, f_U);
-  if ((e = cudaGetLastError())) return e;
-  if ((e = grad_pair(W(8), nullptr, W(30), W(31), nullptr, nullptr))) return e;
-  k2_rhs_stage<double><<<gb, 256, 0, s>>>(3, P, g, eta, u, h, gradh, w, f_eta, f_U);
-  return cudaGetLastError();
-}
-
-}  // namespace
-
-cudaError_t launch_rhs2d(const Layout2d& L, const void* tw64, const void* tw32, int precision,
-                         double g, const double* eta, const double* u, const double* h,
-                         const double* gradh, double* f_eta, double* f_U, cudaStream_t s) {
-  if (L.mr) return mr2d_rhs(L, g, eta, u, h, gradh, f_eta, f_U, s);
-  return precision == SGN_PREC_MIXED
-             ? rhs2d<df>(L, tw64, tw32, g, eta, u, h, gradh, f_eta, f_U, s)
-             : rhs2d<double>(L, tw64, tw32, g, eta, u, h, gradh, f_eta, f_U, s);
-}
-
 cudaError_t launch_lincomb2d(const Layout2d& L, const double* dt, double* out,
                              const double* const* x, const double* a, int nx,
                              const double* const* f, const double* c, int nf, int components,
@@ -2249,8 +2034,8 @@ cudaError_t launch_linimp_solve2d(const Layout2d& L, const void* tw64, const Sol
   cudaError_t e = cudaGetLastError();
   if (e) return e;
   const Modes2d M = modes_of(L);
-  k2_spec<double, OP_AINV><<<grid_for(L.HP, 256), 256, 0, s>>>(
-      M, slot(L, 4), slot(L, 5), slot(L, 6), slot(L, 7), nullptr, nullptr, nullptr, A);
+  k2_ainv<double><<<grid_for(L.HP, 256), 256, 0, s>>>(
+      M, slot(L, 4), slot(L, 5), slot(L, 6), slot(L, 7), nullptr, A);
   if ((e = cudaGetLastError())) return e;
   return c2r_vec<double>(L, tw64, nullptr, slot(L, 6), slot(L, 7), u, s);
 }

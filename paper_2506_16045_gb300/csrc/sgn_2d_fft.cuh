@@ -26,6 +26,10 @@ __device__ __forceinline__ int sw2(int a) {
   return a ^ (int)((0x0356217447126530ull >> (4 * u)) & 7);
 }
 
+// Stride of TW columns of ny: the columns lie 8 / TW 16-byte banks apart.
+template <int TW>
+__host__ __device__ constexpr int col_stride(int ny) { return TW == 1 ? ny : ny + 8 / TW; }
+
 // digits of two bits, reversed (bits even)
 __device__ __forceinline__ int dig_rev(int x, int bits) {
   const unsigned r = __brev((unsigned)x) >> (32 - bits);
@@ -54,14 +58,55 @@ __device__ __forceinline__ void fill_tw2(cplx<T>* tab, int l, const cplx<T>* __r
   }
 }
 
+template <typename T, bool INV>
+__device__ __forceinline__ void dft4(cplx<T>& a0, cplx<T>& a1, cplx<T>& a2, cplx<T>& a3) {
+  const cplx<T> s02 = a0 + a2, d02 = a0 - a2, s13 = a1 + a3, d13 = a1 - a3;
+  const cplx<T> r13 = INV ? mul_pi(d13) : mul_mi(d13);
+  a0 = s02 + s13;
+  a1 = d02 + r13;
+  a2 = s02 - s13;
+  a3 = d02 - r13;
+}
+
+// The radix-4 stage of element distance 2^ls, and its barrier.
+template <typename T, bool INV>
+__device__ __forceinline__ void stage4(cplx<T>* buf, int l, int nb, int stride,
+                                       const cplx<T>* tab, int ls) {
+  const int lb = l - 2, sg = 1 << ls;
+  const cplx<T>* w = tab + (1 << l) - 4 * sg;
+  const int d1 = sw2(sg), d2 = sw2(2 * sg);
+#pragma unroll 1
+  for (int g = threadIdx.x; g < (nb << lb); g += blockDim.x) {
+    const int x = g & ((1 << lb) - 1), i = x & (sg - 1);
+    cplx<T>* s = buf + (g >> lb) * stride;
+    const int a = sw2(((x ^ i) << 2) | i);
+    cplx<T> a0 = s[a], a1 = s[a ^ d1], a2 = s[a ^ d2], a3 = s[a ^ d1 ^ d2];
+    if (INV && ls > 0) {
+      a1 = cmul_tw(a1, w[i], true);
+      a2 = cmul_tw(a2, w[sg + i], true);
+      a3 = cmul_tw(a3, w[2 * sg + i], true);
+    }
+    dft4<T, INV>(a0, a1, a2, a3);
+    if (!INV && ls > 0) {
+      a1 = cmul_tw(a1, w[i], false);
+      a2 = cmul_tw(a2, w[sg + i], false);
+      a3 = cmul_tw(a3, w[2 * sg + i], false);
+    }
+    s[a] = a0;
+    s[a ^ d1] = a1;
+    s[a ^ d2] = a2;
+    s[a ^ d1 ^ d2] = a3;
+  }
+  __syncthreads();
+}
+
 // nb sequences of length 2^l, sequence s at buf + s * stride (element a at sw2(a)).  Every thread
 // of the block calls it, after a barrier; it returns after one.
 template <typename T, bool INV>
 __device__ __forceinline__ void fft2d(cplx<T>* buf, int l, int nb, int stride,
                                       const cplx<T>* tab) {
-  const int q = l >> 1, odd = l & 1, lb = l - 2, n = 1 << l;
+  const int q = l >> 1, odd = l & 1, lp = l - 1;
   auto pairs = [&]() {
-    const int lp = l - 1;
 #pragma unroll 1
     for (int g = threadIdx.x; g < (nb << lp); g += blockDim.x) {
       cplx<T>* s = buf + (g >> lp) * stride;
@@ -74,40 +119,55 @@ __device__ __forceinline__ void fft2d(cplx<T>* buf, int l, int nb, int stride,
   };
   if (INV && odd) pairs();
 #pragma unroll 1
-  for (int j = 0; j < q; ++j) {
-    const int ls = INV ? odd + 2 * j : l - 2 - 2 * j, sg = 1 << ls;
-    const cplx<T>* w = tab + n - 4 * sg;
-    const int d1 = sw2(sg), d2 = sw2(2 * sg);
+  for (int j = 0; j < q; ++j)
+    stage4<T, INV>(buf, l, nb, stride, tab, INV ? odd + 2 * j : l - 2 - 2 * j);
+  if (!INV && odd) pairs();
+}
+
+// Derivative along the sequences: forward, times i kn m (m the signed mode, 0 for n/2), inverse;
+// kn = 2 pi / (L n) takes the inverse's normalisation in.  A sequence a + i b of two real
+// fields becomes a' + i b'.  The last forward stage, the product and the first inverse stage
+// touch the same elements and stay in registers.
+template <typename T>
+__device__ __forceinline__ void deriv2d(cplx<T>* buf, int l, int nb, int stride,
+                                        const cplx<T>* tab, T kn) {
+  const int q = l >> 1, odd = l & 1, h = 1 << (l - 1), h2 = h >> 1;
+#pragma unroll 1
+  for (int j = 0; j < q - 1 + odd; ++j) stage4<T, false>(buf, l, nb, stride, tab, l - 2 - 2 * j);
+  auto ik = [&](cplx<T> v, int m) { return mul_ik(v, from_int<T>(m) * kn); };
+  if (odd) {
+    const int lp = l - 1;
+#pragma unroll 1
+    for (int g = threadIdx.x; g < (nb << lp); g += blockDim.x) {
+      cplx<T>* s = buf + (g >> lp) * stride;
+      const int p = (g & ((1 << lp) - 1)) << 1, a = sw2(p), m = mode_at(p, l);
+      const cplx<T> x = s[a], y = s[a ^ 1];
+      const cplx<T> X = ik(x + y, m), Y = ik(x - y, m ? m - h : 0);
+      s[a] = X + Y;
+      s[a ^ 1] = X - Y;
+    }
+  } else {
+    const int lb = l - 2, d1 = sw2(1), d2 = sw2(2);
 #pragma unroll 1
     for (int g = threadIdx.x; g < (nb << lb); g += blockDim.x) {
-      const int x = g & ((1 << lb) - 1), i = x & (sg - 1);
       cplx<T>* s = buf + (g >> lb) * stride;
-      const int a = sw2(((x ^ i) << 2) | i);
+      const int p = (g & ((1 << lb) - 1)) << 2, a = sw2(p), m = mode_at(p, l);
       cplx<T> a0 = s[a], a1 = s[a ^ d1], a2 = s[a ^ d2], a3 = s[a ^ d1 ^ d2];
-      if (INV && ls > 0) {
-        a1 = cmul_tw(a1, w[i], true);
-        a2 = cmul_tw(a2, w[sg + i], true);
-        a3 = cmul_tw(a3, w[2 * sg + i], true);
-      }
-      const cplx<T> s02 = a0 + a2, d02 = a0 - a2, s13 = a1 + a3, d13 = a1 - a3;
-      const cplx<T> r13 = INV ? mul_pi(d13) : mul_mi(d13);
-      a0 = s02 + s13;
-      a1 = d02 + r13;
-      a2 = s02 - s13;
-      a3 = d02 - r13;
-      if (!INV && ls > 0) {
-        a1 = cmul_tw(a1, w[i], false);
-        a2 = cmul_tw(a2, w[sg + i], false);
-        a3 = cmul_tw(a3, w[2 * sg + i], false);
-      }
+      dft4<T, false>(a0, a1, a2, a3);
+      a0 = ik(a0, m);
+      a1 = ik(a1, m + h2);
+      a2 = ik(a2, m ? m - h : 0);
+      a3 = ik(a3, m - h2);
+      dft4<T, true>(a0, a1, a2, a3);
       s[a] = a0;
       s[a ^ d1] = a1;
       s[a ^ d2] = a2;
       s[a ^ d1 ^ d2] = a3;
     }
-    __syncthreads();
   }
-  if (!INV && odd) pairs();
+  __syncthreads();
+#pragma unroll 1
+  for (int j = 1 - odd; j < q; ++j) stage4<T, true>(buf, l, nb, stride, tab, odd + 2 * j);
 }
 
 // C2R of one packed pair: z <- A + i B at the modes' positions from two half rows.
