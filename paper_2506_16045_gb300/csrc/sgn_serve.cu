@@ -14,8 +14,12 @@
 //     inner solves are cooperative persistent launches, which must not wait on one another;
 //   * each piece of work ends with an event; the worker polls the events, completes the
 //     finished requests and issues the next chunk, so the lanes' work overlaps on the device.
-// Work that frees device memory (cudaFree waits for the whole device) is deferred until no
-// lane is busy, or until the deferred bytes pass a threshold.
+// Work that frees device memory is deferred until no lane is busy, or until the deferred bytes
+// pass a threshold: it waits for the whole device once, since a client may still be reading the
+// results that it gave up.  Requests' arrays come from a pool that keeps at most kPoolBytes,
+// and the layouts of finished 2d requests are kept, up to kIdleBytes of them, for later
+// requests on the same grid (a 2d layout is 11 allocations and a solve graph: 0.9 ms to make
+// and to destroy at 512 x 512, against 0.5 ms for a solve).
 // RK4 is a one-step method and every instance of a batched launch is computed by its own
 // CTAs, and a 2d or multistep request runs on its own layout and state, so a request's
 // result does not depend on which requests ran beside it.
@@ -47,6 +51,8 @@ namespace {
 constexpr int kChunk = 16;           // RUN steps per scheduling round
 constexpr int kSolveLanes = 2;       // high-priority lanes of the 1d solve groups
 constexpr size_t kReapBytes = (size_t)2 << 30;   // deferred frees forced past this many bytes
+constexpr size_t kPoolBytes = (size_t)1 << 30;   // free memory that the requests' pool keeps
+constexpr size_t kIdleBytes = (size_t)2 << 30;   // 2d layouts kept for later requests
 
 struct Req {
   uint64_t ticket = 0;
@@ -54,7 +60,9 @@ struct Req {
   int d = 1;
   long long N = 0;
   size_t footprint = 0;
-  // device arrays owned by the request
+  // device arrays owned by the request, in two blocks: results and working arrays
+  void* res_block = nullptr;
+  void* work_block = nullptr;
   double* eta = nullptr;
   double* u = nullptr;                // u (RUN) or the solution x (SOLVE)
   double* b = nullptr;                // SOLVE right-hand side
@@ -132,7 +140,18 @@ struct sgn_server {
   std::vector<Req*> reap_reqs;
   std::vector<sgn_layout*> reap_lays;
   std::vector<sgn_state*> reap_states;
+  std::vector<Req*> reap_results;     // released after their working memory (under mu)
   size_t reap_bytes = 0;
+  size_t res_bytes = 0;               // of reap_results (under mu)
+  cudaMemPool_t pool = nullptr;       // requests' arrays
+  // layouts of finished 2d requests, oldest first
+  struct Idle {
+    sgn_grid g;
+    sgn_layout* lay;
+    size_t bytes;
+  };
+  std::deque<Idle> idle;
+  size_t idle_bytes = 0, idle_cap = 0;
   // cached batch objects for 1d RK4 runs
   std::vector<uint64_t> run_members;
   bool batch_busy = false;
@@ -154,46 +173,118 @@ size_t footprint_of(int d, long long N) {
   return io + work + big + (1 << 16);
 }
 
-void free_req_work(Req* r) {
+bool same_grid(const sgn_grid& a, const sgn_grid& b) {
+  return a.dim == b.dim && a.nx == b.nx && a.ny == b.ny && a.Lx == b.Lx && a.Ly == b.Ly &&
+         a.g == b.g;
+}
+
+void drop_idle(sgn_server* S, size_t keep) {
+  while (S->idle_bytes > keep) {
+    S->idle_bytes -= S->idle.front().bytes;
+    sgn_layout_destroy(S->idle.front().lay);
+    S->idle.pop_front();
+  }
+}
+
+// The layout of a 2d request: one kept from an earlier request on the same grid, or a new one
+// (when memory runs out, after the kept ones have been given back).
+sgn_status take_layout(sgn_server* S, const sgn_grid& g, sgn_layout** out) {
+  for (auto it = S->idle.begin(); it != S->idle.end(); ++it)
+    if (same_grid(it->g, g)) {
+      *out = it->lay;
+      S->idle_bytes -= it->bytes;
+      S->idle.erase(it);
+      return SGN_OK;
+    }
+  sgn_status e = sgn_layout_create(S->ctx, 1, &g, out);
+  if (e && !S->idle.empty()) {
+    drop_idle(S, 0);
+    cudaGetLastError();
+    e = sgn_layout_create(S->ctx, 1, &g, out);
+  }
+  return e;
+}
+
+// Device arrays of `count` doubles each, in one block of the pool (on the copy stream).
+cudaError_t take_block(sgn_server* S, void** block,
+                       std::initializer_list<std::pair<double**, long long>> v) {
+  const size_t al = 32;               // doubles: 256 bytes
+  size_t n = 0;
+  for (auto& x : v) n += ((size_t)x.second + al - 1) / al * al;
+  const cudaError_t e = cudaMallocFromPoolAsync(block, sizeof(double) * n, S->pool, S->copy);
+  if (e) {
+    *block = nullptr;
+    return e;
+  }
+  double* p = static_cast<double*>(*block);
+  for (auto& x : v) {
+    *x.first = x.second ? p : nullptr;
+    p += ((size_t)x.second + al - 1) / al * al;
+  }
+  return cudaSuccess;
+}
+
+// Both only when the device has finished with the request's arrays.
+void free_req_work(sgn_server* S, Req* r) {
   if (r->st) sgn_state_free(r->st);
-  if (r->lay) sgn_layout_destroy(r->lay);
+  if (r->lay && r->d == 2 && r->footprint <= S->idle_cap) {
+    S->idle.push_back({r->q.grid, r->lay, r->footprint});
+    S->idle_bytes += r->footprint;
+    drop_idle(S, S->idle_cap);
+  } else if (r->lay) {
+    sgn_layout_destroy(r->lay);
+  }
   r->st = nullptr;
   r->lay = nullptr;
-  cudaFree(r->h);
-  cudaFree(r->gh);
-  cudaFree(r->b);
-  cudaFree(r->hist);
+  if (r->work_block) cudaFreeAsync(r->work_block, S->copy);
+  r->work_block = nullptr;
   r->h = r->gh = r->b = r->hist = nullptr;
-  if (r->ready) cudaEventDestroy(r->ready);
+  if (r->ready) S->events.push_back(r->ready);
   r->ready = nullptr;
   if (r->own) cudaStreamDestroy(r->own);
   r->own = nullptr;
 }
 
-void free_req_all(Req* r) {
-  free_req_work(r);
-  cudaFree(r->eta);
-  cudaFree(r->u);
-  cudaFree(r->U);
+void free_req_all(sgn_server* S, Req* r) {
+  free_req_work(S, r);
+  if (r->res_block) cudaFreeAsync(r->res_block, S->copy);
   delete r;
 }
 
-// Frees deferred work, which waits for the device: only when no lane is busy, unless the
-// deferred memory has grown past kReapBytes.  A request the client has already released
-// is deleted here; otherwise sgn_result_release deletes it later.
+// Frees deferred work: only when no lane is busy, unless the deferred memory has grown past
+// kReapBytes.  A request the client has already released is deleted here; otherwise
+// sgn_result_release hands it over again.
 void reap(sgn_server* S, bool force) {
-  if (S->reap_reqs.empty() && S->reap_lays.empty() && S->reap_states.empty()) return;
-  if (!force && !S->inflight.empty() && S->reap_bytes < kReapBytes) return;
-  for (Req* r : S->reap_reqs) {
-    free_req_work(r);
-    bool gone;
-    {
-      std::lock_guard<std::mutex> lk(S->mu);
-      r->reaped = true;
-      gone = r->released;
-    }
-    if (gone) free_req_all(r);
+  std::vector<Req*> gone;
+  {
+    std::lock_guard<std::mutex> lk(S->mu);
+    if (S->reap_reqs.empty() && S->reap_lays.empty() && S->reap_states.empty() &&
+        S->reap_results.empty())
+      return;
+    if (!force && !S->inflight.empty() && S->reap_bytes + S->res_bytes < kReapBytes) return;
+    gone.swap(S->reap_results);
+    S->res_bytes = 0;
   }
+  // requests whose results were released by now: their readers' work is part of what the
+  // synchronisation waits for
+  std::vector<Req*> both;
+  {
+    std::lock_guard<std::mutex> lk(S->mu);
+    for (Req* r : S->reap_reqs)
+      if (r->released) both.push_back(r);
+  }
+  cudaDeviceSynchronize();
+  for (Req* r : S->reap_reqs) free_req_work(S, r);
+  {
+    std::lock_guard<std::mutex> lk(S->mu);
+    for (Req* r : S->reap_reqs) {
+      r->reaped = true;
+      if (r->released && std::find(both.begin(), both.end(), r) == both.end())
+        S->reap_results.push_back(r);
+    }
+  }
+  for (Req* r : both) free_req_all(S, r);
+  for (Req* r : gone) free_req_all(S, r);
   for (sgn_state* st : S->reap_states) sgn_state_free(st);
   for (sgn_layout* l : S->reap_lays) sgn_layout_destroy(l);
   S->reap_reqs.clear();
@@ -269,21 +360,21 @@ sgn_status start(sgn_server* S, Req* r) {
     if (!lay) return SGN_ERR_NOMEM;
     // the request's own RK4 history travels with it through the batched state, so its
     // result does not depend on the requests beside it (no history yet: NaN)
-    if (cudaMalloc(&r->hist, sizeof(double) * 2 * (size_t)r->N) != cudaSuccess ||
-        cudaMemsetAsync(r->hist + r->N, 0xff, sizeof(double) * (size_t)r->N, S->stream) !=
-            cudaSuccess) {
+    if (cudaMemsetAsync(r->hist + r->N, 0xff, sizeof(double) * (size_t)r->N, S->stream) !=
+        cudaSuccess) {
       cudaGetLastError();
-      return SGN_ERR_NOMEM;
+      return SGN_ERR_CUDA;
     }
     e = sgn_spectral_grad(S->ctx, lay, r->h, r->gh, s);
     if (!e) e = sgn_apply_operator(S->ctx, lay, r->eta, r->gh, r->u, r->U, s);
   } else if (r->q.kind == SGN_REQ_RUN) {
-    e = sgn_layout_create(S->ctx, 1, &r->q.grid, &r->lay);
+    e = r->d == 2 ? take_layout(S, r->q.grid, &r->lay)
+                  : sgn_layout_create(S->ctx, 1, &r->q.grid, &r->lay);
     if (!e) e = sgn_state_create(S->ctx, r->lay, r->eta, r->U, r->u, r->h, r->gh, &r->st);
     if (!e) e = sgn_state_init(r->st, s);
   } else if (r->d == 2) {
     // SOLVE: grad h now (2d solves also get their layout here)
-    e = sgn_layout_create(S->ctx, 1, &r->q.grid, &r->lay);
+    e = take_layout(S, r->q.grid, &r->lay);
     if (!e) e = sgn_spectral_grad(S->ctx, r->lay, r->h, r->gh, s);
   } else {
     sgn_layout* lay = one_layout(S, r->q.grid);
@@ -579,6 +670,8 @@ void worker_main(sgn_server* S) {
         }
       }
     }
+    if (!admit_now.empty())              // the kept layouts stay within the budget too
+      drop_idle(S, S->budget > S->used ? S->budget - S->used : 0);
     for (Req* r : admit_now) {
       sgn_status e = start(S, r);
       if (e) {
@@ -653,7 +746,7 @@ void worker_main(sgn_server* S) {
       issue_single(S, next2d);
       ++issued;
     }
-    reap(S, S->reap_bytes >= kReapBytes);
+    reap(S, false);
     if (!completed && !issued) {
       std::unique_lock<std::mutex> lk(S->mu);
       S->cv.wait_for(lk, std::chrono::microseconds(50), [&] { return S->stop || !S->pending.empty(); });
@@ -697,6 +790,13 @@ extern "C" sgn_status sgn_server_create(sgn_ctx* ctx, double budget_fraction, sg
   ok = ok && cudaStreamCreateWithPriority(&S->lane_batch, cudaStreamNonBlocking, S->prio_lo) ==
                  cudaSuccess;
   ok = ok && cudaMalloc(&S->info_dev, sizeof(sgn_pcg_info) * kInfoSlots) == cudaSuccess;
+  cudaMemPoolProps pp = {};
+  pp.allocType = cudaMemAllocationTypePinned;
+  pp.location.type = cudaMemLocationTypeDevice;
+  pp.location.id = dev;
+  uint64_t keep = kPoolBytes;
+  ok = ok && cudaMemPoolCreate(&S->pool, &pp) == cudaSuccess &&
+       cudaMemPoolSetAttribute(S->pool, cudaMemPoolAttrReleaseThreshold, &keep) == cudaSuccess;
   ok = ok && cudaMallocHost(&S->info_host, sizeof(sgn_pcg_info) * kInfoSlots) == cudaSuccess;
   if (!ok) {
     cudaGetLastError();
@@ -705,6 +805,7 @@ extern "C" sgn_status sgn_server_create(sgn_ctx* ctx, double budget_fraction, sg
       if (t) cudaStreamDestroy(t);
     cudaFree(S->info_dev);
     cudaFreeHost(S->info_host);
+    if (S->pool) cudaMemPoolDestroy(S->pool);
     sgn_destroy(S->ctx);
     delete S;
     return SGN_ERR_CUDA;
@@ -712,9 +813,18 @@ extern "C" sgn_status sgn_server_create(sgn_ctx* ctx, double budget_fraction, sg
   S->info_used.assign(kInfoSlots, 0);
   const double f = budget_fraction > 0.0 ? budget_fraction : 0.8;
   S->budget = (size_t)(f * (double)tot);
+  S->idle_cap = std::min(kIdleBytes, S->budget / 8);
   S->worker = std::thread(worker_main, S);
   *out = S;
   return SGN_OK;
+}
+
+// A submission that failed: its blocks in the order of the copy stream that filled them.
+static void refuse(sgn_server* S, Req* r) {
+  if (r->res_block) cudaFreeAsync(r->res_block, S->copy);
+  if (r->work_block) cudaFreeAsync(r->work_block, S->copy);
+  cudaGetLastError();
+  delete r;
 }
 
 extern "C" sgn_status sgn_batch_submit(sgn_server* S, const sgn_request* q, uint64_t* ticket) {
@@ -751,14 +861,14 @@ extern "C" sgn_status sgn_batch_submit(sgn_server* S, const sgn_request* q, uint
   r->remaining = q->kind == SGN_REQ_RUN ? q->nsteps : 0;
   r->t_submit = now_s();
   const size_t sN = sizeof(double) * (size_t)r->N;
+  const long long N = r->N, V = d * N;
   cudaSetDevice(S->device);
-  bool ok = cudaMalloc(&r->eta, sN) == cudaSuccess && cudaMalloc(&r->h, sN) == cudaSuccess &&
-            cudaMalloc(&r->u, d * sN) == cudaSuccess && cudaMalloc(&r->gh, d * sN) == cudaSuccess &&
-            cudaMalloc(&r->U, d * sN) == cudaSuccess;
-  if (ok && q->kind == SGN_REQ_SOLVE) ok = cudaMalloc(&r->b, d * sN) == cudaSuccess;
-  if (!ok) {
+  if (take_block(S, &r->res_block, {{&r->eta, N}, {&r->u, V}, {&r->U, V}}) != cudaSuccess ||
+      take_block(S, &r->work_block,
+                 {{&r->h, N}, {&r->gh, V}, {&r->b, q->kind == SGN_REQ_SOLVE ? V : 0},
+                  {&r->hist, is_batched_run(r) ? 2 * N : 0}}) != cudaSuccess) {
     cudaGetLastError();
-    free_req_all(r);
+    refuse(S, r);
     return SGN_ERR_NOMEM;
   }
   const cudaMemcpyKind k = q->host_memory ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice;
@@ -767,7 +877,7 @@ extern "C" sgn_status sgn_batch_submit(sgn_server* S, const sgn_request* q, uint
   cudaMemcpyAsync(q->kind == SGN_REQ_SOLVE ? r->b : r->u, q->u_or_b, d * sN, k, S->copy);
   if (cudaStreamSynchronize(S->copy) != cudaSuccess) {
     cudaGetLastError();
-    free_req_all(r);
+    refuse(S, r);
     return SGN_ERR_CUDA;
   }
   {
@@ -810,14 +920,13 @@ extern "C" sgn_status sgn_result_release(sgn_server* S, uint64_t ticket) {
     if (!it->second->done) return SGN_ERR_PENDING;
     r = it->second;
     S->all.erase(it);
-    // the worker still holds the request in its deferred frees: it deletes it there
-    if (!r->reaped) {
-      r->released = true;
-      return SGN_OK;
+    // the worker frees it, once the device has finished what the client has issued so far
+    r->released = true;
+    if (r->reaped) {
+      S->reap_results.push_back(r);
+      S->res_bytes += r->footprint;
     }
   }
-  cudaSetDevice(S->device);
-  free_req_all(r);
   return SGN_OK;
 }
 
@@ -830,12 +939,17 @@ extern "C" void sgn_server_destroy(sgn_server* S) {
   S->cv.notify_one();
   if (S->worker.joinable()) S->worker.join();
   cudaSetDevice(S->device);
-  for (auto& kv : S->all) free_req_all(kv.second);
+  cudaDeviceSynchronize();
+  for (auto& kv : S->all) free_req_all(S, kv.second);
+  for (Req* r : S->reap_results) free_req_all(S, r);
+  drop_idle(S, 0);
   if (S->run_st) sgn_state_free(S->run_st);
   if (S->run_lay) sgn_layout_destroy(S->run_lay);
   for (auto& kv : S->one1d) sgn_layout_destroy(kv.second);
   cudaFree(S->pk);
   for (cudaEvent_t e : S->events) cudaEventDestroy(e);
+  cudaStreamSynchronize(S->copy);
+  cudaMemPoolDestroy(S->pool);
   for (cudaStream_t t : {S->stream, S->copy, S->lane_solve[0], S->lane_solve[1], S->lane_2d,
                          S->lane_batch})
     cudaStreamDestroy(t);
