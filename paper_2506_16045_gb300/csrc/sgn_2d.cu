@@ -14,6 +14,7 @@
 // (C2R, pointwise w and q, R2C), column FFT whose epilogue forms (G p)^ = w^ - i k q^.
 // A^{-1} per mode (Def:A): z = (r - alpha k (k.r) / (sigma + alpha |k|^2)) / sigma.
 // The n/2 wavenumbers are 0 in both directions (§6.1).
+#include <algorithm>
 #include <cstdio>
 #include <vector>
 
@@ -193,26 +194,28 @@ __global__ void __launch_bounds__(NT, NT < 512 ? 2 : 1) k2_cols(Modes2d M, int l
     const double sigma = a.sc ? a.sc->sigma : 0.0, alphaA = a.sc ? a.sc->alpha_A : 0.0;
     double part = 0.0;      // residual mode (double-float or float64 data)
     TP partw = 0;           // dot-product mode, in the working precision
+    // a thread's column is the same in every pass of the loop
+    const int c = threadIdx.x % TW, col = c0 + c;
+    const T kx = mode_k<T>(MT, col < H ? col : 0, true);
+    const double kxd = M.kx(col), wd = M.weight(col);
     for (int e = threadIdx.x; e < TW * ny; e += NT) {
-      const int p = e / TW, c = e % TW, col = c0 + c, y = mode_at(p, log2ny), sp = sw2(p);
+      const int p = e / TW, y = mode_at(p, log2ny), sp = sw2(p);
       if (col >= H) continue;
       const long long gi = (long long)y * H + col;
-      const T kx = mode_k<T>(MT, col, true), ky = mode_k<T>(MT, y, false);
+      const T ky = mode_k<T>(MT, y, false);
       cplx<T> w1 = buf[(0 * TW + c) * stride + sp], w2 = buf[(1 * TW + c) * stride + sp];
       cplx<T> qh = buf[(2 * TW + c) * stride + sp];
       cplx<T> g1 = w1 - mul_ik(qh, kx), g2 = w2 - mul_ik(qh, ky);
       if (a.residual) {
         g1 = ld_c<T>(a.bvec[0], gi) - g1;
         g2 = ld_c<T>(a.bvec[1], gi) - g2;
-        // r.A^{-1}r for the stopping test
-        const double kxd = M.kx(col), kyd = M.ky(y);
-        const double k2 = kxd * kxd + kyd * kyd;
-        const double f = alphaA / (sigma + alphaA * k2);
-        double r1x = to_f64(g1.x), r1y = to_f64(g1.y), r2x = to_f64(g2.x), r2y = to_f64(g2.y);
-        double krx = kxd * r1x + kyd * r2x, kry = kxd * r1y + kyd * r2y;
-        double z1x = r1x - f * kxd * krx, z1y = r1y - f * kxd * kry;
-        double z2x = r2x - f * kyd * krx, z2y = r2y - f * kyd * kry;
-        part += M.weight(col) * (r1x * z1x + r1y * z1y + r2x * z2x + r2y * z2y);   // sigma times
+        // sigma r.A^{-1}r = |r|^2 - f |k.r|^2 for the stopping test
+        const double kyd = M.ky(y);
+        const double f = alphaA / (sigma + alphaA * (kxd * kxd + kyd * kyd));
+        const double r1x = to_f64(g1.x), r1y = to_f64(g1.y), r2x = to_f64(g2.x), r2y = to_f64(g2.y);
+        const double krx = kxd * r1x + kyd * r2x, kry = kxd * r1y + kyd * r2y;
+        part += wd * ((r1x * r1x + r1y * r1y + r2x * r2x + r2y * r2y) -
+                      f * (krx * krx + kry * kry));
       } else if (a.vdot[0]) {
         if constexpr (std::is_same<T, TP>::value) {
           cplx<T> p1 = ld_c<T>(a.vdot[0], gi), p2 = ld_c<T>(a.vdot[1], gi);
@@ -549,11 +552,22 @@ __global__ void __launch_bounds__(256) k2_bnorm(Modes2d M, const void* b1, const
     const double f = alphaA / (sigma + alphaA * (kx * kx + ky * ky));
     double r1x = to_f64(a.x), r1y = to_f64(a.y), r2x = to_f64(b.x), r2y = to_f64(b.y);
     double krx = kx * r1x + ky * r2x, kry = kx * r1y + ky * r2y;
-    part += M.weight(c) * ((r1x * (r1x - f * kx * krx) + r1y * (r1y - f * kx * kry) +
-                            r2x * (r2x - f * ky * krx) + r2y * (r2y - f * ky * kry)) / sigma);
+    part += M.weight(c) * ((r1x * r1x + r1y * r1y + r2x * r2x + r2y * r2y) -
+                           f * (krx * krx + kry * kry));
   }
-  grid_reduce<256>(part, parts, sc, [&](double s) { sc->bb = s; });
+  grid_reduce<256>(part, parts, sc, [&](double s) { sc->bb = s / sigma; });
 }
+
+// v as a double-float: by integer operations where its exponent lets both parts be normal
+// (float64 conversions cost 64 clocks per warp each; the planes below took 25.8 us at 512 x 512
+// with four of them per value, 19.8 so), else by conversions.
+__device__ __forceinline__ df split_any(double v) {
+  const int e = (int)((__double_as_longlong(v) >> 52) & 0x7ff);
+  if (e == 0 || (e >= 949 && e <= 1150)) return df(v);        // float64 subnormals are zero
+  const float h = (float)v;
+  return df(h, (float)(v - (double)h));
+}
+
 
 // coefficient planes (Def:MatrixM) from eta, grad h
 // (and float32 eta, h_x, h_y for the persistent inner solve, which forms its coefficients
@@ -563,47 +577,95 @@ __global__ void k2_coef_planes(long long P, const double* eta, const double* gh,
   for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < P;
        j += (long long)gridDim.x * blockDim.x) {
     const double e = eta[j], hx = gh[j], hy = gh[P + j];
-    ehh[j] = (float)e;
-    ehh[P + j] = (float)hx;
-    ehh[2 * P + j] = (float)hy;
-    const double c[6] = {e * (1.0 + hx * hx), e * hx * hy, e * (1.0 + hy * hy), 0.5 * e * e * hx,
-                         0.5 * e * e * hy, e * e * e / 3.0};
+    ehh[j] = split_any(e).hi;
+    ehh[P + j] = split_any(hx).hi;
+    ehh[2 * P + j] = split_any(hy).hi;
+    const double eh = e * hx, e2 = 0.5 * e * e;
+    const double c[6] = {fma(eh, hx, e), eh * hy, fma(e * hy, hy, e), e2 * hx, e2 * hy,
+                         e2 * e * (2.0 / 3.0)};
 #pragma unroll
     for (int q = 0; q < 6; ++q) {
-      const float h = (float)c[q];
-      hi[q * P + j] = h;
-      lo[q * P + j] = (float)(c[q] - (double)h);
+      const df v = split_any(c[q]);
+      hi[q * P + j] = v.hi;
+      lo[q * P + j] = v.lo;
     }
   }
 }
 
 // a1 in 2d: block reductions of eta_min, eta_max, max |grad h|^2, max eta(1 + l+ |grad h|^2)
+// The five maxima go through unsigned keys in the order of the doubles (NaN left out, as fmin
+// and fmax do): a float64 minimum or maximum is several instructions of 64 clocks per warp.
+__device__ __forceinline__ unsigned long long dkey(double v) {
+  const long long b = __double_as_longlong(v);
+  return (unsigned long long)(b ^ ((b >> 63) | (long long)0x8000000000000000ull));
+}
+__device__ __forceinline__ double of_dkey(unsigned long long k) {
+  const long long b = (long long)k;
+  return __longlong_as_double(b < 0 ? b ^ (long long)0x8000000000000000ull : ~b);
+}
+__device__ __forceinline__ bool is_nan_bits(double v) {
+  return (__double_as_longlong(v) & 0x7fffffffffffffffll) > 0x7ff0000000000000ll;
+}
+// a0 = min(a0, b0), the others their maxima
+struct Keys {
+  unsigned long long emin, emax, g2, sopt;
+  unsigned bad;
+  __device__ __forceinline__ void take(const Keys& o) {
+    emin = emin < o.emin ? emin : o.emin;
+    emax = emax > o.emax ? emax : o.emax;
+    g2 = g2 > o.g2 ? g2 : o.g2;
+    sopt = sopt > o.sopt ? sopt : o.sopt;
+    bad |= o.bad;
+  }
+  __device__ __forceinline__ Keys from_lane(int o) const {
+    return Keys{__shfl_xor_sync(0xffffffffu, emin, o), __shfl_xor_sync(0xffffffffu, emax, o),
+                __shfl_xor_sync(0xffffffffu, g2, o), __shfl_xor_sync(0xffffffffu, sopt, o),
+                __shfl_xor_sync(0xffffffffu, bad, o)};
+  }
+};
+// over the block of 256; the result on thread 0
+__device__ __forceinline__ void block_keys(Keys& k, Keys* slot) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) k.take(k.from_lane(o));
+  if ((threadIdx.x & 31) == 0) slot[threadIdx.x >> 5] = k;
+  __syncthreads();
+  if (threadIdx.x == 0)
+    for (int w = 1; w < 8; ++w) k.take(slot[w]);
+}
+
+// Bound by float64 issue (four instructions per point) and the reductions.  512 x 512:
+// 36.2 us with float64 minima and maxima and a point per thread; 13.22 with keys and
+// kCoeffBlocks blocks.
+constexpr int kCoeffBlocks = 2 * kSMs;
+
 __global__ void __launch_bounds__(256) k2_coeffs(long long P, const double* eta, const double* gh,
                                                  int kind, double* parts, Scal2d* sc,
                                                  SolveRec* rec) {
-  __shared__ double red[256 / 32 + 1];
-  double emin = 1e308, emax = -1e308, g2max = 0.0, sopt = -1e308, bad = 0.0;
+  __shared__ Keys slot[8];
+  Keys k{dkey(1e308), dkey(-1e308), dkey(0.0), dkey(-1e308), 0u};
   for (long long j = blockIdx.x * 256ll + threadIdx.x; j < P; j += (long long)gridDim.x * 256) {
     const double e = eta[j], hx = gh[j], hy = gh[P + j], g2 = hx * hx + hy * hy;
-    if (!(e > 0.0) || !(g2 < 1e300)) bad = 1.0;
-    emin = fmin(emin, e);
-    emax = fmax(emax, e);
-    g2max = fmax(g2max, g2);
-    sopt = fmax(sopt, e + kLambdaPlus * e * g2);
+    const double so = e + kLambdaPlus * e * g2;
+    const unsigned long long eb = (unsigned long long)__double_as_longlong(e);
+    const unsigned long long gb = (unsigned long long)__double_as_longlong(g2);
+    // !(e > 0) or !(g2 < 1e300)
+    if (eb - 1ull >= 0x7ff0000000000000ull ||
+        gb >= (unsigned long long)__double_as_longlong(1e300))
+      k.bad = 1u;
+    if (!is_nan_bits(e)) {
+      const unsigned long long ke = dkey(e);
+      k.emin = ke < k.emin ? ke : k.emin;
+      k.emax = ke > k.emax ? ke : k.emax;
+    }
+    if (!is_nan_bits(g2) && dkey(g2) > k.g2) k.g2 = dkey(g2);
+    if (!is_nan_bits(so) && dkey(so) > k.sopt) k.sopt = dkey(so);
   }
-  emin = block_min<256>(emin, red);
-  emax = block_max<256>(emax, red);
-  g2max = block_max<256>(g2max, red);
-  sopt = block_max<256>(sopt, red);
-  bad = block_max<256>(bad, red);
+  block_keys(k, slot);
   __shared__ bool last;
+  Keys* kp = reinterpret_cast<Keys*>(parts);           // 5 doubles per block
+  static_assert(sizeof(Keys) <= 5 * sizeof(double), "the partials' slots");
   if (threadIdx.x == 0) {
-    double* p = parts + 5 * blockIdx.x;
-    p[0] = emin;
-    p[1] = emax;
-    p[2] = g2max;
-    p[3] = sopt;
-    p[4] = bad;
+    kp[blockIdx.x] = k;
     __threadfence();
     last = atomicAdd(&sc->ticket, 1u) == gridDim.x - 1;
   }
@@ -611,27 +673,21 @@ __global__ void __launch_bounds__(256) k2_coeffs(long long P, const double* eta,
   if (!last) return;
   {
     // the last block reduces the per-block partials with all its threads
-    volatile double* vp = parts;
-    double a = 1e308, b = -1e308, g = 0.0, s = -1e308, bd = 0.0;
+    __threadfence();
+    k = Keys{dkey(1e308), dkey(-1e308), dkey(0.0), dkey(-1e308), 0u};
     for (int i = threadIdx.x; i < (int)gridDim.x; i += 256) {
-      a = fmin(a, vp[5 * i]);
-      b = fmax(b, vp[5 * i + 1]);
-      g = fmax(g, vp[5 * i + 2]);
-      s = fmax(s, vp[5 * i + 3]);
-      bd = fmax(bd, vp[5 * i + 4]);
+      const volatile Keys* v = kp + i;
+      k.take(Keys{v->emin, v->emax, v->g2, v->sopt, v->bad});
     }
-    a = block_min<256>(a, red);
-    b = block_max<256>(b, red);
-    g = block_max<256>(g, red);
-    s = block_max<256>(s, red);
-    bd = block_max<256>(bd, red);
+    block_keys(k, slot);
+    const double a = of_dkey(k.emin), b = of_dkey(k.emax), g = of_dkey(k.g2), s = of_dkey(k.sopt);
     if (threadIdx.x != 0) return;
     sc->ticket = 0;
     if (kind < 0) kind = sc->kind;          // the solve graph passes the kind through sc
     SolveRec R = {};
     R.eta_min = a;
     R.eta_max = b;
-    if (bd > 0.0) {
+    if (k.bad) {
       R.status = SGN_ERR_NONPOSITIVE_DEPTH;
     } else {
       const double ratio3 = (b / a) * (b / a) * (b / a);
@@ -873,6 +929,19 @@ cudaError_t r2c_vec(const Layout2d& L, const void* t64, const void* t32, const d
   a.planes[1] = o2;
   a.K = 2;
   return cols<T, COL_FWD>(L, t64, t32, a, s);
+}
+
+// Forward transforms of two real vector fields a, b into the half planes o1 .. o4.
+template <typename T>
+cudaError_t r2c_vec2(const Layout2d& L, const void* t64, const void* t32, const double* a,
+                     const double* b, void* o1, void* o2, void* o3, void* o4, cudaStream_t s) {
+  cudaError_t e = rows_r2c<T>(L, t64, t32, a, a + L.P, b, b + L.P, o1, o2, o3, o4, 2, s);
+  if (e) return e;
+  ColArgs c{};
+  void* o[4] = {o1, o2, o3, o4};
+  for (int q = 0; q < 4; ++q) c.planes[q] = o[q];
+  c.K = 4;
+  return cols<T, COL_FWD>(L, t64, t32, c, s);
 }
 
 // Inverse transform of 2 half planes into a real vector field (the half planes are
@@ -1271,7 +1340,7 @@ cudaError_t launch_rhs_nc2d(const Layout2d& L, const void* tw64, double g, const
 
 cudaError_t launch_coeffs2d(const Layout2d& L, const double* eta, const double* gradh, int kind,
                             SolveRec* rec, cudaStream_t s) {
-  k2_coeffs<<<grid_for(L.P, 256), 256, 0, s>>>(L.P, eta, gradh, kind, L.parts, L.sc, rec);
+  k2_coeffs<<<std::min(grid_for(L.P, 256), kCoeffBlocks), 256, 0, s>>>(L.P, eta, gradh, kind, L.parts, L.sc, rec);
   return cudaGetLastError();
 }
 
@@ -1466,7 +1535,7 @@ cudaError_t build_solve_graph(const Layout2d& L, const void* tw64, const void* t
     if (given) {
       k2_set_given<<<1, 1, 0, cs[0]>>>(L.sc, L.stage_rec);
     } else {
-      k2_coeffs<<<grid_for(P, 256), 256, 0, cs[0]>>>(P, eta, gh, -1, L.parts, L.sc, nullptr);
+      k2_coeffs<<<std::min(grid_for(P, 256), kCoeffBlocks), 256, 0, cs[0]>>>(P, eta, gh, -1, L.parts, L.sc, nullptr);
     }
     k2_coef_planes<<<grid_for(P, 256), 256, 0, cs[0]>>>(P, eta, gh, L.coef, L.coef_lo, L.ehh);
     e = cudaGetLastError();
@@ -1474,8 +1543,8 @@ cudaError_t build_solve_graph(const Layout2d& L, const void* tw64, const void* t
   if (mixed) {
     cudaGraphConditionalHandle hout, hin;
     cudaGraph_t body = nullptr, ibody = nullptr;
-    if (!e) e = r2c_vec<df>(L, tw64, tw32, b, slot(L, 0), slot(L, 1), cs[0]);
-    if (!e) e = r2c_vec<df>(L, tw64, tw32, x, slot(L, 2), slot(L, 3), cs[0]);
+    if (!e)
+      e = r2c_vec2<df>(L, tw64, tw32, b, x, slot(L, 0), slot(L, 1), slot(L, 2), slot(L, 3), cs[0]);
     if (!e) {
       k2_bnorm<df><<<blocks, 256, 0, cs[0]>>>(M, slot(L, 0), slot(L, 1), L.sc, L.parts);
       e = cudaGetLastError();
@@ -1529,8 +1598,8 @@ cudaError_t build_solve_graph(const Layout2d& L, const void* tw64, const void* t
   } else {
     cudaGraphConditionalHandle hin;
     cudaGraph_t ibody = nullptr;
-    if (!e) e = r2c_vec<double>(L, tw64, tw32, b, slot(L, 0), slot(L, 1), cs[0]);
-    if (!e) e = r2c_vec<double>(L, tw64, tw32, x, slot(L, 2), slot(L, 3), cs[0]);
+    if (!e)
+      e = r2c_vec2<double>(L, tw64, tw32, b, x, slot(L, 0), slot(L, 1), slot(L, 2), slot(L, 3), cs[0]);
     if (!e) {
       k2_bnorm<double><<<blocks, 256, 0, cs[0]>>>(M, slot(L, 0), slot(L, 1), L.sc, L.parts);
       e = cudaGetLastError();
@@ -1633,7 +1702,7 @@ cudaError_t launch_pcg2d(const Layout2d& L, const void* tw64, const void* tw32, 
   if (given) {
     k2_set_given<<<1, 1, 0, s>>>(L.sc, given);
   } else {
-    k2_coeffs<<<grid_for(L.P, 256), 256, 0, s>>>(L.P, eta, gradh, kind, L.parts, L.sc, nullptr);
+    k2_coeffs<<<std::min(grid_for(L.P, 256), kCoeffBlocks), 256, 0, s>>>(L.P, eta, gradh, kind, L.parts, L.sc, nullptr);
   }
   k2_coef_planes<<<grid_for(L.P, 256), 256, 0, s>>>(L.P, eta, gradh, L.coef, L.coef_lo, L.ehh);
   if ((e = cudaGetLastError())) return e;
@@ -1647,12 +1716,12 @@ cudaError_t launch_pcg2d(const Layout2d& L, const void* tw64, const void* tw32, 
   const bool mixed = precision == SGN_PREC_MIXED;
   // b^ -> slots 0-1, x0^ -> slots 2-3 (high precision)
   if (mixed) {
-    if ((e = r2c_vec<df>(L, tw64, tw32, b, slot(L, 0), slot(L, 1), s))) return e;
-    if ((e = r2c_vec<df>(L, tw64, tw32, x, slot(L, 2), slot(L, 3), s))) return e;
+    if ((e = r2c_vec2<df>(L, tw64, tw32, b, x, slot(L, 0), slot(L, 1), slot(L, 2), slot(L, 3), s)))
+      return e;
     k2_bnorm<df><<<grid_for(L.HP, 256), 256, 0, s>>>(M, slot(L, 0), slot(L, 1), L.sc, L.parts);
   } else {
-    if ((e = r2c_vec<double>(L, tw64, tw32, b, slot(L, 0), slot(L, 1), s))) return e;
-    if ((e = r2c_vec<double>(L, tw64, tw32, x, slot(L, 2), slot(L, 3), s))) return e;
+    if ((e = r2c_vec2<double>(L, tw64, tw32, b, x, slot(L, 0), slot(L, 1), slot(L, 2), slot(L, 3), s)))
+      return e;
     k2_bnorm<double><<<grid_for(L.HP, 256), 256, 0, s>>>(M, slot(L, 0), slot(L, 1), L.sc,
                                                          L.parts);
   }
@@ -1860,12 +1929,12 @@ cudaError_t launch_pcg2d_batch(Layout2d& first, Batch2d& Bt, const void* tw64, c
     if (given) {
       k2_set_given<<<1, 1, 0, s>>>(L.sc, given + i);
     } else {
-      k2_coeffs<<<grid_for(P, 256), 256, 0, s>>>(P, st, st + P, kind, L.parts, L.sc, nullptr);
+      k2_coeffs<<<std::min(grid_for(P, 256), kCoeffBlocks), 256, 0, s>>>(P, st, st + P, kind, L.parts, L.sc, nullptr);
     }
     k2_coef_planes<<<grid_for(P, 256), 256, 0, s>>>(P, st, st + P, L.coef, L.coef_lo, L.ehh);
     if ((e = cudaGetLastError()) ||
-        (e = r2c_vec<df>(L, tw64, tw32, st + 3 * P, slot(L, 0), slot(L, 1), s)) ||
-        (e = r2c_vec<df>(L, tw64, tw32, st + 5 * P, slot(L, 2), slot(L, 3), s)))
+        (e = r2c_vec2<df>(L, tw64, tw32, st + 3 * P, st + 5 * P, slot(L, 0), slot(L, 1), slot(L, 2),
+                          slot(L, 3), s)))
       return e;
     k2_bnorm<df><<<grid_for(L.HP, 256), 256, 0, s>>>(M, slot(L, 0), slot(L, 1), L.sc, L.parts);
     if ((e = cudaGetLastError())) return e;
