@@ -42,17 +42,16 @@ __global__ void k_twiddles(cplx<double>* tw64, cplx<float>* tw32, cplx<df>* twdf
   }
 }
 
-// f_x = D f, one field per CTA (complex transform with zero imaginary part)
+// f_x = D f for n <= 128, one field per CTA (complex transform with zero imaginary part); larger
+// sizes: k_field of sgn_split_1d.cuh
 template <int NT, int MAXB>
 __global__ void __launch_bounds__(NT, 1) k_deriv1d(const Inst1d* __restrict__ insts,
                                                 const int* __restrict__ ids,
-                                                cplx<double>* big,
                                                 const cplx<double>* __restrict__ tw,
                                                 const double* __restrict__ f,
                                                 double* __restrict__ fx) {
   extern __shared__ __align__(16) unsigned char smem[];
-  cplx<double>* buf = big ? big + ((size_t)blockIdx.x << kMaxLog1d)
-                          : reinterpret_cast<cplx<double>*>(smem);
+  cplx<double>* buf = reinterpret_cast<cplx<double>*>(smem);
   const Inst1d I = insts[ids[blockIdx.x]];
   const int n = I.n;
   const double kunit = 2.0 * kPi / I.L;
@@ -69,19 +68,17 @@ __global__ void __launch_bounds__(NT, 1) k_deriv1d(const Inst1d* __restrict__ in
   for (int j = threadIdx.x; j < n; j += NT) fx[I.off + j] = buf[j].x;
 }
 
-// Gu (Def:G) in float64
+// Gu (Def:G) in float64, n <= 128
 template <int NT, int MAXB>
 __global__ void __launch_bounds__(NT, 1) k_apply_G1d(const Inst1d* __restrict__ insts,
                                                   const int* __restrict__ ids,
-                                                  cplx<double>* big,
                                                   const cplx<double>* __restrict__ tw,
                                                   const double* __restrict__ eta,
                                                   const double* __restrict__ hx,
                                                   const double* __restrict__ u,
                                                   double* __restrict__ Gu) {
   extern __shared__ __align__(16) unsigned char smem[];
-  cplx<double>* buf = big ? big + ((size_t)blockIdx.x << kMaxLog1d)
-                          : reinterpret_cast<cplx<double>*>(smem);
+  cplx<double>* buf = reinterpret_cast<cplx<double>*>(smem);
   const Inst1d I = insts[ids[blockIdx.x]];
   const int n = I.n, h = n >> 1;
   for (int j = threadIdx.x; j < n; j += NT) buf[j] = mk(u[I.off + j], 0.0);
@@ -401,14 +398,14 @@ cudaError_t launch_deriv1d(const Layout1d& lay, const void* tw64, const double* 
   auto tw = static_cast<const cplx<double>*>(tw64);
   return for_each_class(lay, s, [&](auto NTc, auto MBc, int l, int first, int num, cudaStream_t s) {
     constexpr int NT = decltype(NTc)::value, MB = decltype(MBc)::value;
-    const bool gl = l > kSmemLog1d;                // transform buffer in global scratch
-    const size_t sm = gl ? 0 : (size_t)16 << l;
-    cplx<double>* big = gl ? static_cast<cplx<double>*>(lay.big) : nullptr;
-    auto k = k_deriv1d<NT, MB>;
-    cudaError_t e = set_smem(k, sm);
-    if (e) return e;
-    k<<<num, NT, sm, s>>>(lay.d_inst, lay.d_ids + first, big, tw, f, fx);
-    return cudaGetLastError();
+    if (l >= kSplitLog1d) return launch_field_split(lay, l, first, num, tw64, f, nullptr, nullptr, fx, s);
+    if constexpr (MB > 1) {                       // n <= 128 has one butterfly per thread
+      return cudaErrorInvalidValue;
+    } else {
+      auto k = k_deriv1d<NT, MB>;
+      k<<<num, NT, (size_t)16 << l, s>>>(lay.d_inst, lay.d_ids + first, tw, f, fx);
+      return cudaGetLastError();
+    }
   }, [&](int first, int num, cudaStream_t s) {
     return mr_launch_deriv(lay, first, num, f, fx, s);
   });
@@ -419,14 +416,14 @@ cudaError_t launch_apply_G1d(const Layout1d& lay, const void* tw64, const double
   auto tw = static_cast<const cplx<double>*>(tw64);
   return for_each_class(lay, s, [&](auto NTc, auto MBc, int l, int first, int num, cudaStream_t s) {
     constexpr int NT = decltype(NTc)::value, MB = decltype(MBc)::value;
-    const bool gl = l > kSmemLog1d;                // transform buffer in global scratch
-    const size_t sm = gl ? 0 : (size_t)16 << l;
-    cplx<double>* big = gl ? static_cast<cplx<double>*>(lay.big) : nullptr;
-    auto k = k_apply_G1d<NT, MB>;
-    cudaError_t e = set_smem(k, sm);
-    if (e) return e;
-    k<<<num, NT, sm, s>>>(lay.d_inst, lay.d_ids + first, big, tw, eta, hx, u, Gu);
-    return cudaGetLastError();
+    if (l >= kSplitLog1d) return launch_field_split(lay, l, first, num, tw64, u, eta, hx, Gu, s);
+    if constexpr (MB > 1) {                       // n <= 128 has one butterfly per thread
+      return cudaErrorInvalidValue;
+    } else {
+      auto k = k_apply_G1d<NT, MB>;
+      k<<<num, NT, (size_t)16 << l, s>>>(lay.d_inst, lay.d_ids + first, tw, eta, hx, u, Gu);
+      return cudaGetLastError();
+    }
   }, [&](int first, int num, cudaStream_t s) {
     return mr_launch_apply_G(lay, first, num, eta, hx, u, Gu, s);
   });

@@ -25,30 +25,44 @@ extern template cudaError_t split_pcg_launch<8>(const PcgArgs&, int, int, int, c
 extern template cudaError_t split_rhs_launch<8>(const RhsArgs&, int, int, int, cudaStream_t);
 extern template cudaError_t split_linimp_launch<8>(const sp::LinArgs&, int, int, int,
                                                      cudaStream_t);
+extern template cudaError_t split_field_launch<8>(const sp::FieldArgs&, int, int, int,
+                                                   cudaStream_t);
 extern template cudaError_t split_pcg_launch<9>(const PcgArgs&, int, int, int, cudaStream_t);
 extern template cudaError_t split_rhs_launch<9>(const RhsArgs&, int, int, int, cudaStream_t);
 extern template cudaError_t split_linimp_launch<9>(const sp::LinArgs&, int, int, int,
                                                      cudaStream_t);
+extern template cudaError_t split_field_launch<9>(const sp::FieldArgs&, int, int, int,
+                                                   cudaStream_t);
 extern template cudaError_t split_pcg_launch<10>(const PcgArgs&, int, int, int, cudaStream_t);
 extern template cudaError_t split_rhs_launch<10>(const RhsArgs&, int, int, int, cudaStream_t);
 extern template cudaError_t split_linimp_launch<10>(const sp::LinArgs&, int, int, int,
                                                      cudaStream_t);
+extern template cudaError_t split_field_launch<10>(const sp::FieldArgs&, int, int, int,
+                                                   cudaStream_t);
 extern template cudaError_t split_pcg_launch<11>(const PcgArgs&, int, int, int, cudaStream_t);
 extern template cudaError_t split_rhs_launch<11>(const RhsArgs&, int, int, int, cudaStream_t);
 extern template cudaError_t split_linimp_launch<11>(const sp::LinArgs&, int, int, int,
                                                      cudaStream_t);
+extern template cudaError_t split_field_launch<11>(const sp::FieldArgs&, int, int, int,
+                                                   cudaStream_t);
 extern template cudaError_t split_pcg_launch<12>(const PcgArgs&, int, int, int, cudaStream_t);
 extern template cudaError_t split_rhs_launch<12>(const RhsArgs&, int, int, int, cudaStream_t);
 extern template cudaError_t split_linimp_launch<12>(const sp::LinArgs&, int, int, int,
                                                      cudaStream_t);
+extern template cudaError_t split_field_launch<12>(const sp::FieldArgs&, int, int, int,
+                                                   cudaStream_t);
 extern template cudaError_t split_pcg_launch<13>(const PcgArgs&, int, int, int, cudaStream_t);
 extern template cudaError_t split_rhs_launch<13>(const RhsArgs&, int, int, int, cudaStream_t);
 extern template cudaError_t split_linimp_launch<13>(const sp::LinArgs&, int, int, int,
                                                      cudaStream_t);
+extern template cudaError_t split_field_launch<13>(const sp::FieldArgs&, int, int, int,
+                                                   cudaStream_t);
 extern template cudaError_t split_pcg_launch<14>(const PcgArgs&, int, int, int, cudaStream_t);
 extern template cudaError_t split_rhs_launch<14>(const RhsArgs&, int, int, int, cudaStream_t);
 extern template cudaError_t split_linimp_launch<14>(const sp::LinArgs&, int, int, int,
                                                      cudaStream_t);
+extern template cudaError_t split_field_launch<14>(const sp::FieldArgs&, int, int, int,
+                                                   cudaStream_t);
 
 // log2 of the CTAs per instance of class l.  At least 2048 points per CTA stay together; from
 // there the classes are halved, the one with the largest share per CTA first, while every CTA
@@ -258,6 +272,24 @@ cudaError_t launch_linimp_split(const Layout1d& lay, int l, int first, int num, 
     case 12: return split_linimp_launch<12>(a, first, num, lcl, s);
     case 13: return split_linimp_launch<13>(a, first, num, lcl, s);
     case 14: return split_linimp_launch<14>(a, first, num, lcl, s);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+cudaError_t launch_field_split(const Layout1d& lay, int l, int first, int num, const void* tw64,
+                               const double* f, const double* eta, const double* hx, double* out,
+                               cudaStream_t s) {
+  const sp::FieldArgs a{lay.d_inst, lay.d_ids, static_cast<const cplx<double>*>(tw64), f, eta, hx,
+                        out};
+  const int lcl = split_lcl(lay, l);
+  switch (l) {
+    case 8: return split_field_launch<8>(a, first, num, lcl, s);
+    case 9: return split_field_launch<9>(a, first, num, lcl, s);
+    case 10: return split_field_launch<10>(a, first, num, lcl, s);
+    case 11: return split_field_launch<11>(a, first, num, lcl, s);
+    case 12: return split_field_launch<12>(a, first, num, lcl, s);
+    case 13: return split_field_launch<13>(a, first, num, lcl, s);
+    case 14: return split_field_launch<14>(a, first, num, lcl, s);
     default: return cudaErrorInvalidValue;
   }
 }

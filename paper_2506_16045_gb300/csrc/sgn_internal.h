@@ -155,6 +155,10 @@ cudaError_t launch_linimp_split(const Layout1d& lay, int l, int first, int num, 
                                 const double* U, const void* res0_hat, void* res1_hat, double c1,
                                 double c0, bool solve, double* u_out, void* ux_out,
                                 cudaStream_t s);
+// The same for the derivative (eta null: out = f_x) and the operator (out = G f), float64.
+cudaError_t launch_field_split(const Layout1d& lay, int l, int first, int num, const void* tw64,
+                               const double* f, const double* eta, const double* hx, double* out,
+                               cudaStream_t s);
 
 // Sizes n = 2^a 3^b 5^c (a >= 1) that are not powers of two, 6 <= n <= 16384: one CTA per
 // instance with a mixed-radix transform in shared memory (n <= 6144; above, in global

@@ -6,4 +6,5 @@ namespace sgn {
 template cudaError_t split_pcg_launch<13>(const PcgArgs&, int, int, int, cudaStream_t);
 template cudaError_t split_rhs_launch<13>(const RhsArgs&, int, int, int, cudaStream_t);
 template cudaError_t split_linimp_launch<13>(const sp::LinArgs&, int, int, int, cudaStream_t);
+template cudaError_t split_field_launch<13>(const sp::FieldArgs&, int, int, int, cudaStream_t);
 }  // namespace sgn
