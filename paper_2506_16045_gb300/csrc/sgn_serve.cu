@@ -15,8 +15,10 @@
 //   * each piece of work ends with an event; the worker polls the events, completes the
 //     finished requests and issues the next chunk, so the lanes' work overlaps on the device.
 // Work that frees device memory is deferred until no lane is busy, or until the deferred bytes
-// pass a threshold: it waits for the whole device once, since a client may still be reading the
-// results that it gave up.  Requests' arrays come from a pool that keeps at most kPoolBytes,
+// pass a threshold.  A request's results are one allocation, freed by cudaFree, which waits for
+// whatever a client still reads from them (a device synchronisation would do for all of them
+// at once, but fails, and breaks the capture, while any thread captures a graph).  Its working
+// arrays, which only the server's streams use, come from a pool that keeps at most kPoolBytes,
 // and the layouts of finished 2d requests are kept, up to kIdleBytes of them, for later
 // requests on the same grid (a 2d layout is 11 allocations and a solve graph: 0.9 ms to make
 // and to destroy at 512 x 512, against 0.5 ms for a solve).
@@ -140,10 +142,8 @@ struct sgn_server {
   std::vector<Req*> reap_reqs;
   std::vector<sgn_layout*> reap_lays;
   std::vector<sgn_state*> reap_states;
-  std::vector<Req*> reap_results;     // released after their working memory (under mu)
   size_t reap_bytes = 0;
-  size_t res_bytes = 0;               // of reap_results (under mu)
-  cudaMemPool_t pool = nullptr;       // requests' arrays
+  cudaMemPool_t pool = nullptr;       // requests' working arrays
   // layouts of finished 2d requests, oldest first
   struct Idle {
     sgn_grid g;
@@ -205,26 +205,20 @@ sgn_status take_layout(sgn_server* S, const sgn_grid& g, sgn_layout** out) {
   return e;
 }
 
-// Device arrays of `count` doubles each, in one block of the pool (on the copy stream).
-cudaError_t take_block(sgn_server* S, void** block,
-                       std::initializer_list<std::pair<double**, long long>> v) {
-  const size_t al = 32;               // doubles: 256 bytes
+// Places device arrays of the given numbers of doubles in one block (256-byte aligned): its
+// size, or with `block` their addresses.
+using Arrays = std::initializer_list<std::pair<double**, long long>>;
+size_t place(void* block, Arrays v) {
+  const size_t al = 32;
   size_t n = 0;
-  for (auto& x : v) n += ((size_t)x.second + al - 1) / al * al;
-  const cudaError_t e = cudaMallocFromPoolAsync(block, sizeof(double) * n, S->pool, S->copy);
-  if (e) {
-    *block = nullptr;
-    return e;
-  }
-  double* p = static_cast<double*>(*block);
   for (auto& x : v) {
-    *x.first = x.second ? p : nullptr;
-    p += ((size_t)x.second + al - 1) / al * al;
+    if (block) *x.first = x.second ? static_cast<double*>(block) + n : nullptr;
+    n += ((size_t)x.second + al - 1) / al * al;
   }
-  return cudaSuccess;
+  return sizeof(double) * n;
 }
 
-// Both only when the device has finished with the request's arrays.
+// When the server's streams have finished with the request.
 void free_req_work(sgn_server* S, Req* r) {
   if (r->st) sgn_state_free(r->st);
   if (r->lay && r->d == 2 && r->footprint <= S->idle_cap) {
@@ -247,44 +241,37 @@ void free_req_work(sgn_server* S, Req* r) {
 
 void free_req_all(sgn_server* S, Req* r) {
   free_req_work(S, r);
-  if (r->res_block) cudaFreeAsync(r->res_block, S->copy);
+  cudaFree(r->res_block);
   delete r;
+}
+
+// Waits for the server's own streams: a request that failed when it was issued may have work
+// on them.
+void drain(sgn_server* S) {
+  for (cudaStream_t t : {S->stream, S->copy, S->lane_solve[0], S->lane_solve[1], S->lane_2d,
+                         S->lane_batch})
+    cudaStreamSynchronize(t);
+  for (Req* r : S->reap_reqs)
+    if (r->own) cudaStreamSynchronize(r->own);
 }
 
 // Frees deferred work: only when no lane is busy, unless the deferred memory has grown past
 // kReapBytes.  A request the client has already released is deleted here; otherwise
-// sgn_result_release hands it over again.
+// sgn_result_release deletes it later.
 void reap(sgn_server* S, bool force) {
-  std::vector<Req*> gone;
-  {
-    std::lock_guard<std::mutex> lk(S->mu);
-    if (S->reap_reqs.empty() && S->reap_lays.empty() && S->reap_states.empty() &&
-        S->reap_results.empty())
-      return;
-    if (!force && !S->inflight.empty() && S->reap_bytes + S->res_bytes < kReapBytes) return;
-    gone.swap(S->reap_results);
-    S->res_bytes = 0;
-  }
-  // requests whose results were released by now: their readers' work is part of what the
-  // synchronisation waits for
-  std::vector<Req*> both;
-  {
-    std::lock_guard<std::mutex> lk(S->mu);
-    for (Req* r : S->reap_reqs)
-      if (r->released) both.push_back(r);
-  }
-  cudaDeviceSynchronize();
-  for (Req* r : S->reap_reqs) free_req_work(S, r);
-  {
-    std::lock_guard<std::mutex> lk(S->mu);
-    for (Req* r : S->reap_reqs) {
+  if (S->reap_reqs.empty() && S->reap_lays.empty() && S->reap_states.empty()) return;
+  if (!force && !S->inflight.empty() && S->reap_bytes < kReapBytes) return;
+  drain(S);
+  for (Req* r : S->reap_reqs) {
+    free_req_work(S, r);
+    bool gone;
+    {
+      std::lock_guard<std::mutex> lk(S->mu);
       r->reaped = true;
-      if (r->released && std::find(both.begin(), both.end(), r) == both.end())
-        S->reap_results.push_back(r);
+      gone = r->released;
     }
+    if (gone) free_req_all(S, r);
   }
-  for (Req* r : both) free_req_all(S, r);
-  for (Req* r : gone) free_req_all(S, r);
   for (sgn_state* st : S->reap_states) sgn_state_free(st);
   for (sgn_layout* l : S->reap_lays) sgn_layout_destroy(l);
   S->reap_reqs.clear();
@@ -746,7 +733,7 @@ void worker_main(sgn_server* S) {
       issue_single(S, next2d);
       ++issued;
     }
-    reap(S, false);
+    reap(S, S->reap_bytes >= kReapBytes);
     if (!completed && !issued) {
       std::unique_lock<std::mutex> lk(S->mu);
       S->cv.wait_for(lk, std::chrono::microseconds(50), [&] { return S->stop || !S->pending.empty(); });
@@ -819,10 +806,10 @@ extern "C" sgn_status sgn_server_create(sgn_ctx* ctx, double budget_fraction, sg
   return SGN_OK;
 }
 
-// A submission that failed: its blocks in the order of the copy stream that filled them.
+// A submission that failed.
 static void refuse(sgn_server* S, Req* r) {
-  if (r->res_block) cudaFreeAsync(r->res_block, S->copy);
   if (r->work_block) cudaFreeAsync(r->work_block, S->copy);
+  cudaFree(r->res_block);
   cudaGetLastError();
   delete r;
 }
@@ -863,14 +850,19 @@ extern "C" sgn_status sgn_batch_submit(sgn_server* S, const sgn_request* q, uint
   const size_t sN = sizeof(double) * (size_t)r->N;
   const long long N = r->N, V = d * N;
   cudaSetDevice(S->device);
-  if (take_block(S, &r->res_block, {{&r->eta, N}, {&r->u, V}, {&r->U, V}}) != cudaSuccess ||
-      take_block(S, &r->work_block,
-                 {{&r->h, N}, {&r->gh, V}, {&r->b, q->kind == SGN_REQ_SOLVE ? V : 0},
-                  {&r->hist, is_batched_run(r) ? 2 * N : 0}}) != cudaSuccess) {
+  const Arrays res = {{&r->eta, N}, {&r->u, V}, {&r->U, V}};
+  const Arrays work = {{&r->h, N}, {&r->gh, V}, {&r->b, q->kind == SGN_REQ_SOLVE ? V : 0},
+                       {&r->hist, is_batched_run(r) ? 2 * N : 0}};
+  if (cudaMalloc(&r->res_block, place(nullptr, res)) != cudaSuccess ||
+      cudaMallocFromPoolAsync(&r->work_block, place(nullptr, work), S->pool, S->copy) !=
+          cudaSuccess) {
     cudaGetLastError();
+    r->work_block = nullptr;
     refuse(S, r);
     return SGN_ERR_NOMEM;
   }
+  place(r->res_block, res);
+  place(r->work_block, work);
   const cudaMemcpyKind k = q->host_memory ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice;
   cudaMemcpyAsync(r->eta, q->eta, sN, k, S->copy);
   cudaMemcpyAsync(r->h, q->h, sN, k, S->copy);
@@ -920,13 +912,14 @@ extern "C" sgn_status sgn_result_release(sgn_server* S, uint64_t ticket) {
     if (!it->second->done) return SGN_ERR_PENDING;
     r = it->second;
     S->all.erase(it);
-    // the worker frees it, once the device has finished what the client has issued so far
-    r->released = true;
-    if (r->reaped) {
-      S->reap_results.push_back(r);
-      S->res_bytes += r->footprint;
+    // the worker still holds the request in its deferred frees: it deletes it there
+    if (!r->reaped) {
+      r->released = true;
+      return SGN_OK;
     }
   }
+  cudaSetDevice(S->device);
+  free_req_all(S, r);                 // its working memory is gone already
   return SGN_OK;
 }
 
@@ -939,9 +932,8 @@ extern "C" void sgn_server_destroy(sgn_server* S) {
   S->cv.notify_one();
   if (S->worker.joinable()) S->worker.join();
   cudaSetDevice(S->device);
-  cudaDeviceSynchronize();
+  drain(S);
   for (auto& kv : S->all) free_req_all(S, kv.second);
-  for (Req* r : S->reap_results) free_req_all(S, r);
   drop_idle(S, 0);
   if (S->run_st) sgn_state_free(S->run_st);
   if (S->run_lay) sgn_layout_destroy(S->run_lay);

@@ -78,3 +78,34 @@ def test_kept_layouts_and_pool(S, frac):
             fail = (sgn.REQ_SOLVE, g[0], problem(64, 64, 1), dict(rtol=1e-14, maxit=1))
             assert serve(sgn, srv, [fail]) == [None]
     srv.close()
+
+
+def test_servers_beside_each_other(S):
+    """Three servers take turns, each on grids of its own, so that one builds layouts and solve
+    graphs while another cleans up: no request of one may fail by what another does."""
+    import threading
+    sgn, ctx = S
+    sizes = [16, 24, 32, 48, 64, 80, 96, 128]
+    failed = []
+
+    def client(k, srv):
+        for rep in range(12):
+            reqs = []
+            for i in range(4):
+                n = sizes[(k + 3 * rep + i) % len(sizes)]
+                L = 10.0 + k + 0.5 * rep                      # a new grid each time
+                reqs.append((sgn.REQ_SOLVE, sgn.Grid(2, n, L, ny=n, Ly=L, g=9.81),
+                             problem(n, n, rep), {}))
+            for i, u in enumerate(serve(sgn, srv, reqs)):
+                if u is None or not np.isfinite(u).all():
+                    failed.append((k, rep, i))
+
+    servers = [sgn.Server(ctx) for _ in range(3)]
+    threads = [threading.Thread(target=client, args=(k, s)) for k, s in enumerate(servers)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    for s in servers:
+        s.close()
+    assert not failed
