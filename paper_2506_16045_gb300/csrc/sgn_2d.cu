@@ -1008,7 +1008,7 @@ cudaError_t matvec(const Layout2d& L, const void* t64, const void* t32, const vo
 namespace {
 
 // The persistent inner solve's view of one instance: correction d^ (slots 8-9), r^ (4-5),
-// p^ (6-7) and the first three transform planes, as float32 half planes.
+// p^ (6-7) and, interleaved, three transform planes, as float32 half planes.
 PInst2d pinst_of(const Layout2d& L) {
   PInst2d pi;
   auto fp = [&](int q) { return reinterpret_cast<cplx<float>*>(slot(L, q)); };
@@ -1018,7 +1018,7 @@ PInst2d pinst_of(const Layout2d& L) {
   pi.r[1] = fp(5);
   pi.p[0] = fp(6);
   pi.p[1] = fp(7);
-  for (int q = 0; q < 3; ++q) pi.t[q] = reinterpret_cast<cplx<float>*>(tplane(L, q));
+  pi.t = reinterpret_cast<cplx<float>*>(tplane(L, 0));
   pi.ehh = L.ehh;
   pi.sc = L.sc;
   pi.kxu = 2.0 * kPi / L.Lx;

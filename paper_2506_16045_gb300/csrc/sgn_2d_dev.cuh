@@ -187,7 +187,7 @@ struct PInst2d {
   cplx<float>* x[2];      // correction
   cplx<float>* r[2];      // residual
   cplx<float>* p[2];      // search direction
-  cplx<float>* t[3];      // transform planes
+  cplx<float>* t;         // three transform planes, [H][ny/2][3][2]
   const float* ehh;       // float32 eta, h_x, h_y: three planes of nx ny
   Scal2d* sc;             // tolerance, cap, A's symbol in; iterations, r.z, status out
   double kxu, kyu;        // 2 pi / Lx, 2 pi / Ly

@@ -736,7 +736,7 @@ PInst2d mr_pinst(const Mr& M) {
     I.x[c] = half(2 + c);
     I.p[c] = half(4 + c);
   }
-  for (int q = 0; q < 3; ++q) I.t[q] = half(6 + q);
+  I.t = half(6);                     // the three interleaved planes
   I.ehh = M.L.ehh;
   I.sc = M.L.sc;
   I.kxu = M.G.kx;

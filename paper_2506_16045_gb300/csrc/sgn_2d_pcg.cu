@@ -436,12 +436,11 @@ __device__ __forceinline__ int neg_mode(int m, int n) {
 }
 
 // Sizes in complex float32 entries, both even (16-byte aligned buffers).  A and B each hold
-// three padded transforms; staged, B also takes the raw row pairs of a row unit (6 (nx/2 + 1)
-// entries).  C holds the largest unit input: six columns of ny (the C2 update vectors) or
+// three padded transforms, and B the raw row pairs of a row unit (6 (nx/2 + 1) entries).  C holds the largest unit input: six columns of ny (the C2 update vectors) or
 // three planes' float32 coefficients of two rows (3 nx entries).
-__host__ __device__ inline int persist_be(int nx, int ny, bool stg) {
+__host__ __device__ inline int persist_be(int nx, int ny) {
   int be = 3 * pad_len(nx > ny ? nx : ny);
-  if (stg && be < 6 * (nx / 2 + 1)) be = 6 * (nx / 2 + 1);
+  if (be < 6 * (nx / 2 + 1)) be = 6 * (nx / 2 + 1);
   return (be + 1) & ~1;
 }
 __host__ __device__ inline int persist_bc(int nx, int ny, bool stg) {
@@ -449,8 +448,17 @@ __host__ __device__ inline int persist_bc(int nx, int ny, bool stg) {
   return 6 * ny > 3 * nx ? 6 * ny : 3 * nx;
 }
 
+// The solve's vectors are column-major, [H][ny]: a column is contiguous.  So is a column of the
+// three transform planes together, with row pairs interleaved ([H][ny / 2][3 planes][2 rows]):
+// a row pair takes 48 contiguous bytes of each column, two sectors, and a warp that reads or
+// writes it touches 11 or 12 lines, where planes of their own cost three half-used sectors and 32
+// lines (512 x 512, 4 RK4 steps: 12.2 -> 11.9 ms; 16 solves of 512 x 512: 15.1 -> 14.4 ms).
+// 16-byte entry i = 3 y/2 + q of column c: plane q, rows y and y + 1.
+__device__ __forceinline__ cplx<float>* t_entry(const PInst2d& I, int ny, int c, int i) {
+  return I.t + ((long long)c * (3 * (ny >> 1)) + i) * 2;
+}
+
 // ---- C1: p update, projection, divergence, column iFFT (column c, group g) -------------
-// The solve's vectors and transform planes are column-major, [H][ny]: a column is contiguous.
 template <bool STG, int GT, bool MR>
 __device__ __forceinline__ void col_inverse(const PersistArgs2d& a, const PInst2d& I,
                                          const IScal& s, int c, const PSmem& sm, int t, int g) {
@@ -541,9 +549,10 @@ __device__ __forceinline__ void col_inverse(const PersistArgs2d& a, const PInst2
   }
   gsync<GT>(g);
   const cplx<float>* o = pfft<GT, MR>(sm.A, sm.B, sm.ly, 3, S, true, sm.twy, t, g);
-  for (int y = t; y < ny; y += GT) {
-#pragma unroll
-    for (int q = 0; q < 3; ++q) stcg(I.t[q] + cb + y, o[q * S + pad(y)]);
+  for (int i = t; i < 3 * (ny >> 1); i += GT) {
+    const int y = 2 * (i / 3), q = i % 3;
+    const cplx<float> a0 = o[q * S + pad(y)], a1 = o[q * S + pad(y + 1)];
+    __stcg(reinterpret_cast<float4*>(t_entry(I, ny, c, i)), make_float4(a0.x, a0.y, a1.x, a1.y));
   }
 }
 
@@ -554,69 +563,40 @@ __device__ __forceinline__ float row_matvec(const PersistArgs2d& a, const PInst2
   const int nx = a.nx, h = nx >> 1, S = pad_len(nx);
   const long long P = (long long)nx * a.ny;
   const int y1 = y0 + 1;
-  // Column m of the transform planes holds rows y0 and y1 side by side (16 bytes): one load
-  // per plane gives packed row 0 (t0, t1 of y0), row 1 (t0, t1 of y1) and row 2 (t2 of y0,
-  // t2 of y1) at mode m; modes above nx/2 are the conjugates of nx - m.
+  // Entry q of column m holds rows y0 and y1 of plane q: they give packed row 0 (t0, t1 of y0),
+  // row 1 (t0, t1 of y1) and row 2 (t2 of y0, t2 of y1) at mode m; modes above nx/2 are the
+  // conjugates of nx - m.
   cplx<float>* z = sm.A;
-  auto pair_ld = [&](int q, int m) {
-    return __ldcg(reinterpret_cast<const float4*>(I.t[q] + (long long)m * a.ny + y0));
-  };
   auto put = [&](int m, cplx<float> u0, cplx<float> v0, cplx<float> u1, cplx<float> v1,
                  cplx<float> u2, cplx<float> v2) {
     z[pad(m)] = mk(u0.x - v0.y, u0.y + v0.x);          // u + i v
     z[S + pad(m)] = mk(u1.x - v1.y, u1.y + v1.x);
     z[2 * S + pad(m)] = mk(u2.x - v2.y, u2.y + v2.x);
   };
-  // staged: the raw row pairs of the three planes go to B (16-byte entries [q (h + 1) + m])
-  // and the six coefficient rows (eta, h_x, h_y of rows y0, y1) to C ([(2 j + r) nx + x]),
-  // all copies in flight at once; the packing then reads shared memory
+  // The raw entries go to B ([m][q]) and, staged, the six coefficient rows (eta, h_x, h_y of
+  // rows y0, y1) to C ([(2 j + r) nx + x]), all copies in flight at once; the packing then
+  // reads shared memory.
   const float* ef = reinterpret_cast<const float*>(sm.C);
+  float4* raw = reinterpret_cast<float4*>(sm.B);
+  const int e0 = 3 * (y0 >> 1);
+  for (int i = t; i < 3 * (h + 1); i += GT) cp16(raw + i, t_entry(I, a.ny, i / 3, e0 + i % 3));
   if constexpr (STG) {
-    float4* raw = reinterpret_cast<float4*>(sm.B);
-    const int hp = h + 1;
-#pragma unroll
-    for (int q = 0; q < 3; ++q)
-      for (int m = t; m <= h; m += GT) cp16(raw + q * hp + m, I.t[q] + (long long)m * a.ny + y0);
     float* ed = reinterpret_cast<float*>(sm.C);
     const int lc = a.lognx - 2, nch = 6 << lc;
     for (int i = t; i < nch; i += GT) {
       const int row = i >> lc, e = (i - (row << lc)) << 2, j = row >> 1, r = row & 1;
       cp16(ed + row * nx + e, I.ehh + j * P + (long long)(y0 + r) * nx + e);
     }
-    cp_wait_all();
-    gsync<GT>(g);
-    for (int m = t; m <= h; m += GT) {
-      const float4 A0 = raw[m], A1 = raw[hp + m], A2 = raw[2 * hp + m];
-      const cplx<float> a0 = mk(A0.x, A0.y), a1 = mk(A0.z, A0.w);
-      const cplx<float> b0 = mk(A1.x, A1.y), b1 = mk(A1.z, A1.w);
-      const cplx<float> d0 = mk(A2.x, A2.y), d1 = mk(A2.z, A2.w);
-      put(m, a0, b0, a1, b1, d0, d1);
-      if (m > 0 && m < h) put(nx - m, conj(a0), conj(b0), conj(a1), conj(b1), conj(d0), conj(d1));
-    }
-  } else
-  for (int m0 = 0; m0 <= h; m0 += kRows * GT) {
-    float4 A0[kRows], A1[kRows], A2[kRows];
-#pragma unroll
-    for (int k = 0; k < kRows; ++k) {
-      const int m = m0 + t + k * GT;
-      if (m <= h) {
-        A0[k] = pair_ld(0, m);
-        A1[k] = pair_ld(1, m);
-        A2[k] = pair_ld(2, m);
-      }
-    }
-#pragma unroll
-    for (int k = 0; k < kRows; ++k) {
-      const int m = m0 + t + k * GT;
-      if (m <= h) {
-        // t0 = (p1(y0), p1(y1)), t1 = (p2(y0), p2(y1)), t2 = (d(y0), d(y1))
-        const cplx<float> a0 = mk(A0[k].x, A0[k].y), a1 = mk(A0[k].z, A0[k].w);
-        const cplx<float> b0 = mk(A1[k].x, A1[k].y), b1 = mk(A1[k].z, A1[k].w);
-        const cplx<float> d0 = mk(A2[k].x, A2[k].y), d1 = mk(A2[k].z, A2[k].w);
-        put(m, a0, b0, a1, b1, d0, d1);
-        if (m > 0 && m < h) put(nx - m, conj(a0), conj(b0), conj(a1), conj(b1), conj(d0), conj(d1));
-      }
-    }
+  }
+  cp_wait_all();
+  gsync<GT>(g);
+  for (int m = t; m <= h; m += GT) {
+    const float4 A0 = raw[3 * m], A1 = raw[3 * m + 1], A2 = raw[3 * m + 2];
+    const cplx<float> a0 = mk(A0.x, A0.y), a1 = mk(A0.z, A0.w);
+    const cplx<float> b0 = mk(A1.x, A1.y), b1 = mk(A1.z, A1.w);
+    const cplx<float> d0 = mk(A2.x, A2.y), d1 = mk(A2.z, A2.w);
+    put(m, a0, b0, a1, b1, d0, d1);
+    if (m > 0 && m < h) put(nx - m, conj(a0), conj(b0), conj(a1), conj(b1), conj(d0), conj(d1));
   }
   gsync<GT>(g);
   cplx<float>* w = pfft<GT, MR>(sm.A, sm.B, sm.lx, 3, S, true, sm.twx, t, g);
@@ -673,20 +653,20 @@ __device__ __forceinline__ float row_matvec(const PersistArgs2d& a, const PInst2
   cplx<float>* other = w == sm.A ? sm.B : sm.A;
   const cplx<float>* Y = pfft<GT, MR>(w, other, sm.lx, 3, S, false, sm.twx, t, g);
   // R2C split of the three packed rows, A = (Y_m + conj Y_{n-m})/2, B = (Y_m - conj Y_{n-m})/(2i),
-  // stored back as row pairs of columns m: t0 = (A_0, A_1), t1 = (B_0, B_1), t2 = (A_2, B_2)
-  for (int m = t; m <= h; m += GT) {
-    cplx<float> A_[3], B_[3];
-#pragma unroll
-    for (int r = 0; r < 3; ++r) {
-      const cplx<float> yv = Y[r * S + pad(m)], yc = conj(Y[r * S + pad(neg_mode<MR>(m, nx))]);
-      const cplx<float> sm2 = yv + yc, dm = mul_mi(yv - yc);
-      A_[r] = mk(0.5f * sm2.x, 0.5f * sm2.y);
-      B_[r] = mk(0.5f * dm.x, 0.5f * dm.y);
-    }
-    const long long o = (long long)m * a.ny + y0;
-    __stcg(reinterpret_cast<float4*>(I.t[0] + o), make_float4(A_[0].x, A_[0].y, A_[1].x, A_[1].y));
-    __stcg(reinterpret_cast<float4*>(I.t[1] + o), make_float4(B_[0].x, B_[0].y, B_[1].x, B_[1].y));
-    __stcg(reinterpret_cast<float4*>(I.t[2] + o), make_float4(A_[2].x, A_[2].y, B_[2].x, B_[2].y));
+  // stored back as row pairs of columns m: t0 = (A_0, A_1), t1 = (B_0, B_1), t2 = (A_2, B_2); a
+  // lane per entry
+  for (int i = t; i < 3 * (h + 1); i += GT) {
+    const int m = i / 3, q = i % 3, mm = neg_mode<MR>(m, nx);
+    const cplx<float>* Ya = Y + (q == 2 ? 2 : 0) * S;
+    const cplx<float>* Yb = Y + (q == 2 ? 2 : 1) * S;
+    auto part_of = [&](const cplx<float>* r, bool odd) {
+      const cplx<float> yv = r[pad(m)], yc = conj(r[pad(mm)]);
+      const cplx<float> s = odd ? mul_mi(yv - yc) : yv + yc;
+      return mk(0.5f * s.x, 0.5f * s.y);
+    };
+    const cplx<float> v0 = part_of(Ya, q == 1), v1 = part_of(Yb, q != 0);
+    __stcg(reinterpret_cast<float4*>(t_entry(I, a.ny, m, e0 + q)),
+           make_float4(v0.x, v0.y, v1.x, v1.y));
   }
   return part;
 }
@@ -700,47 +680,25 @@ __device__ __forceinline__ float col_forward_update(const PersistArgs2d& a, cons
   const long long cb = (long long)c * ny;
   cplx<float>* buf = sm.A;
   const cplx<float>* Cb = sm.C;
+  // every load of the unit in flight at once: the three plane columns to B (as they lie) and,
+  // staged, p1, p2, x1, x2, r1, r2 to C, as 16-byte copies; then the planes are spread into A's
+  // padded transform layout
+  for (int i = t; i < 3 * (ny >> 1); i += GT) cp16(sm.B + 2 * i, t_entry(I, ny, c, i));
   if constexpr (STG) {
-    // every load of the unit in flight at once: the three plane columns to B (unpadded) and
-    // p1, p2, x1, x2, r1, r2 to C, as 16-byte copies; then the planes are spread into A's
-    // padded transform layout
-    cplx<float>* Bb = sm.B;
-    cplx<float>* Cw = sm.C;
-    const int lch = a.logny - 1;
-#pragma unroll
-    for (int q = 0; q < 3; ++q)
-      for (int e = 2 * t; e < ny; e += 2 * GT) cp16(Bb + q * ny + e, I.t[q] + cb + e);
-    const int nch = 6 << lch;
+    const int lch = a.logny - 1, nch = 6 << lch;
     for (int i = t; i < nch; i += GT) {
       const int q = i >> lch, e = (i - (q << lch)) << 1;
       const cplx<float>* src = q < 2 ? I.p[q] : (q < 4 ? I.x[q - 2] : I.r[q - 4]);
-      cp16(Cw + q * ny + e, src + cb + e);
+      cp16(sm.C + q * ny + e, src + cb + e);
     }
-    cp_wait_all();
-    gsync<GT>(g);
-    for (int y = t; y < ny; y += GT) {
-#pragma unroll
-      for (int q = 0; q < 3; ++q) buf[q * S + pad(y)] = Bb[q * ny + y];
-    }
-  } else
-  for (int y0 = 0; y0 < ny; y0 += kRows * GT) {
-    cplx<float> v[3][kRows];
-#pragma unroll
-    for (int k = 0; k < kRows; ++k) {
-      const int y = y0 + t + k * GT;
-      if (y < ny) {
-#pragma unroll
-        for (int q = 0; q < 3; ++q) v[q][k] = ldcg(I.t[q] + cb + y);
-      }
-    }
-#pragma unroll
-    for (int k = 0; k < kRows; ++k) {
-      const int y = y0 + t + k * GT;
-      if (y < ny) {
-#pragma unroll
-        for (int q = 0; q < 3; ++q) buf[q * S + pad(y)] = v[q][k];
-      }
-    }
+  }
+  cp_wait_all();
+  gsync<GT>(g);
+  for (int i = t; i < 3 * (ny >> 1); i += GT) {
+    const int y = 2 * (i / 3), q = i % 3;
+    const float4 v = reinterpret_cast<const float4*>(sm.B)[i];
+    buf[q * S + pad(y)] = mk(v.x, v.y);
+    buf[q * S + pad(y + 1)] = mk(v.z, v.w);
   }
   gsync<GT>(g);
   const cplx<float>* o = pfft<GT, MR>(sm.A, sm.B, sm.ly, 3, S, false, sm.twy, t, g);
@@ -812,7 +770,7 @@ __global__ void __launch_bounds__(kPNT, 1) k2_pcg_persist(const __grid_constant_
   __shared__ MrStages mst[MR ? 2 : 1];
   // thread t of group g; the group's buffers after the twiddle table
   const int g = threadIdx.x / GT, t = threadIdx.x - g * GT;
-  const int be = persist_be(a.nx, a.ny, STG), bc = persist_bc(a.nx, a.ny, STG);
+  const int be = persist_be(a.nx, a.ny), bc = persist_bc(a.nx, a.ny, STG);
   const int ntw = a.nx + (a.ny == a.nx ? 0 : a.ny);
   PSmem sm;
   sm.twx = reinterpret_cast<cplx<float>*>(smem);
@@ -974,7 +932,7 @@ __global__ void k2_persist_arm(unsigned* bar, int* err) {
 // padded transforms (and the staged form's input buffer).
 static size_t persist_smem(int nx, int ny, bool stg, int gt) {
   const long long ntw = nx + (ny == nx ? 0 : ny);
-  const long long per = 2ll * persist_be(nx, ny, stg) + persist_bc(nx, ny, stg);
+  const long long per = 2ll * persist_be(nx, ny) + persist_bc(nx, ny, stg);
   return sizeof(cplx<float>) * (ntw + per * (kPNT / gt));
 }
 
