@@ -308,7 +308,8 @@ struct CoefFor<df> {
   using type = CoefGlobalDF;
 };
 
-// One SBDF2 velocity update in one launch, transforms in T (float64, or double-float for
+// One SBDF2 velocity update in one launch (n <= 128; larger sizes: k_linimp of
+// sgn_split_1d.cuh), transforms in T (float64, or double-float for
 // the mixed path):
 //   res1^ = (sigma + alpha k^2) u^ - (G u - U)^           stored as a half spectrum (float64)
 //   u_out <- F^{-1}[(c1 res1^ + c0 res0^) / (sigma + alpha k^2)]   (SOLVE only)
@@ -319,7 +320,6 @@ struct CoefFor<df> {
 template <typename T, int NT, int MAXB, bool SOLVE>
 __global__ void __launch_bounds__(NT, 1) k_linimp_step1d(const Inst1d* __restrict__ insts,
                                                       const int* __restrict__ ids,
-                                                      cplx<double>* big,
                                                       const cplx<T>* __restrict__ tw,
                                                       const SolveRec* __restrict__ A,
                                                       const double* __restrict__ eta_all,
@@ -333,8 +333,7 @@ __global__ void __launch_bounds__(NT, 1) k_linimp_step1d(const Inst1d* __restric
                                                       double* __restrict__ u_out,
                                                       void* __restrict__ ux_out) {
   extern __shared__ __align__(16) unsigned char smem[];
-  cplx<T>* buf = big ? reinterpret_cast<cplx<T>*>(big + ((size_t)blockIdx.x << kMaxLog1d))
-                     : reinterpret_cast<cplx<T>*>(smem);
+  cplx<T>* buf = reinterpret_cast<cplx<T>*>(smem);
   const int id = ids[blockIdx.x];
   const Inst1d I = insts[id];
   const int n = I.n, h = n >> 1;
@@ -398,9 +397,8 @@ cudaError_t launch_deriv1d(const Layout1d& lay, const void* tw64, const double* 
   auto tw = static_cast<const cplx<double>*>(tw64);
   return for_each_class(lay, s, [&](auto NTc, auto MBc, int l, int first, int num, cudaStream_t s) {
     constexpr int NT = decltype(NTc)::value, MB = decltype(MBc)::value;
-    if (l >= kSplitLog1d) return launch_field_split(lay, l, first, num, tw64, f, nullptr, nullptr, fx, s);
-    if constexpr (MB > 1) {                       // n <= 128 has one butterfly per thread
-      return cudaErrorInvalidValue;
+    if constexpr (MB > 1) {                       // n >= 2^kSplitLog1d
+      return launch_field_split(lay, l, first, num, tw64, f, nullptr, nullptr, fx, s);
     } else {
       auto k = k_deriv1d<NT, MB>;
       k<<<num, NT, (size_t)16 << l, s>>>(lay.d_inst, lay.d_ids + first, tw, f, fx);
@@ -416,9 +414,8 @@ cudaError_t launch_apply_G1d(const Layout1d& lay, const void* tw64, const double
   auto tw = static_cast<const cplx<double>*>(tw64);
   return for_each_class(lay, s, [&](auto NTc, auto MBc, int l, int first, int num, cudaStream_t s) {
     constexpr int NT = decltype(NTc)::value, MB = decltype(MBc)::value;
-    if (l >= kSplitLog1d) return launch_field_split(lay, l, first, num, tw64, u, eta, hx, Gu, s);
-    if constexpr (MB > 1) {                       // n <= 128 has one butterfly per thread
-      return cudaErrorInvalidValue;
+    if constexpr (MB > 1) {                       // n >= 2^kSplitLog1d
+      return launch_field_split(lay, l, first, num, tw64, u, eta, hx, Gu, s);
     } else {
       auto k = k_apply_G1d<NT, MB>;
       k<<<num, NT, (size_t)16 << l, s>>>(lay.d_inst, lay.d_ids + first, tw, eta, hx, u, Gu);
@@ -524,26 +521,26 @@ cudaError_t launch_linimp_step1d(const Layout1d& lay, const void* tw64, const vo
                         : tw64;
   return for_each_class(lay, s, [&](auto NTc, auto MBc, int l, int first, int num, cudaStream_t s) {
     constexpr int NT = decltype(NTc)::value, MB = decltype(MBc)::value;
-    if (l >= kSplitLog1d)
+    if constexpr (MB > 1) {                       // n >= 2^kSplitLog1d
       return launch_linimp_split(lay, l, first, num, tw64, tw32, precision, A, eta, hx, u, U,
                                  res0_hat, res1_hat, c1, c0, solve, u_out ? u_out : u, ux_out, s);
-    const size_t sm = (size_t)16 << l;             // cplx<double> and cplx<df>: 16 bytes
-    auto run = [&](auto kern, auto twp) -> cudaError_t {
-      cudaError_t e = set_smem(kern, sm);
-      if (e) return e;
-      kern<<<num, NT, sm, s>>>(lay.d_inst, lay.d_ids + first, nullptr, twp, A, eta, hx, u, U,
-                               static_cast<const cplx<double>*>(res0_hat),
-                               static_cast<cplx<double>*>(res1_hat), c1, c0,
-                               static_cast<cplx<double>*>(ws), u_out ? u_out : u, ux_out);
-      return cudaGetLastError();
-    };
-    auto twd = static_cast<const cplx<double>*>(twT);
-    auto twf = static_cast<const cplx<df>*>(twT);
-    if (dfp)
-      return solve ? run(k_linimp_step1d<df, NT, MB, true>, twf)
-                   : run(k_linimp_step1d<df, NT, MB, false>, twf);
-    return solve ? run(k_linimp_step1d<double, NT, MB, true>, twd)
-                 : run(k_linimp_step1d<double, NT, MB, false>, twd);
+    } else {
+      const size_t sm = (size_t)16 << l;           // cplx<double> and cplx<df>: 16 bytes
+      auto run = [&](auto kern, auto twp) -> cudaError_t {
+        kern<<<num, NT, sm, s>>>(lay.d_inst, lay.d_ids + first, twp, A, eta, hx, u, U,
+                                 static_cast<const cplx<double>*>(res0_hat),
+                                 static_cast<cplx<double>*>(res1_hat), c1, c0,
+                                 static_cast<cplx<double>*>(ws), u_out ? u_out : u, ux_out);
+        return cudaGetLastError();
+      };
+      auto twd = static_cast<const cplx<double>*>(twT);
+      auto twf = static_cast<const cplx<df>*>(twT);
+      if (dfp)
+        return solve ? run(k_linimp_step1d<df, NT, MB, true>, twf)
+                     : run(k_linimp_step1d<df, NT, MB, false>, twf);
+      return solve ? run(k_linimp_step1d<double, NT, MB, true>, twd)
+                   : run(k_linimp_step1d<double, NT, MB, false>, twd);
+    }
   });
 }
 

@@ -1,6 +1,8 @@
 // a5/a6: preconditioned conjugate gradients for G_{eta,h} x = b in 1d (§3.2, Eq:PCGLinSyst,
 // preconditioner A of §4), one CTA per instance, in spectral space (see sgn_1d.cu for the
-// formulation) on the register-blocked FFT of sgn_fft1d.cuh.
+// formulation) on the register-blocked FFT of sgn_fft1d.cuh: the sizes up to n = 128, and the
+// two-CTA form of n = 4096 and 8192 where it is asked for (the split kernels of
+// sgn_split_1d.cuh run every other size).
 //
 //   MIXED = false: float64 PCG from the caller's initial guess; the Krylov vectors are
 //                  half spectra in the workspace, each thread touching only the modes of
@@ -15,8 +17,8 @@
 //                  a thread) and the correction d in shared memory; its dot products reduce
 //                  in double-float and one thread forms alpha, beta and the stopping test.
 //
-// n = 16384 runs on a thread-block cluster of two CTAs (CL = 2, sgn_fft1d.cuh's two-CTA
-// transforms): each CTA holds half of the points and, in spectral space, the modes of one
+// CL = 2 runs on a thread-block cluster of two CTAs (sgn_fft1d.cuh's two-CTA transforms):
+// each CTA holds half of the points and, in spectral space, the modes of one
 // parity; dot products add the two CTAs' block sums in rank order through distributed
 // shared memory, so both CTAs take every decision from the same numbers.
 //
@@ -54,7 +56,7 @@ struct PcgArgs {
 };
 
 // LG = log2 n; CL = CTAs per instance (2: thread-block clusters of two CTAs of the
-// 2^(LG-1)-point kernel; the only form for LG = 14)
+// 2^(LG-1)-point kernel)
 template <int LG, int CL>
 cudaError_t pcg1d_launch(const PcgArgs& a, int first, int num, cudaStream_t s);
 
@@ -746,7 +748,7 @@ __global__ void __launch_bounds__(Plan<L>::NT, Plan<L>::kMinBlocks)
 template <int LG, int CL>
 cudaError_t pcg1d_launch(const PcgArgs& a, int first, int num, cudaStream_t s) {
   static_assert(CL == 1 || CL == 2, "one CTA or a cluster of two per instance");
-  static_assert(LG <= kSmemLog1d || CL == 2, "n = 16384 needs two CTAs");
+  static_assert(LG <= kSmemLog1d, "larger sizes run on the split kernels");
   constexpr int L = LG - (CL - 1);          // points per CTA: 2^L
   using PL = f1::Plan<L>;
   const bool mixed = a.precision == SGN_PREC_MIXED;

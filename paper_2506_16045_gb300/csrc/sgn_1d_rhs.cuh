@@ -6,9 +6,9 @@
 //   flux -(eta u^2)_x folded in), Q = u d_x - d^2, S = u s_x (reading R6);
 // and f_eta = -m, f_U = -g eta zeta_x + Phi'_x - h_x Psi, Psi = eta^2 Q/2 + eta m d + eta S
 // + m s.  Every pointwise step works on the thread's natural elements j = t + e NTA, so the
-// intermediate planes in `scratch` are written and read by the same thread.  n = 16384 runs
-// on a cluster of two CTAs, each holding half of the points (sgn_fft1d.cuh's two-CTA
-// transforms).
+// intermediate planes in `scratch` are written and read by the same thread.  It runs the
+// sizes up to n = 128 and, where it is asked for, the two-CTA form of n = 4096 and 8192 (each
+// CTA holds half of the points); every other size: k_rhs of sgn_split_1d.cuh.
 #pragma once
 #include <type_traits>
 
@@ -36,7 +36,7 @@ struct RhsArgs {
 };
 
 // LG = log2 n; CL = CTAs per instance (2: thread-block clusters of two CTAs of the
-// 2^(LG-1)-point kernel; the only form for LG = 14)
+// 2^(LG-1)-point kernel)
 template <int LG, int CL>
 cudaError_t rhs1d_launch(const RhsArgs& a, int first, int num, cudaStream_t s);
 
@@ -213,7 +213,7 @@ __global__ void __launch_bounds__(Plan<L>::NT, Plan<L>::kMinBlocks)
 template <int LG, int CL>
 cudaError_t rhs1d_launch(const RhsArgs& a, int first, int num, cudaStream_t s) {
   static_assert(CL == 1 || CL == 2, "one CTA or a cluster of two per instance");
-  static_assert(LG <= kSmemLog1d || CL == 2, "n = 16384 needs two CTAs");
+  static_assert(LG <= kSmemLog1d, "larger sizes run on the split kernels");
   constexpr int L = LG - (CL - 1);          // points per CTA: 2^L
   using PL = f1::Plan<L>;
   const size_t sm = (size_t)16 << L;

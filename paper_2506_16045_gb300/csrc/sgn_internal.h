@@ -40,7 +40,7 @@ struct SolveRec {
 };
 
 constexpr int kWsVectors = 6;          // half-spectrum vectors per instance in the workspace
-constexpr int kMaxLog1d = 14;          // 1d n <= 16384 (n = 16384: two-CTA clusters)
+constexpr int kMaxLog1d = 14;          // 1d n <= 16384
 constexpr int kSmemLog1d = 13;         // largest 1d n whose float64 transform fits in one CTA
 constexpr int kClusterLog1d = 12;      // smallest 1d log2 n with a two-CTA cluster form
 constexpr int kSplitLog1d = 8;         // smallest 1d log2 n of the split kernels
@@ -69,10 +69,11 @@ struct Layout1d {
   // float64 transform buffers (n complex doubles per instance) of the cta_fft kernels for
   // the instances above kSmemLog1d, indexed by position in their size class
   void* big = nullptr;
-  // CTAs per instance of each size class's solve (form) and right-hand side (rform; 0: the
-  // default, one CTA up to kSmemLog1d and two above, and the right-hand side as the solve);
-  // set_form(s) / autotune change them for the classes from kClusterLog1d, and `gen` counts
-  // the changes (captured step graphs hold the old forms)
+  // CTAs per instance asked for by set_form(s) / autotune for each size class's solve (form)
+  // and right-hand side (rform; 0: as the solve's), for the classes from kClusterLog1d: 2 takes
+  // the two-CTA kernels of n = 4096 and 8192, anything else the split kernels with the number
+  // of CTAs that split_lcl chooses; `gen` counts the changes (captured step graphs hold the
+  // old forms)
   int form[16] = {0};
   int rform[16] = {0};                 // the right-hand side's own form (0: as the solve's)
   int gen = 0;

@@ -48,7 +48,8 @@ def serve(sgn, srv, reqs):
             srv.release(t)                                        # given up at once
             out[i] = u if r["status"] == 0 else None
         time.sleep(0.0005)
-    torch.cuda.synchronize()
+    # not the whole device: another server may be capturing its solve graph
+    torch.cuda.current_stream().synchronize()
     return [None if out[i] is None else out[i].cpu().numpy() for i in range(len(reqs))]
 
 
