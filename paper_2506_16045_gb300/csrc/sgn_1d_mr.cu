@@ -24,6 +24,11 @@ using mr::MrPlan;
 using mr::mr_plan;
 using mr::k_mr_twiddles;
 constexpr int kMrNT = 512;
+// Largest n whose float64 solve takes 256 threads: the float64 pipe is the bound
+// either way, and the barriers of 16 warps cost more than they hide while a thread has one or
+// two modes.  512 against 256 threads: a solve at n = 240 1009 and 957 us, at n = 1500 3475 and
+// 3670 us; six RK4 steps at n = 768 equal, at n = 1000 21.5 and 23.1 ms.
+constexpr int kMrSmall64 = 768;
 constexpr int kMrMaxN = 16384;       // largest generic n
 constexpr int kMrSmemN = 6144;       // largest n whose two transform buffers (192 KB) are in
                                      // shared memory; above it they are in global memory
@@ -76,15 +81,15 @@ __device__ __forceinline__ cplx<T>* tbuf(const MrArgs& A, const Inst1d& I, int w
 }
 
 // f_x of the real fields a + i b packed in buf (transform, i k / n, inverse): re / im
-template <typename T>
+template <int NT, typename T>
 __device__ __forceinline__ cplx<T>* mr_deriv_pair(cplx<T>* A, cplx<T>* B, const MrPlan& P,
                                                   double kunit, const cplx<T>* tw) {
   const int n = P.n;
-  cplx<T>* F = mr::mr_fft<T, kMrNT>(A, B, P, false, tw);
+  cplx<T>* F = mr::mr_fft<T, NT>(A, B, P, false, tw);
   const T kn = num<T>(kunit / n);
-  for (int m = threadIdx.x; m < n; m += kMrNT) F[m] = mul_pi(F[m]) * mr_k<T>(m, n, kn);
+  for (int m = threadIdx.x; m < n; m += NT) F[m] = mul_pi(F[m]) * mr_k<T>(m, n, kn);
   __syncthreads();
-  return mr::mr_fft<T, kMrNT>(F, F == A ? B : A, P, true, tw);
+  return mr::mr_fft<T, NT>(F, F == A ? B : A, P, true, tw);
 }
 
 // ---- operators (float64) ----------------------------------------------------------------
@@ -97,18 +102,18 @@ __global__ void __launch_bounds__(kMrNT) k_mr_deriv(const MrArgs A, const double
   cplx<double>* b = tbuf<double>(A, I, 1);
   for (int j = threadIdx.x; j < I.n; j += kMrNT) a[j] = mk(f[I.off + j], 0.0);
   __syncthreads();
-  const cplx<double>* o = mr_deriv_pair<double>(a, b, P, 2.0 * kPi / I.L, mr_tw(A, I).d);
+  const cplx<double>* o = mr_deriv_pair<kMrNT, double>(a, b, P, 2.0 * kPi / I.L, mr_tw(A, I).d);
   for (int j = threadIdx.x; j < I.n; j += kMrNT) fx[I.off + j] = o[j].x;
 }
 
 // The transform of v + i v_x from the half spectrum of the real field v: a_m = (1 - k) v_m and
 // a_{n-m} = (1 + k) conj v_m, the DC and Nyquist coefficients taken real (their imaginary
 // parts are rounding residue).  get(m): v_m, m = 0..n/2.  Ends with a barrier.
-template <typename T, typename Get>
+template <int NT, typename T, typename Get>
 __device__ __forceinline__ void mr_fill(cplx<T>* a, int n, T ku, Get get) {
   const int h = n / 2;
   const T one = from_int<T>(1);
-  for (int m = threadIdx.x; m <= h; m += kMrNT) {
+  for (int m = threadIdx.x; m <= h; m += NT) {
     const cplx<T> v = get(m);
     if (m == 0 || m == h) {
       a[m] = mk(v.x, from_int<T>(0));
@@ -124,12 +129,12 @@ __device__ __forceinline__ void mr_fill(cplx<T>* a, int n, T ku, Get get) {
 // With Z = F(v + i v_x) in a (mr_fill): back to real space, pointwise w = c1 v + c2 v_x,
 // q = c2 v + c3 v_x, and the transform Y of w + i q, from which mr_gv takes (G v)^ (Def:G as
 // w - q_x).  point(j, v, v_x) may keep the field.  Returns Y, after a barrier.
-template <typename T, typename Coef, typename Point>
+template <int NT, typename T, typename Coef, typename Point>
 __device__ __forceinline__ cplx<T>* mr_wq(cplx<T>* a, cplx<T>* b, const MrPlan& P, T inv_n,
                                           const cplx<T>* tw, const Coef& coef, Point point) {
   const int n = P.n;
-  cplx<T>* z = mr::mr_fft<T, kMrNT>(a, b, P, true, tw);
-  for (int j = threadIdx.x; j < n; j += kMrNT) {
+  cplx<T>* z = mr::mr_fft<T, NT>(a, b, P, true, tw);
+  for (int j = threadIdx.x; j < n; j += NT) {
     const T v = z[j].x * inv_n, vx = z[j].y * inv_n;
     T c1, c2, c3;
     coef(j, c1, c2, c3);
@@ -137,7 +142,7 @@ __device__ __forceinline__ cplx<T>* mr_wq(cplx<T>* a, cplx<T>* b, const MrPlan& 
     z[j] = mk(c1 * v + c2 * vx, c2 * v + c3 * vx);
   }
   __syncthreads();
-  return mr::mr_fft<T, kMrNT>(z, z == a ? b : a, P, false, tw);
+  return mr::mr_fft<T, NT>(z, z == a ? b : a, P, false, tw);
 }
 struct NoPoint {
   template <typename T>
@@ -183,7 +188,7 @@ __global__ void __launch_bounds__(kMrNT) k_mr_apply_G(const MrArgs A, const doub
   cplx<double>* o = V == a ? b : a;
   for (int m = threadIdx.x; m < n; m += kMrNT) V[m] = V[m] * (1.0 - mr_k<double>(m, n, kunit));
   __syncthreads();
-  cplx<double>* Y = mr_wq<double>(V, o, P, 1.0 / n, tw, Coef64{eta + I.off, hx + I.off}, NoPoint());
+  cplx<double>* Y = mr_wq<kMrNT, double>(V, o, P, 1.0 / n, tw, Coef64{eta + I.off, hx + I.off}, NoPoint());
   o = Y == a ? b : a;
   // the Hermitian full spectrum of G u into the other buffer, and back
   for (int m = threadIdx.x; m <= h; m += kMrNT) {
@@ -270,8 +275,9 @@ struct DfSum {
 };
 // over the CTA (fixed tree); slot[2][warps] and out[2] are used in turn, so a half is written
 // again only after the barriers of the sum between
+template <int NT>
 __device__ __forceinline__ float mr_sum(df v, df* slots, float* outs, int& turn) {
-  df* slot = slots + turn * (kMrNT / 32);
+  df* slot = slots + turn * (NT / 32);
   float* out = outs + turn;
   turn ^= 1;
 #pragma unroll
@@ -281,7 +287,7 @@ __device__ __forceinline__ float mr_sum(df v, df* slots, float* outs, int& turn)
   if (l == 0) slot[w] = v;
   __syncthreads();
   if (w == 0) {
-    df r = l < kMrNT / 32 ? slot[l] : df(0.0f, 0.0f);
+    df r = l < NT / 32 ? slot[l] : df(0.0f, 0.0f);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1)
       r = r + df(__shfl_xor_sync(0xffffffffu, r.hi, o), __shfl_xor_sync(0xffffffffu, r.lo, o));
@@ -289,6 +295,29 @@ __device__ __forceinline__ float mr_sum(df v, df* slots, float* outs, int& turn)
   }
   __syncthreads();
   return *out;
+}
+// The float64 sum over the CTA of values of the modes m <= h (thread t holds m = t + k kMrNT):
+// block_sum's tree over the warps that hold any, with the same bits (the others add zeros).  A
+// float64 add costs a warp 64 clocks of its sub-partition, idle lanes or not: n = 240 in
+// float64, 6 RK4 steps, took 6.47 ms with all 16 warps in every sum.
+template <int NT>
+__device__ __forceinline__ double mr_sum64(double v, double* scratch, int h) {
+  const int nw = min(NT / 32, (h >> 5) + 1), w = threadIdx.x >> 5, l = threadIdx.x & 31;
+  __syncthreads();                       // scratch may still be read by a previous call
+  if (w < nw) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (l == 0) scratch[w] = v;
+  }
+  __syncthreads();
+  if (w == 0) {
+    double r = l < nw ? scratch[l] : 0.0;
+    for (int o = nw > 8 ? 8 : nw > 4 ? 4 : nw > 2 ? 2 : nw - 1; o > 0; o >>= 1)
+      r += __shfl_xor_sync(0xffffffffu, r, o);
+    if (l == 0) scratch[NT / 32] = r;
+  }
+  __syncthreads();
+  return scratch[NT / 32];
 }
 // 1/a in double-float: a float32 reciprocal and one residual
 __device__ __forceinline__ df mr_recip(df a) {
@@ -303,10 +332,10 @@ __device__ __forceinline__ df mr_recip(df a) {
 // k^2), Parseval weights, dot products and the float32 coefficients in float64 inside the
 // float32 loop; they are float32 and double-float now (the two norms of a refinement pass stay
 // float64).
-template <bool MIXED>
-__global__ void __launch_bounds__(kMrNT) k_mr_pcg(const MrArgs A, const MrPcgArgs a) {
-  __shared__ double red[kMrNT / 32 + 1];
-  __shared__ df slot[2 * (kMrNT / 32)];
+template <bool MIXED, int NT>
+__device__ __forceinline__ void mr_pcg(const MrArgs& A, const MrPcgArgs& a) {
+  __shared__ double red[NT / 32 + 1];
+  __shared__ df slot[2 * (NT / 32)];
   __shared__ float sums[2];
   int turn = 0;
   const int id = A.ids[blockIdx.x];
@@ -325,7 +354,7 @@ __global__ void __launch_bounds__(kMrNT) k_mr_pcg(const MrArgs A, const MrPcgArg
     R = a.given[id];
     R.status = SGN_OK;
   } else {
-    d1::coeffs_block<kMrNT>(eta, hx, n, a.kind, red, R);
+    d1::coeffs_block<NT>(eta, hx, n, a.kind, red, R);
   }
   R.iters = 0;
   R.refinements = 0;
@@ -341,10 +370,10 @@ __global__ void __launch_bounds__(kMrNT) k_mr_pcg(const MrArgs A, const MrPcgArg
   // ---- b^ and x0^ (slots 0 and 1) from one transform of b + i x0, and b.A^{-1}b
   cplx<TH>* d0 = tbuf<TH>(A, I, 0);
   cplx<TH>* d1 = tbuf<TH>(A, I, 1);
-  for (int j = threadIdx.x; j < n; j += kMrNT)
+  for (int j = threadIdx.x; j < n; j += NT)
     d0[j] = mk(num<TH>(a.b[I.off + j]), num<TH>(a.x[I.off + j]));
   __syncthreads();
-  cplx<TH>* Y = mr::mr_fft<TH, kMrNT>(d0, d1, P, false, tw_of<TH>(tws));
+  cplx<TH>* Y = mr::mr_fft<TH, NT>(d0, d1, P, false, tw_of<TH>(tws));
   cplx<TH>* Bh = reinterpret_cast<cplx<TH>*>(ws);
   cplx<TH>* Xh = reinterpret_cast<cplx<TH>*>(ws + S);
   auto half_of = [&](int m, cplx<TH>& bh, cplx<TH>& xh) {
@@ -355,7 +384,7 @@ __global__ void __launch_bounds__(kMrNT) k_mr_pcg(const MrArgs A, const MrPcgArg
   };
   int iters = 0, status = SGN_OK;
   auto no_rhs = [&](double bb) {                   // b = 0 solves exactly, else a breakdown
-    for (int j = threadIdx.x; j < n; j += kMrNT) a.x[I.off + j] = 0.0;
+    for (int j = threadIdx.x; j < n; j += NT) a.x[I.off + j] = 0.0;
     R.status = (bb == 0.0) ? SGN_OK : SGN_ERR_BREAKDOWN;
     if (threadIdx.x == 0) a.rec[id] = R;
   };
@@ -367,7 +396,7 @@ __global__ void __launch_bounds__(kMrNT) k_mr_pcg(const MrArgs A, const MrPcgArg
     double* Dv = reinterpret_cast<double*>(ws + 5 * S);
     auto wgt = [&](int m) { return (m == 0 || m == h) ? 1.0 : 2.0; };
     double bb = 0.0;
-    for (int m = threadIdx.x; m <= h; m += kMrNT) {
+    for (int m = threadIdx.x; m <= h; m += NT) {
       const double k = kunit * wave_index(m, n), di = 1.0 / (sigma + alpha * k * k);
       Dv[m] = di;
       cplx<double> bh, xh;
@@ -376,7 +405,7 @@ __global__ void __launch_bounds__(kMrNT) k_mr_pcg(const MrArgs A, const MrPcgArg
       Xh[m] = xh;
       bb += wgt(m) * (bh.x * bh.x + bh.y * bh.y) * di;
     }
-    bb = block_sum<kMrNT>(bb, red);
+    bb = mr_sum64<NT>(bb, red, h);
     const double bnorm = sqrt(bb);
     if (!(bnorm > 0.0)) {
       no_rhs(bb);
@@ -385,21 +414,21 @@ __global__ void __launch_bounds__(kMrNT) k_mr_pcg(const MrArgs A, const MrPcgArg
     const Coef64 coef{eta, hx};
     const double inv_n = 1.0 / n;
     auto matvec = [&](const cplx<double>* Vh) {     // Gh = (G v)^
-      mr_fill<double>(d0, n, kunit, [&](int m) { return Vh[m]; });
-      const cplx<double>* W = mr_wq<double>(d0, d1, P, inv_n, tws.d, coef, NoPoint());
-      for (int m = threadIdx.x; m <= h; m += kMrNT) Gh[m] = mr_gv<double>(W, m, n, kunit);
+      mr_fill<NT, double>(d0, n, kunit, [&](int m) { return Vh[m]; });
+      const cplx<double>* W = mr_wq<NT, double>(d0, d1, P, inv_n, tws.d, coef, NoPoint());
+      for (int m = threadIdx.x; m <= h; m += NT) Gh[m] = mr_gv<double>(W, m, n, kunit);
       __syncthreads();
     };
     matvec(Xh);
     double rz = 0.0;
-    for (int m = threadIdx.x; m <= h; m += kMrNT) {
+    for (int m = threadIdx.x; m <= h; m += NT) {
       const cplx<double> r = Bh[m] - Gh[m];
       const double di = Dv[m];
       Rh[m] = r;
       Ph[m] = r * di;
       rz += wgt(m) * (r.x * r.x + r.y * r.y) * di;
     }
-    rz = block_sum<kMrNT>(rz, red);
+    rz = mr_sum64<NT>(rz, red, h);
     const double tol = a.rtol * bnorm;
     while (sqrt(rz) > tol) {
       if (iters >= a.maxit) {
@@ -409,22 +438,22 @@ __global__ void __launch_bounds__(kMrNT) k_mr_pcg(const MrArgs A, const MrPcgArg
       __syncthreads();
       matvec(Ph);
       double pq = 0.0;
-      for (int m = threadIdx.x; m <= h; m += kMrNT)
+      for (int m = threadIdx.x; m <= h; m += NT)
         pq += wgt(m) * (Ph[m].x * Gh[m].x + Ph[m].y * Gh[m].y);
-      pq = block_sum<kMrNT>(pq, red);
+      pq = mr_sum64<NT>(pq, red, h);
       if (!(pq > 0.0) || !isfinite(pq)) {
         status = SGN_ERR_BREAKDOWN;
         break;
       }
       const double al = rz / pq;
       double rzn = 0.0;
-      for (int m = threadIdx.x; m <= h; m += kMrNT) {
+      for (int m = threadIdx.x; m <= h; m += NT) {
         Xh[m] = Xh[m] + Ph[m] * al;
         const cplx<double> r = Rh[m] - Gh[m] * al;
         Rh[m] = r;
         rzn += wgt(m) * (r.x * r.x + r.y * r.y) * Dv[m];
       }
-      rzn = block_sum<kMrNT>(rzn, red);
+      rzn = mr_sum64<NT>(rzn, red, h);
       ++iters;
       if (!isfinite(rzn)) {
         status = SGN_ERR_BREAKDOWN;
@@ -432,15 +461,15 @@ __global__ void __launch_bounds__(kMrNT) k_mr_pcg(const MrArgs A, const MrPcgArg
       }
       const double be = rzn / rz;
       rz = rzn;
-      for (int m = threadIdx.x; m <= h; m += kMrNT) Ph[m] = Rh[m] * Dv[m] + Ph[m] * be;
+      for (int m = threadIdx.x; m <= h; m += NT) Ph[m] = Rh[m] * Dv[m] + Ph[m] * be;
     }
     R.ratio = sqrt(rz) / bnorm;
     __syncthreads();
     // x + i x_x from one transform
-    mr_fill<double>(d0, n, kunit, [&](int m) { return Xh[m]; });
-    const cplx<double>* x = mr::mr_fft<double, kMrNT>(d0, d1, P, true, tws.d);
+    mr_fill<NT, double>(d0, n, kunit, [&](int m) { return Xh[m]; });
+    const cplx<double>* x = mr::mr_fft<double, NT>(d0, d1, P, true, tws.d);
     double* ux = a.ux ? static_cast<double*>(a.ux) + I.off : nullptr;
-    for (int j = threadIdx.x; j < n; j += kMrNT) {
+    for (int j = threadIdx.x; j < n; j += NT) {
       a.x[I.off + j] = x[j].x * inv_n;
       if (ux) ux[j] = x[j].y * inv_n;
     }
@@ -476,16 +505,16 @@ __global__ void __launch_bounds__(kMrNT) k_mr_pcg(const MrArgs A, const MrPcgArg
       return (m == 0 || m == h) ? q : q + q;
     };
     double bb = 0.0;
-    for (int m = threadIdx.x; m <= h; m += kMrNT) {
+    for (int m = threadIdx.x; m <= h; m += NT) {
       cplx<df> bh, xh;
       half_of(m, bh, xh);
       Bh[m] = bh;
       Xh[m] = xh;
       bb += term(m, bh);
     }
-    for (int j = threadIdx.x; j < n; j += kMrNT)
+    for (int j = threadIdx.x; j < n; j += NT)
       eh[j] = make_float2(df(eta[j]).hi, df(hx[j]).hi);
-    bb = block_sum<kMrNT>(bb, red);
+    bb = mr_sum64<NT>(bb, red, h);
     const double bnorm = sqrt(bb);
     if (!(bnorm > 0.0)) {
       no_rhs(bb);
@@ -497,18 +526,18 @@ __global__ void __launch_bounds__(kMrNT) k_mr_pcg(const MrArgs A, const MrPcgArg
     double ratio = 0.0;
     for (;;) {
       // r^ = b^ - (G x)^ in double-float, and r.A^{-1}r; the real-space x on the way
-      mr_fill<df>(d0, n, kuh, [&](int m) { return Xh[m]; });
-      const cplx<df>* W = mr_wq<df>(d0, d1, P, inv_n, tws.h, cdf, [&](int j, df v, df vx) {
+      mr_fill<NT, df>(d0, n, kuh, [&](int m) { return Xh[m]; });
+      const cplx<df>* W = mr_wq<NT, df>(d0, d1, P, inv_n, tws.h, cdf, [&](int j, df v, df vx) {
         xo[j] = __hiloint2double(__float_as_int(v.lo), __float_as_int(v.hi));
         if (ux) ux[j] = vx;
       });
       double rs = 0.0;
-      for (int m = threadIdx.x; m <= h; m += kMrNT) {
+      for (int m = threadIdx.x; m <= h; m += NT) {
         const cplx<df> r = Bh[m] - mr_gv<df>(W, m, n, kuh);
         Gd[m] = r;
         rs += term(m, r);
       }
-      const double nr = sqrt(block_sum<kMrNT>(rs, red));
+      const double nr = sqrt(mr_sum64<NT>(rs, red, h));
       ratio = nr / bnorm;
       if (ratio <= a.rtol) {
         status = SGN_OK;
@@ -525,14 +554,14 @@ __global__ void __launch_bounds__(kMrNT) k_mr_pcg(const MrArgs A, const MrPcgArg
       // float32 PCG for G d = r / ||r||; p = A^{-1} r + beta p is formed with its transform's
       // input (beta = 0 first), and (G p)^ is taken from Y twice instead of being kept
       DfSum z0;
-      for (int m = threadIdx.x; m <= h; m += kMrNT) {
+      for (int m = threadIdx.x; m <= h; m += NT) {
         const cplx<df> g = Gd[m];
         const cplx<float> r = mk((g.x.hi + g.x.lo) * sc, (g.y.hi + g.y.lo) * sc);
         Rf[m] = r;
         Df[m] = Pf[m] = mk(0.0f, 0.0f);
         z0.add(wf(m) * ((r.x * r.x + r.y * r.y) * dinvf(m)));
       }
-      float rz = mr_sum(z0.s, slot, sums, turn), beta = 0.0f;
+      float rz = mr_sum<NT>(z0.s, slot, sums, turn), beta = 0.0f;
       const int it0 = iters;
       int st_in = SGN_OK;
       while (rz > tin2) {
@@ -540,31 +569,31 @@ __global__ void __launch_bounds__(kMrNT) k_mr_pcg(const MrArgs A, const MrPcgArg
           st_in = SGN_ERR_NOT_CONVERGED;
           break;
         }
-        mr_fill<float>(f0, n, kf, [&](int m) {
+        mr_fill<NT, float>(f0, n, kf, [&](int m) {
           const cplx<float> p = Rf[m] * dinvf(m) + Pf[m] * beta;
           Pf[m] = p;
           return p;
         });
-        const cplx<float>* Yf = mr_wq<float>(f0, f1, P, inv_nf, tws.f, c32, NoPoint());
+        const cplx<float>* Yf = mr_wq<NT, float>(f0, f1, P, inv_nf, tws.f, c32, NoPoint());
         DfSum ps;
-        for (int m = threadIdx.x; m <= h; m += kMrNT) {
+        for (int m = threadIdx.x; m <= h; m += NT) {
           const cplx<float> p = Pf[m], g = mr_gv<float>(Yf, m, n, kf);
           ps.add(wf(m) * (p.x * g.x + p.y * g.y));
         }
-        const float pq = mr_sum(ps.s, slot, sums, turn);
+        const float pq = mr_sum<NT>(ps.s, slot, sums, turn);
         if (!(pq > 0.0f) || !isfinite(pq)) {
           st_in = SGN_ERR_BREAKDOWN;
           break;
         }
         const float al = rz / pq;
         DfSum zs;
-        for (int m = threadIdx.x; m <= h; m += kMrNT) {
+        for (int m = threadIdx.x; m <= h; m += NT) {
           Df[m] = Df[m] + Pf[m] * al;
           const cplx<float> r = Rf[m] - mr_gv<float>(Yf, m, n, kf) * al;
           Rf[m] = r;
           zs.add(wf(m) * ((r.x * r.x + r.y * r.y) * dinvf(m)));
         }
-        const float rzn = mr_sum(zs.s, slot, sums, turn);
+        const float rzn = mr_sum<NT>(zs.s, slot, sums, turn);
         ++iters;
         if (!isfinite(rzn)) {
           st_in = SGN_ERR_BREAKDOWN;
@@ -577,14 +606,14 @@ __global__ void __launch_bounds__(kMrNT) k_mr_pcg(const MrArgs A, const MrPcgArg
       // decides); the iteration cap is reported by the refinement loop
       if (st_in == SGN_ERR_BREAKDOWN && iters == it0) status = SGN_ERR_BREAKDOWN;
       const df un(nr);
-      for (int m = threadIdx.x; m <= h; m += kMrNT)
+      for (int m = threadIdx.x; m <= h; m += NT)
         Xh[m] = mk(Xh[m].x + df(Df[m].x, 0.0f) * un, Xh[m].y + df(Df[m].y, 0.0f) * un);
       ++refinements;
       __syncthreads();                             // d has been read; d0 is filled next
     }
     R.refinements = refinements;
     R.ratio = ratio;
-    for (int j = threadIdx.x; j < n; j += kMrNT) {
+    for (int j = threadIdx.x; j < n; j += NT) {
       const double v = xo[j];
       xo[j] = to_f64(df(__int_as_float(__double2loint(v)), __int_as_float(__double2hiint(v))));
     }
@@ -592,6 +621,17 @@ __global__ void __launch_bounds__(kMrNT) k_mr_pcg(const MrArgs A, const MrPcgArg
   R.iters = iters;
   R.status = status;
   if (threadIdx.x == 0) a.rec[id] = R;
+}
+
+// The threads follow the instance, so that its result does not depend on the ones beside it.
+template <bool MIXED>
+__global__ void __launch_bounds__(kMrNT) k_mr_pcg(const MrArgs A, const MrPcgArgs a) {
+  if (!MIXED && A.insts[A.ids[blockIdx.x]].n <= kMrSmall64) {
+    if (threadIdx.x >= 256) return;      // the barriers wait for the threads that are left
+    mr_pcg<MIXED, 256>(A, a);
+    return;
+  }
+  mr_pcg<MIXED, kMrNT>(A, a);
 }
 
 // ---- right-hand side (Eq:DAE_DSWE with Def:bigF, reading R6) ----------------------------
@@ -644,7 +684,7 @@ __global__ void __launch_bounds__(kMrNT) k_mr_rhs(const MrArgs A, double g, cons
       }
       __syncthreads();
     }
-    const cplx<T>* r = mr_deriv_pair<T>(b0, b1, P, kunit, tw);
+    const cplx<T>* r = mr_deriv_pair<kMrNT, T>(b0, b1, P, kunit, tw);
     if (what == 5) {
       for (int j = threadIdx.x; j < n; j += kMrNT) {
         const T e = num<T>(eta[o + j]), g1 = num<T>(hx[o + j]);
