@@ -43,7 +43,8 @@ struct RhsArgs2d {
 enum { W_UX = 0, W_MX, W_ZX, W_SX, W_TXX, W_TXY, W_D, W_M, W_PX, W_PY, W_SY, W_DY, W_PHI, W_R };
 
 // Columns per CTA: four float64 fill a 32-byte sector; fewer on narrow grids, where tiles of
-// four would leave SMs idle (nx = 256: 64 tiles).
+// four would leave SMs idle (nx = 256: 64 tiles; 256 x 256 float64, 2 RK4 steps: 10.66 ms with
+// four, 10.46 with two).
 int rhs_tw(int nx) { return nx >= 512 ? 4 : (nx >= 256 ? 2 : 1); }
 
 template <typename T>
