@@ -383,8 +383,12 @@ __device__ __forceinline__ void mr_pcg(const MrArgs& A, const MrPcgArgs& a) {
     xh = mk(half(sx.x), half(sx.y));
   };
   int iters = 0, status = SGN_OK;
-  auto no_rhs = [&](double bb) {                   // b = 0 solves exactly, else a breakdown
-    for (int j = threadIdx.x; j < n; j += NT) a.x[I.off + j] = 0.0;
+  // b = 0 solves exactly, else a breakdown; x_x goes to the right-hand side with x
+  auto no_rhs = [&](double bb) {
+    for (int j = threadIdx.x; j < n; j += NT) {
+      a.x[I.off + j] = 0.0;
+      if (a.ux) static_cast<TH*>(a.ux)[I.off + j] = from_int<TH>(0);
+    }
     R.status = (bb == 0.0) ? SGN_OK : SGN_ERR_BREAKDOWN;
     if (threadIdx.x == 0) a.rec[id] = R;
   };

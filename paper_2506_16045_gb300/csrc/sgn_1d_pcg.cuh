@@ -302,7 +302,10 @@ __device__ __forceinline__ void pcg_body(const PcgArgs& A, int first, void* ux) 
   if (!(bnorm > 0.0)) {
     if (g.act)
 #pragma unroll
-      for (int e = 0; e < E; ++e) x[t + e * NTA] = 0.0;
+      for (int e = 0; e < E; ++e) {
+        x[t + e * NTA] = 0.0;
+        if (ux) static_cast<TH*>(ux)[own + t + e * NTA] = from_int<TH>(0);
+      }
     R.status = (bb == 0.0) ? SGN_OK : SGN_ERR_BREAKDOWN;
     if (ts) A.rec[id] = R;
     return;

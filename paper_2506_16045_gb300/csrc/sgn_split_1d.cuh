@@ -327,9 +327,13 @@ __global__ void SGN_SPLIT_BOUNDS(PL, 3)
     reduce<PL>(df(bb, 0.0f), slots, hb, g, [&](df s) { sc.bb = s; });
   }
   const float bbf = sc.bb.hi;
-  if (!(bbf > 0.0f)) {
+  const df zero(0.0f, 0.0f);
+  if (!(bbf > 0.0f)) {                   // x = 0, and its derivative for the right-hand side
 #pragma unroll
-    for (int e = 0; e < E; ++e) x[g.pt + e * PS] = 0.0;
+    for (int e = 0; e < E; ++e) {
+      x[g.pt + e * PS] = 0.0;
+      if (ux) ux[g.pt + e * PS] = zero;
+    }
     if (ts) {
       st.R.status = bbf == 0.0f ? SGN_OK : SGN_ERR_BREAKDOWN;
       A.rec[id] = st.R;
@@ -340,7 +344,7 @@ __global__ void SGN_SPLIT_BOUNDS(PL, 3)
 
   const df inv_n(1.0f / (float)n, 0.0f);                              // exact
   const float inv_nf = 1.0f / (float)n;
-  const df one(1.0f, 0.0f), zero(0.0f, 0.0f);
+  const df one(1.0f, 0.0f);
   const float rtolf = (float)A.rtol;
   const df rtol2 = df(A.rtol * A.rtol);
   int iters = 0, status = SGN_OK, refinements = 0;
@@ -704,9 +708,12 @@ __global__ void SGN_SPLIT_BOUNDS(PL, 2)
       sc.tol2 = sc.tol * sc.tol;
     });
   }
-  if (!(sc.bb > 0.0)) {
+  if (!(sc.bb > 0.0)) {                  // x = 0, and its derivative for the right-hand side
 #pragma unroll
-    for (int e = 0; e < E; ++e) x[g.pt + e * PS] = 0.0;
+    for (int e = 0; e < E; ++e) {
+      x[g.pt + e * PS] = 0.0;
+      if (ux) ux[g.pt + e * PS] = 0.0;
+    }
     if (ts) {
       st.R.status = sc.bb == 0.0 ? SGN_OK : SGN_ERR_BREAKDOWN;
       A.rec[id] = st.R;
