@@ -191,8 +191,10 @@ __device__ __forceinline__ df recip_t(df a) { return recip_df(a); }
 
 // ---- solve, mixed precision ---------------------------------------------------------------
 struct MixedScalars {
-  df bb, ratio2;            // b.A^{-1}b; r.A^{-1}r over it
-  float scale, unscale, tin2;
+  double bb, lim, rz64;     // b.A^{-1}b, rtol^2 times it, r.A^{-1}r: their quotients and squares
+                            // may leave the float32 range
+  df unscale;               // ||r||_{A^{-1}}
+  float ibn, scale, tin2;   // 1 / ||b||_{A^{-1}}, 1 / ||r||_{A^{-1}}, (inner tolerance)^2
   int go, status;
   float rz, alpha, beta;    // inner solve
   int state;                // 0 iterate, 1 converged, 2 breakdown, 3 iteration cap
@@ -324,18 +326,22 @@ __global__ void SGN_SPLIT_BOUNDS(PL, 3)
       Xh[h] = mk(y.y, df(0.0f, 0.0f));
       bb += y.x.hi * y.x.hi * dN;
     }
-    reduce<PL>(df(bb, 0.0f), slots, hb, g, [&](df s) { sc.bb = s; });
+    reduce<PL>(df(bb, 0.0f), slots, hb, g, [&](df s) {
+      sc.bb = (double)s.hi + (double)s.lo;
+      sc.lim = A.rtol * A.rtol * sc.bb;
+      sc.ibn = recip(sqrtf(s.hi));
+    });
   }
-  const float bbf = sc.bb.hi;
+  const double bb = sc.bb;
   const df zero(0.0f, 0.0f);
-  if (!(bbf > 0.0f)) {                   // x = 0, and its derivative for the right-hand side
+  if (!(bb > 0.0)) {                     // x = 0, and its derivative for the right-hand side
 #pragma unroll
     for (int e = 0; e < E; ++e) {
       x[g.pt + e * PS] = 0.0;
       if (ux) ux[g.pt + e * PS] = zero;
     }
     if (ts) {
-      st.R.status = bbf == 0.0f ? SGN_OK : SGN_ERR_BREAKDOWN;
+      st.R.status = bb == 0.0 ? SGN_OK : SGN_ERR_BREAKDOWN;
       A.rec[id] = st.R;
     }
     if (lcl) cluster_sync();
@@ -346,7 +352,6 @@ __global__ void SGN_SPLIT_BOUNDS(PL, 3)
   const float inv_nf = 1.0f / (float)n;
   const df one(1.0f, 0.0f);
   const float rtolf = (float)A.rtol;
-  const df rtol2 = df(A.rtol * A.rtol);
   int iters = 0, status = SGN_OK, refinements = 0;
   for (;;) {
     // ---- double-float residual r^ = b^ - (G x)^, keeping the real-space x on the way
@@ -393,33 +398,31 @@ __global__ void SGN_SPLIT_BOUNDS(PL, 3)
         rN = mk(rr.hi + rr.lo, 0.0f);
         rz += rN.x * rN.x * dN;
       }
-      // one thread decides the pass: converged, out of budget, or the next inner solve
+      // one thread decides the pass: converged (r.A^{-1}r against rtol^2 b.A^{-1}b in float64),
+      // out of budget, or the next inner solve
       reduce<PL>(df(rz, 0.0f), slots, hb, g, [&](df s) {
-        const df bb = sc.bb, ib = recip_df(bb);
-        const df q2 = s * ib;
-        sc.ratio2 = q2;
+        const double rzd = (double)s.hi + (double)s.lo;
+        sc.rz64 = rzd;
         sc.go = 0;
         sc.status = status;
-        const df d = q2 - rtol2;
-        if (d.hi <= 0.0f || status != SGN_OK) return;
+        if (rzd <= sc.lim || status != SGN_OK) return;
         if (refinements >= A.max_refine || iters >= A.maxit) {
           sc.status = SGN_ERR_NOT_CONVERGED;
           return;
         }
-        const float tin = A.rtol_inner > 0.0
-                              ? (float)A.rtol_inner
-                              : fminf(0.1f, fmaxf(1e-6f, 0.3f * rtolf * rsqrtf(q2.hi)));
-        const float nr = sqrtf(s.hi);
-        sc.unscale = nr;
+        // the root of s in double-float: a float32 root and its residual
+        const float nr = sqrtf(s.hi), dn = 0.5f * (fmaf(-nr, nr, s.hi) + s.lo) / nr;
+        const float tin = fminf(0.1f, fmaxf(1e-6f, 0.3f * rtolf / (nr * sc.ibn)));
+        sc.tin2 = A.rtol_inner > 0.0 ? (float)(A.rtol_inner * A.rtol_inner) : tin * tin;
+        sc.unscale = df(nr, dn);
         sc.scale = recip(nr);
-        sc.tin2 = tin * tin;
         sc.go = 1;
       });
     }
     status = sc.status;
     if (!sc.go) break;
     const float scale = sc.scale, tin2 = sc.tin2;
-    const df unscale(sc.unscale, 0.0f);
+    const df unscale = sc.unscale;
 
     // ---- float32 PCG for G d = r / ||r||
     const int it_before = iters;
@@ -555,7 +558,7 @@ __global__ void SGN_SPLIT_BOUNDS(PL, 3)
   }
   if (ts) {
     SolveRec R = st.R;
-    R.ratio = sqrt(to_f64(sc.ratio2));
+    R.ratio = sqrt(sc.rz64 / sc.bb);
     R.refinements = refinements;
     R.iters = iters;
     R.status = status;
