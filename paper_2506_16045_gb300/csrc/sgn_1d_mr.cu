@@ -263,22 +263,13 @@ struct Coef32 {            // from float32 copies of eta and h_x
   }
 };
 
-// A sum kept in double-float (48 bits; its terms are float32 or double-float): no float64 in
-// the loops of the mixed path.
-struct DfSum {
-  df s{0.0f, 0.0f};
-  __device__ __forceinline__ void add(float v) {
-    const float h = __fadd_rn(s.hi, v), bb = __fsub_rn(h, s.hi);
-    const float e = __fadd_rn(__fsub_rn(s.hi, __fsub_rn(h, bb)), __fsub_rn(v, bb));
-    s = df(h, __fadd_rn(s.lo, e));
-  }
-};
-// over the CTA (fixed tree); slot[2][warps] and out[2] are used in turn, so a half is written
+// The mixed path's sums over the CTA in double-float (48 bits; no float64 in its loops), by a
+// fixed tree; slot[2][warps] and out[2] are used in turn, so a half is written
 // again only after the barriers of the sum between
 template <int NT>
-__device__ __forceinline__ float mr_sum(df v, df* slots, float* outs, int& turn) {
+__device__ __forceinline__ df mr_sum(df v, df* slots, df* outs, int& turn) {
   df* slot = slots + turn * (NT / 32);
-  float* out = outs + turn;
+  df* out = outs + turn;
   turn ^= 1;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1)
@@ -291,7 +282,7 @@ __device__ __forceinline__ float mr_sum(df v, df* slots, float* outs, int& turn)
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1)
       r = r + df(__shfl_xor_sync(0xffffffffu, r.hi, o), __shfl_xor_sync(0xffffffffu, r.lo, o));
-    if (l == 0) *out = r.hi + r.lo;
+    if (l == 0) *out = r;
   }
   __syncthreads();
   return *out;
@@ -319,13 +310,6 @@ __device__ __forceinline__ double mr_sum64(double v, double* scratch, int h) {
   __syncthreads();
   return scratch[NT / 32];
 }
-// 1/a in double-float: a float32 reciprocal and one residual
-__device__ __forceinline__ df mr_recip(df a) {
-  const float r = __frcp_rn(a.hi);
-  const float e = fmaf(-a.lo, r, fmaf(-a.hi, r, 1.0f));
-  const float c = __fmul_rn(r, e), h = __fadd_rn(r, c);
-  return df(h, __fsub_rn(c, __fsub_rn(h, r)));
-}
 
 // One CTA per instance.  Bound by its SM: transforms through shared memory (n = 6144: 192 KB,
 // one CTA per SM) with a barrier per stage.  The mixed form had wavenumbers, 1/(sigma + alpha
@@ -336,7 +320,7 @@ template <bool MIXED, int NT>
 __device__ __forceinline__ void mr_pcg(const MrArgs& A, const MrPcgArgs& a) {
   __shared__ double red[NT / 32 + 1];
   __shared__ df slot[2 * (NT / 32)];
-  __shared__ float sums[2];
+  __shared__ df sums[2];
   int turn = 0;
   const int id = A.ids[blockIdx.x];
   const Inst1d I = A.insts[id];
@@ -494,7 +478,7 @@ __device__ __forceinline__ void mr_pcg(const MrArgs& A, const MrPcgArgs& a) {
     df* ux = a.ux ? static_cast<df*>(a.ux) + I.off : nullptr;
     const float sigf = (float)sigma, alf = (float)alpha, kf = (float)kunit;
     const float inv_nf = recip((float)n);
-    const df sigh(sigma), alh(alpha), inv_n = mr_recip(df(n));
+    const df sigh(sigma), alh(alpha), inv_n = recip(df(n));
     auto dinvf = [&](int m) {
       const float k = kf * (float)wave_index(m, n);
       return recip(fmaf(alf * k, k, sigf));
@@ -505,7 +489,7 @@ __device__ __forceinline__ void mr_pcg(const MrArgs& A, const MrPcgArgs& a) {
     auto term = [&](int m, cplx<df> v) {
       const df k = mr_k<df>(m, n, kuh);
       const double x = to_f64(v.x), y = to_f64(v.y);
-      const double q = (x * x + y * y) * to_f64(mr_recip(sigh + alh * (k * k)));
+      const double q = (x * x + y * y) * to_f64(recip(sigh + alh * (k * k)));
       return (m == 0 || m == h) ? q : q + q;
     };
     double bb = 0.0;
@@ -554,7 +538,8 @@ __device__ __forceinline__ void mr_pcg(const MrArgs& A, const MrPcgArgs& a) {
       }
       const double tin = a.rtol_inner > 0.0 ? a.rtol_inner
                                             : fmin(0.1, fmax(1e-6, 0.3 * a.rtol / ratio));
-      const float sc = (float)(1.0 / nr), tin2 = (float)(tin * tin);
+      const float sc = (float)(1.0 / nr);
+      const df tin2(tin * tin);
       // float32 PCG for G d = r / ||r||; p = A^{-1} r + beta p is formed with its transform's
       // input (beta = 0 first), and (G p)^ is taken from Y twice instead of being kept
       DfSum z0;
@@ -565,10 +550,11 @@ __device__ __forceinline__ void mr_pcg(const MrArgs& A, const MrPcgArgs& a) {
         Df[m] = Pf[m] = mk(0.0f, 0.0f);
         z0.add(wf(m) * ((r.x * r.x + r.y * r.y) * dinvf(m)));
       }
-      float rz = mr_sum<NT>(z0.s, slot, sums, turn), beta = 0.0f;
+      df rz = mr_sum<NT>(z0.s, slot, sums, turn);
+      float beta = 0.0f;
       const int it0 = iters;
       int st_in = SGN_OK;
-      while (rz > tin2) {
+      while ((rz - tin2).hi > 0.0f) {
         if (iters >= a.maxit) {
           st_in = SGN_ERR_NOT_CONVERGED;
           break;
@@ -584,12 +570,12 @@ __device__ __forceinline__ void mr_pcg(const MrArgs& A, const MrPcgArgs& a) {
           const cplx<float> p = Pf[m], g = mr_gv<float>(Yf, m, n, kf);
           ps.add(wf(m) * (p.x * g.x + p.y * g.y));
         }
-        const float pq = mr_sum<NT>(ps.s, slot, sums, turn);
-        if (!(pq > 0.0f) || !isfinite(pq)) {
+        const df pq = mr_sum<NT>(ps.s, slot, sums, turn);
+        if (!(pq.hi > 0.0f) || !isfinite(pq.hi)) {
           st_in = SGN_ERR_BREAKDOWN;
           break;
         }
-        const float al = rz / pq;
+        const float al = quot(rz, pq);
         DfSum zs;
         for (int m = threadIdx.x; m <= h; m += NT) {
           Df[m] = Df[m] + Pf[m] * al;
@@ -597,13 +583,13 @@ __device__ __forceinline__ void mr_pcg(const MrArgs& A, const MrPcgArgs& a) {
           Rf[m] = r;
           zs.add(wf(m) * ((r.x * r.x + r.y * r.y) * dinvf(m)));
         }
-        const float rzn = mr_sum<NT>(zs.s, slot, sums, turn);
+        const df rzn = mr_sum<NT>(zs.s, slot, sums, turn);
         ++iters;
-        if (!isfinite(rzn)) {
+        if (!isfinite(rzn.hi)) {
           st_in = SGN_ERR_BREAKDOWN;
           break;
         }
-        beta = rzn / rz;
+        beta = quot(rzn, rz);
         rz = rzn;
       }
       // a float32 breakdown after some progress keeps the correction (the next residual

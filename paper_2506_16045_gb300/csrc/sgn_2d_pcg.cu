@@ -348,12 +348,6 @@ __device__ __forceinline__ df ld_part(const double* p) {
   const float2 v = __ldcg(reinterpret_cast<const float2*>(p));
   return df(v.x, v.y);
 }
-// a / b rounded to float32 (the float32 quotient corrected by its double-float remainder)
-__device__ __forceinline__ float quot(df a, df b) {
-  const float q = a.hi / b.hi;
-  const df r = a - b * df(q, 0.0f);
-  return q + r.hi / b.hi;
-}
 
 // Sum of the per-unit partials (double-float) of every live instance (units [b U, b U + U)),
 // each summed by one warp in a fixed order; fin(b, total) runs on one lane per instance.
@@ -396,11 +390,25 @@ __device__ __forceinline__ void ainv(const IScal& s, float kx, float ky, cplx<fl
   z2 = (r2 - kr * (f * ky)) * s.isigf;
 }
 
-// Sum of the float partials of group g in double-float, stored to `out` by the group's
-// thread 0 (warp shuffles, then the group's four warp totals in order).
+// A thread's share of a dot product, float32 terms: in float32 on power-of-two grids, in
+// double-float on the others, whose sums were float64 as a kernel per iteration.
+template <bool MR>
+struct Part {
+  float v = 0.0f;
+  __device__ __forceinline__ void add(float a) { v += a; }
+  __device__ __forceinline__ df sum() const { return df(v, 0.0f); }
+};
+template <>
+struct Part<true> {
+  DfSum v;
+  __device__ __forceinline__ void add(float a) { v.add(a); }
+  __device__ __forceinline__ df sum() const { return v.s; }
+};
+
+// Sum of the threads' shares of group g in double-float, stored to `out` by the group's
+// thread 0 (warp shuffles, then the group's warp totals in order).
 template <int GT>
-__device__ __forceinline__ void group_part(float v, df* slot, double* out, int t, int g) {
-  df a(v, 0.0f);
+__device__ __forceinline__ void group_part(df a, df* slot, double* out, int t, int g) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     df b(__shfl_xor_sync(0xffffffffu, a.hi, o), __shfl_xor_sync(0xffffffffu, a.lo, o));
@@ -558,7 +566,7 @@ __device__ __forceinline__ void col_inverse(const PersistArgs2d& a, const PInst2
 
 // ---- R: C2R, Def:MatrixM pointwise with the p.Gp partial, R2C (row pair y0, group g) -----
 template <bool STG, int GT, bool MR>
-__device__ __forceinline__ float row_matvec(const PersistArgs2d& a, const PInst2d& I, int y0,
+__device__ __forceinline__ df row_matvec(const PersistArgs2d& a, const PInst2d& I, int y0,
                                             const PSmem& sm, int t, int g) {
   const int nx = a.nx, h = nx >> 1, S = pad_len(nx);
   const long long P = (long long)nx * a.ny;
@@ -603,7 +611,7 @@ __device__ __forceinline__ float row_matvec(const PersistArgs2d& a, const PInst2
   // 1 / (nx ny): exact for powers of two
   const float inv = MR ? recip((float)(nx * a.ny)) : __int_as_float((127 - a.lognx - a.logny) << 23);
   const float third = 1.0f / 3.0f;
-  float part = 0.0f;
+  Part<MR> part;
   for (int x0 = 0; x0 < nx; x0 += kRows * GT) {
     // eta, h_x, h_y of both rows for kRows points per thread, loaded before use
     float ev[kRows][2], hxv[kRows][2], hyv[kRows][2];
@@ -643,7 +651,7 @@ __device__ __forceinline__ float row_matvec(const PersistArgs2d& a, const PInst2
         const float w1 = c11 * p1 + c12 * p2 + c13 * d;
         const float w2 = c12 * p1 + c22 * p2 + c23 * d;
         const float q = c13 * p1 + c23 * p2 + c33 * d;
-        part += p1 * w1 + p2 * w2 + d * q;
+        part.add(p1 * w1 + p2 * w2 + d * q);
         w[r * S + pad(x)] = mk(w1, w2);
         if (r) w[2 * S + pad(x)].y = q; else w[2 * S + pad(x)].x = q;
       }
@@ -668,12 +676,12 @@ __device__ __forceinline__ float row_matvec(const PersistArgs2d& a, const PInst2
     __stcg(reinterpret_cast<float4*>(t_entry(I, a.ny, m, e0 + q)),
            make_float4(v0.x, v0.y, v1.x, v1.y));
   }
-  return part;
+  return part.sum();
 }
 
 // ---- C2: column FFT, G p, x and r updates, r.z partial (column c, group g) ---------------
 template <bool STG, int GT, bool MR>
-__device__ __forceinline__ float col_forward_update(const PersistArgs2d& a, const PInst2d& I,
+__device__ __forceinline__ df col_forward_update(const PersistArgs2d& a, const PInst2d& I,
                                                     const IScal& s, int c, const PSmem& sm,
                                                     int t, int g) {
   const int ny = a.ny, S = pad_len(ny), nx = a.nx;
@@ -702,7 +710,7 @@ __device__ __forceinline__ float col_forward_update(const PersistArgs2d& a, cons
   }
   gsync<GT>(g);
   const cplx<float>* o = pfft<GT, MR>(sm.A, sm.B, sm.ly, 3, S, false, sm.twy, t, g);
-  float part = 0.0f;
+  Part<MR> part;
   const float al = s.alpha;
   const float kx = kx_of(s, c, nx);
   const float wgt = (c == 0 || c == (nx >> 1)) ? 1.0f : 2.0f;
@@ -751,11 +759,11 @@ __device__ __forceinline__ float col_forward_update(const PersistArgs2d& a, cons
         stcg(R1 + y, nr2);
         cplx<float> z1, z2;
         ainv(s, kx, ky, nr1, nr2, z1, z2);
-        part += wgt * (nr1.x * z1.x + nr1.y * z1.y + nr2.x * z2.x + nr2.y * z2.y);
+        part.add(wgt * (nr1.x * z1.x + nr1.y * z1.y + nr2.x * z2.x + nr2.y * z2.y));
       }
     }
   }
-  return part;
+  return part.sum();
 }
 
 // STG: the staged form (a third shared buffer per group takes each unit's global inputs
@@ -866,7 +874,7 @@ __global__ void __launch_bounds__(kPNT, 1) k2_pcg_persist(const __grid_constant_
     for (int u = slot0; u < B * RU; u += nslots) {
       const int b = u / RU, pr = u - b * RU;
       if (S[b].done) continue;
-      const float part = row_matvec<STG, GT, MR>(a, a.inst[b], 2 * pr, sm, t, g);
+      const df part = row_matvec<STG, GT, MR>(a, a.inst[b], 2 * pr, sm, t, g);
       group_part<GT>(part, slot, a.parts + (long long)b * RU + pr, t, g);
     }
     if ((stop = grid_barrier(a.bar, a.err, target, &s_stop))) break;
@@ -884,7 +892,7 @@ __global__ void __launch_bounds__(kPNT, 1) k2_pcg_persist(const __grid_constant_
     for (int u = slot0; u < B * CU; u += nslots) {
       const int b = u / CU, c = u - b * CU;
       if (S[b].done) continue;
-      const float part = col_forward_update<STG, GT, MR>(a, a.inst[b], S[b], c, sm, t, g);
+      const df part = col_forward_update<STG, GT, MR>(a, a.inst[b], S[b], c, sm, t, g);
       group_part<GT>(part, slot, parts2 + (long long)b * CU + c, t, g);
     }
     if ((stop = grid_barrier(a.bar, a.err, target, &s_stop))) break;

@@ -129,6 +129,28 @@ __device__ __forceinline__ double half(double a) { return a * 0.5; }
 // reciprocal in the working precision (float: correctly rounded, no float64 involved)
 __device__ __forceinline__ float recip(float a) { return __frcp_rn(a); }
 __device__ __forceinline__ double recip(double a) { return 1.0 / a; }
+// in double-float: a float32 reciprocal and one residual
+__device__ __forceinline__ df recip(df a) {
+  const float r = __frcp_rn(a.hi);
+  const float e = fmaf(-a.lo, r, fmaf(-a.hi, r, 1.0f));
+  const float c = __fmul_rn(r, e), h = __fadd_rn(r, c);
+  return df(h, __fsub_rn(c, __fsub_rn(h, r)));
+}
+// a / b rounded to float32 (the float32 quotient corrected by its double-float remainder)
+__device__ __forceinline__ float quot(df a, df b) {
+  const float q = a.hi / b.hi;
+  const df r = a - b * df(q, 0.0f);
+  return q + r.hi / b.hi;
+}
+// A sum of float32 terms kept in double-float.
+struct DfSum {
+  df s{0.0f, 0.0f};
+  __device__ __forceinline__ void add(float v) {
+    const float h = __fadd_rn(s.hi, v), bb = __fsub_rn(h, s.hi);
+    const float e = __fadd_rn(__fsub_rn(s.hi, __fsub_rn(h, bb)), __fsub_rn(v, bb));
+    s = df(h, __fadd_rn(s.lo, e));
+  }
+};
 __device__ __forceinline__ double to_f64(double v) { return v; }
 __device__ __forceinline__ double to_f64(float v) { return (double)v; }
 __device__ __forceinline__ double to_f64(df v) { return f64_of(v.hi) + f64_of(v.lo); }

@@ -179,15 +179,6 @@ __device__ __forceinline__ double pack_df(df v) {
 __device__ __forceinline__ df unpack_df(double d) {
   return df(__int_as_float(__double2loint(d)), __int_as_float(__double2hiint(d)));
 }
-// 1/a, a quotient and 1/a's use in double-float: one float32 reciprocal and a residual
-__device__ __forceinline__ df recip_df(df a) {
-  const float r = __frcp_rn(a.hi);
-  const float e = fmaf(-a.lo, r, fmaf(-a.hi, r, 1.0f));
-  const float c = __fmul_rn(r, e), h = __fadd_rn(r, c);
-  return df(h, __fsub_rn(c, __fsub_rn(h, r)));
-}
-__device__ __forceinline__ double recip_t(double a) { return 1.0 / a; }
-__device__ __forceinline__ df recip_t(df a) { return recip_df(a); }
 
 // ---- solve, mixed precision ---------------------------------------------------------------
 struct MixedScalars {
@@ -1049,7 +1040,7 @@ __global__ void SGN_SPLIT_BOUNDS(PL, 2)
     A.res1[hs + m] = mk(to_f64(r.x), to_f64(r.y));
     if (A.solve) {
       const cplx<double> p = A.res0[hs + m];
-      const T is = recip_t(sym);
+      const T is = recip(sym);
       z[q] = mk((c1 * r.x + c0 * num<T>(p.x)) * is, (c1 * r.y + c0 * num<T>(p.y)) * is);
       if (ts && q == 0) z[q].y = zero;
     }
@@ -1057,7 +1048,7 @@ __global__ void SGN_SPLIT_BOUNDS(PL, 2)
   if (ts) {
     const T r = uN * sigma - v[NYQ].x;
     A.res1[hs + h] = mk(to_f64(r), 0.0);
-    if (A.solve) zN = (c1 * r + c0 * num<T>(A.res0[hs + h].x)) * recip_t(sigma);
+    if (A.solve) zN = (c1 * r + c0 * num<T>(A.res0[hs + h].x)) * recip(sigma);
   }
   if (A.solve) {                         // uniform over the grid
 #pragma unroll
