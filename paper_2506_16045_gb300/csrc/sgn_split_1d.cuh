@@ -180,12 +180,23 @@ __device__ __forceinline__ df unpack_df(double d) {
   return df(__int_as_float(__double2loint(d)), __int_as_float(__double2hiint(d)));
 }
 
+// exact, subnormal parts included
+__device__ __forceinline__ double f64(df v) { return (double)v.hi + (double)v.lo; }
+// the root of a >= 0, and a / b rounded twice (48 bits)
+__device__ __forceinline__ df root(df a) {
+  const float r = sqrtf(a.hi);
+  return df(r, r > 0.0f ? 0.5f * (fmaf(-r, r, a.hi) + a.lo) / r : 0.0f);
+}
+__device__ __forceinline__ df quot_df(df a, df b) {
+  const float q = a.hi / b.hi;
+  return df(q, (a - b * df(q, 0.0f)).hi / b.hi);
+}
+
 // ---- solve, mixed precision ---------------------------------------------------------------
 struct MixedScalars {
-  double bb, lim, rz64;     // b.A^{-1}b, rtol^2 times it, r.A^{-1}r: their quotients and squares
-                            // may leave the float32 range
-  df unscale;               // ||r||_{A^{-1}}
-  float ibn, scale, tin2;   // 1 / ||b||_{A^{-1}}, 1 / ||r||_{A^{-1}}, (inner tolerance)^2
+  df bb, rz2, unscale;      // b.A^{-1}b; r.A^{-1}r and its root
+  float tol;                // rtol ||b||_{A^{-1}}
+  float scale, tin2;        // 1 / ||r||_{A^{-1}}; (inner tolerance)^2
   int go, status;
   float rz, alpha, beta;    // inner solve
   int state;                // 0 iterate, 1 converged, 2 breakdown, 3 iteration cap
@@ -204,7 +215,9 @@ __global__ void SGN_SPLIT_BOUNDS(PL, 3)
     k_solve_mixed(const __grid_constant__ PcgArgs A, int first, int lcl) {
   using SL = Slot<PL>;
   constexpr int n = PL::n, E = PL::E, RP = PL::RP, h = n / 2, PS = n / E, NYQ = PL::NYQ;
-  extern __shared__ __align__(16) unsigned char smem[];
+  // 128: the partners' stores travel by 128-byte lines (n = 4096, 24 AB4 steps: 5.65 ms, 5.71
+  // with the buffers 32 bytes off)
+  extern __shared__ __align__(128) unsigned char smem[];
   __shared__ Setup st;
   __shared__ MixedScalars sc;
   __shared__ Extrema exs[PL::W];
@@ -318,21 +331,20 @@ __global__ void SGN_SPLIT_BOUNDS(PL, 3)
       bb += y.x.hi * y.x.hi * dN;
     }
     reduce<PL>(df(bb, 0.0f), slots, hb, g, [&](df s) {
-      sc.bb = (double)s.hi + (double)s.lo;
-      sc.lim = A.rtol * A.rtol * sc.bb;
-      sc.ibn = recip(sqrtf(s.hi));
+      sc.bb = s;
+      sc.tol = (float)A.rtol * sqrtf(s.hi);
     });
   }
-  const double bb = sc.bb;
+  const float bb = sc.bb.hi;
   const df zero(0.0f, 0.0f);
-  if (!(bb > 0.0)) {                     // x = 0, and its derivative for the right-hand side
+  if (!(bb > 0.0f)) {                    // x = 0, and its derivative for the right-hand side
 #pragma unroll
     for (int e = 0; e < E; ++e) {
       x[g.pt + e * PS] = 0.0;
       if (ux) ux[g.pt + e * PS] = zero;
     }
     if (ts) {
-      st.R.status = bb == 0.0 ? SGN_OK : SGN_ERR_BREAKDOWN;
+      st.R.status = bb == 0.0f ? SGN_OK : SGN_ERR_BREAKDOWN;
       A.rec[id] = st.R;
     }
     if (lcl) cluster_sync();
@@ -342,7 +354,6 @@ __global__ void SGN_SPLIT_BOUNDS(PL, 3)
   const df inv_n(1.0f / (float)n, 0.0f);                              // exact
   const float inv_nf = 1.0f / (float)n;
   const df one(1.0f, 0.0f);
-  const float rtolf = (float)A.rtol;
   int iters = 0, status = SGN_OK, refinements = 0;
   for (;;) {
     // ---- double-float residual r^ = b^ - (G x)^, keeping the real-space x on the way
@@ -389,31 +400,31 @@ __global__ void SGN_SPLIT_BOUNDS(PL, 3)
         rN = mk(rr.hi + rr.lo, 0.0f);
         rz += rN.x * rN.x * dN;
       }
-      // one thread decides the pass: converged (r.A^{-1}r against rtol^2 b.A^{-1}b in float64),
-      // out of budget, or the next inner solve
+      // one thread decides the pass: converged (r.A^{-1}r against rtol^2 b.A^{-1}b, which may
+      // leave the float32 range: in float64 unless the first is clearly above), out of budget,
+      // or the next inner solve
       reduce<PL>(df(rz, 0.0f), slots, hb, g, [&](df s) {
-        const double rzd = (double)s.hi + (double)s.lo;
-        sc.rz64 = rzd;
+        sc.rz2 = s;
         sc.go = 0;
         sc.status = status;
-        if (rzd <= sc.lim || status != SGN_OK) return;
+        if ((!(s.hi > 2.0f * (sc.tol * sc.tol)) && f64(s) <= A.rtol * A.rtol * f64(sc.bb)) ||
+            status != SGN_OK)
+          return;
         if (refinements >= A.max_refine || iters >= A.maxit) {
           sc.status = SGN_ERR_NOT_CONVERGED;
           return;
         }
-        // the root of s in double-float: a float32 root and its residual
-        const float nr = sqrtf(s.hi), dn = 0.5f * (fmaf(-nr, nr, s.hi) + s.lo) / nr;
-        const float tin = fminf(0.1f, fmaxf(1e-6f, 0.3f * rtolf / (nr * sc.ibn)));
+        const df nr = root(s);
+        const float in = recip(nr.hi), tin = fminf(0.1f, fmaxf(1e-6f, 0.3f * (in * sc.tol)));
         sc.tin2 = A.rtol_inner > 0.0 ? (float)(A.rtol_inner * A.rtol_inner) : tin * tin;
-        sc.unscale = df(nr, dn);
-        sc.scale = recip(nr);
+        sc.unscale = nr;
+        sc.scale = in;
         sc.go = 1;
       });
     }
     status = sc.status;
     if (!sc.go) break;
     const float scale = sc.scale, tin2 = sc.tin2;
-    const df unscale = sc.unscale;
 
     // ---- float32 PCG for G d = r / ||r||
     const int it_before = iters;
@@ -534,6 +545,7 @@ __global__ void SGN_SPLIT_BOUNDS(PL, 3)
     // keep the correction and let the next refinement pass decide.
     if (st_in == SGN_ERR_BREAKDOWN && iters == it_before) status = SGN_ERR_BREAKDOWN;
     ++refinements;
+    const df unscale = sc.unscale;
 #pragma unroll
     for (int q = 0; q < RP; ++q) {
       const int m = g.mode(SL::b(q), SL::s(q));
@@ -549,7 +561,7 @@ __global__ void SGN_SPLIT_BOUNDS(PL, 3)
   }
   if (ts) {
     SolveRec R = st.R;
-    R.ratio = sqrt(sc.rz64 / sc.bb);
+    R.ratio = f64(quot_df(root(sc.rz2), root(sc.bb)));
     R.refinements = refinements;
     R.iters = iters;
     R.status = status;
