@@ -21,7 +21,9 @@
 // arrays, which only the server's streams use, come from a pool that keeps at most kPoolBytes,
 // and the layouts of finished 2d requests are kept, up to kIdleBytes of them, for later
 // requests on the same grid (a 2d layout is 11 allocations and a solve graph: 0.9 ms to make
-// and to destroy at 512 x 512, against 0.5 ms for a solve).
+// and to destroy at 512 x 512, against 0.5 ms for a solve).  What is kept is given back
+// (give_back) when an allocation of the server fails, which is then tried again, and when the
+// server has had nothing to do for kIdleSeconds.
 // RK4 is a one-step method and every instance of a batched launch is computed by its own
 // CTAs, and a 2d or multistep request runs on its own layout and state, so a request's
 // result does not depend on which requests ran beside it.
@@ -55,6 +57,7 @@ constexpr int kSolveLanes = 2;       // high-priority lanes of the 1d solve grou
 constexpr size_t kReapBytes = (size_t)2 << 30;   // deferred frees forced past this many bytes
 constexpr size_t kPoolBytes = (size_t)1 << 30;   // free memory that the requests' pool keeps
 constexpr size_t kIdleBytes = (size_t)2 << 30;   // 2d layouts kept for later requests
+constexpr double kIdleSeconds = 5.0;             // without work: the kept memory is given back
 
 struct Req {
   uint64_t ticket = 0;
@@ -152,6 +155,9 @@ struct sgn_server {
   };
   std::deque<Idle> idle;
   size_t idle_bytes = 0, idle_cap = 0;
+  // submissions that ran out of memory ask the worker to give back what it keeps
+  std::condition_variable given;
+  uint64_t short_asked = 0, short_done = 0;
   // cached batch objects for 1d RK4 runs
   std::vector<uint64_t> run_members;
   bool batch_busy = false;
@@ -186,8 +192,7 @@ void drop_idle(sgn_server* S, size_t keep) {
   }
 }
 
-// The layout of a 2d request: one kept from an earlier request on the same grid, or a new one
-// (when memory runs out, after the kept ones have been given back).
+// The layout of a 2d request: one kept from an earlier request on the same grid, or a new one.
 sgn_status take_layout(sgn_server* S, const sgn_grid& g, sgn_layout** out) {
   for (auto it = S->idle.begin(); it != S->idle.end(); ++it)
     if (same_grid(it->g, g)) {
@@ -196,13 +201,7 @@ sgn_status take_layout(sgn_server* S, const sgn_grid& g, sgn_layout** out) {
       S->idle.erase(it);
       return SGN_OK;
     }
-  sgn_status e = sgn_layout_create(S->ctx, 1, &g, out);
-  if (e && !S->idle.empty()) {
-    drop_idle(S, 0);
-    cudaGetLastError();
-    e = sgn_layout_create(S->ctx, 1, &g, out);
-  }
-  return e;
+  return sgn_layout_create(S->ctx, 1, &g, out);
 }
 
 // Places device arrays of the given numbers of doubles in one block (256-byte aligned): its
@@ -280,6 +279,36 @@ void reap(sgn_server* S, bool force) {
   S->reap_bytes = 0;
 }
 
+// Gives back the memory kept for later requests (the worker only).  The frees may run beside
+// another thread's capture, which they do not touch: relaxed mode, or they would fail and end
+// that capture.
+void give_back(sgn_server* S) {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  reap(S, true);
+  drop_idle(S, 0);
+  cudaStreamSynchronize(S->copy);        // the pool's blocks are freed in its order
+  cudaMemPoolTrimTo(S->pool, 0);
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  cudaGetLastError();
+}
+
+// f(), and once more after give_back when it ran out of memory
+template <typename F>
+sgn_status with_memory(sgn_server* S, F f) {
+  sgn_status e = f();
+  if (e != SGN_ERR_NOMEM) return e;
+  give_back(S);
+  return f();
+}
+
+sgn_status alloc_on(void** p, size_t bytes, cudaStream_t s) {
+  if (cudaMallocAsync(p, bytes, s) == cudaSuccess) return SGN_OK;
+  cudaGetLastError();
+  *p = nullptr;
+  return SGN_ERR_NOMEM;
+}
+
 sgn_layout* one_layout(sgn_server* S, const sgn_grid& g) {
   auto key = std::make_pair(g.nx, g.Lx);
   auto it = S->one1d.find(key);
@@ -338,7 +367,8 @@ void give_info(sgn_server* S, int at, int n) {
   for (int k = 0; k < n; ++k) S->info_used[at + k] = 0;
 }
 
-// Initialise an admitted request on the device (the set-up stream); records r->ready.
+// Initialise an admitted request on the device (the set-up stream); records r->ready.  After
+// SGN_ERR_NOMEM it may be called again.
 sgn_status start(sgn_server* S, Req* r) {
   const sgn_stream s = S->stream;
   sgn_status e = SGN_OK;
@@ -355,13 +385,14 @@ sgn_status start(sgn_server* S, Req* r) {
     e = sgn_spectral_grad(S->ctx, lay, r->h, r->gh, s);
     if (!e) e = sgn_apply_operator(S->ctx, lay, r->eta, r->gh, r->u, r->U, s);
   } else if (r->q.kind == SGN_REQ_RUN) {
-    e = r->d == 2 ? take_layout(S, r->q.grid, &r->lay)
-                  : sgn_layout_create(S->ctx, 1, &r->q.grid, &r->lay);
-    if (!e) e = sgn_state_create(S->ctx, r->lay, r->eta, r->U, r->u, r->h, r->gh, &r->st);
+    if (!r->lay)
+      e = r->d == 2 ? take_layout(S, r->q.grid, &r->lay)
+                    : sgn_layout_create(S->ctx, 1, &r->q.grid, &r->lay);
+    if (!e && !r->st) e = sgn_state_create(S->ctx, r->lay, r->eta, r->U, r->u, r->h, r->gh, &r->st);
     if (!e) e = sgn_state_init(r->st, s);
   } else if (r->d == 2) {
     // SOLVE: grad h now (2d solves also get their layout here)
-    e = take_layout(S, r->q.grid, &r->lay);
+    if (!r->lay) e = take_layout(S, r->q.grid, &r->lay);
     if (!e) e = sgn_spectral_grad(S->ctx, r->lay, r->h, r->gh, s);
   } else {
     sgn_layout* lay = one_layout(S, r->q.grid);
@@ -403,7 +434,9 @@ void issue_solves_1d(sgn_server* S, std::vector<Req*>& v) {
   S->next_solve_lane = (S->next_solve_lane + 1) % kSolveLanes;
   std::vector<sgn_grid> grids;
   for (Req* r : v) grids.push_back(r->q.grid);
-  sgn_status e = sgn_layout_create(S->ctx, (int)v.size(), grids.data(), &J->lay);
+  sgn_status e = with_memory(S, [&] {
+    return sgn_layout_create(S->ctx, (int)v.size(), grids.data(), &J->lay);
+  });
   if (!e && (J->info_at = take_info(S, (int)v.size())) < 0) e = SGN_ERR_NOMEM;
   J->info_n = (int)v.size();
   double* pk = nullptr;
@@ -413,11 +446,9 @@ void issue_solves_1d(sgn_server* S, std::vector<Req*>& v) {
     sgn_layout_offsets(J->lay, off.data());
     P = off.back();
     // the packed arrays of the group live with its layout (stream-ordered allocation)
-    if (cudaMallocAsync(reinterpret_cast<void**>(&pk), sizeof(double) * 4 * (size_t)P, J->s) !=
-        cudaSuccess) {
-      cudaGetLastError();
-      e = SGN_ERR_NOMEM;
-    }
+    e = with_memory(S, [&] {
+      return alloc_on(reinterpret_cast<void**>(&pk), sizeof(double) * 4 * (size_t)P, J->s);
+    });
   }
   if (!e) {
     wait_ready(J->s, v);
@@ -464,24 +495,25 @@ void issue_run_batch(sgn_server* S, std::vector<Req*>& v) {
     S->run_members.clear();
     std::vector<sgn_grid> grids;
     for (Req* r : v) grids.push_back(r->q.grid);
-    e = sgn_layout_create(S->ctx, (int)v.size(), grids.data(), &S->run_lay);
+    e = with_memory(S, [&] {
+      return sgn_layout_create(S->ctx, (int)v.size(), grids.data(), &S->run_lay);
+    });
     long long P = e ? 0 : sgn_layout_points(S->run_lay);
     if (!e && P > S->pk_cap) {
       // the packed buffer may still be read by an earlier chunk on this lane: free it in order
       if (S->pk) cudaFreeAsync(S->pk, J->s);
       S->pk = nullptr;
       S->pk_cap = 0;
-      if (cudaMallocAsync(reinterpret_cast<void**>(&S->pk), sizeof(double) * 5 * (size_t)P,
-                          J->s) != cudaSuccess) {
-        cudaGetLastError();
-        e = SGN_ERR_NOMEM;
-      } else {
-        S->pk_cap = P;
-      }
+      e = with_memory(S, [&] {
+        return alloc_on(reinterpret_cast<void**>(&S->pk), sizeof(double) * 5 * (size_t)P, J->s);
+      });
+      if (!e) S->pk_cap = P;
     }
     if (!e)
-      e = sgn_state_create(S->ctx, S->run_lay, S->pk, S->pk + P, S->pk + 2 * P, S->pk + 3 * P,
-                           S->pk + 4 * P, &S->run_st);
+      e = with_memory(S, [&] {
+        return sgn_state_create(S->ctx, S->run_lay, S->pk, S->pk + P, S->pk + 2 * P,
+                                S->pk + 3 * P, S->pk + 4 * P, &S->run_st);
+      });
     if (!e) S->run_members = members;
   }
   if (!e) {
@@ -639,10 +671,15 @@ int poll_jobs(sgn_server* S) {
 
 void worker_main(sgn_server* S) {
   cudaSetDevice(S->device);
+  double busy_at = now_s();              // when there was last something to do
+  bool keeps = false;                    // since then nothing has been given back
   for (;;) {
     std::vector<Req*> admit_now;
+    uint64_t asked = 0, answered = 0;
     {
       std::unique_lock<std::mutex> lk(S->mu);
+      asked = S->short_asked;
+      answered = S->short_done;
       if (S->stop && S->pending.empty() && S->active.empty() && S->inflight.empty()) break;
       for (auto it = S->pending.begin(); it != S->pending.end();) {
         Req* r = *it;
@@ -657,10 +694,16 @@ void worker_main(sgn_server* S) {
         }
       }
     }
+    if (asked != answered) {
+      give_back(S);
+      std::lock_guard<std::mutex> lk(S->mu);
+      S->short_done = asked;
+      S->given.notify_all();
+    }
     if (!admit_now.empty())              // the kept layouts stay within the budget too
       drop_idle(S, S->budget > S->used ? S->budget - S->used : 0);
     for (Req* r : admit_now) {
-      sgn_status e = start(S, r);
+      sgn_status e = with_memory(S, [&] { return start(S, r); });
       if (e) {
         finish(S, r, e);
         continue;
@@ -734,9 +777,18 @@ void worker_main(sgn_server* S) {
       ++issued;
     }
     reap(S, S->reap_bytes >= kReapBytes);
+    if (!admit_now.empty() || !act.empty() || completed) {
+      busy_at = now_s();
+      keeps = true;
+    } else if (keeps && now_s() - busy_at > kIdleSeconds) {
+      give_back(S);
+      keeps = false;
+    }
     if (!completed && !issued) {
       std::unique_lock<std::mutex> lk(S->mu);
-      S->cv.wait_for(lk, std::chrono::microseconds(50), [&] { return S->stop || !S->pending.empty(); });
+      S->cv.wait_for(lk, std::chrono::microseconds(50), [&] {
+        return S->stop || !S->pending.empty() || S->short_asked != S->short_done;
+      });
     }
   }
   reap(S, true);
@@ -806,6 +858,14 @@ extern "C" sgn_status sgn_server_create(sgn_ctx* ctx, double budget_fraction, sg
   return SGN_OK;
 }
 
+// Has the worker give back the memory it keeps, and waits until it has.
+static void ask_back(sgn_server* S) {
+  std::unique_lock<std::mutex> lk(S->mu);
+  const uint64_t k = ++S->short_asked;
+  S->cv.notify_one();
+  S->given.wait(lk, [&] { return S->stop || S->short_done >= k; });
+}
+
 // A submission that failed.
 static void refuse(sgn_server* S, Req* r) {
   if (r->work_block) cudaFreeAsync(r->work_block, S->copy);
@@ -853,13 +913,21 @@ extern "C" sgn_status sgn_batch_submit(sgn_server* S, const sgn_request* q, uint
   const Arrays res = {{&r->eta, N}, {&r->u, V}, {&r->U, V}};
   const Arrays work = {{&r->h, N}, {&r->gh, V}, {&r->b, q->kind == SGN_REQ_SOLVE ? V : 0},
                        {&r->hist, is_batched_run(r) ? 2 * N : 0}};
-  if (cudaMalloc(&r->res_block, place(nullptr, res)) != cudaSuccess ||
-      cudaMallocFromPoolAsync(&r->work_block, place(nullptr, work), S->pool, S->copy) !=
-          cudaSuccess) {
+  auto alloc = [&] {
+    if (!r->res_block && cudaMalloc(&r->res_block, place(nullptr, res)) != cudaSuccess)
+      r->res_block = nullptr;
+    if (r->res_block && cudaMallocFromPoolAsync(&r->work_block, place(nullptr, work), S->pool,
+                                                S->copy) != cudaSuccess)
+      r->work_block = nullptr;
     cudaGetLastError();
-    r->work_block = nullptr;
-    refuse(S, r);
-    return SGN_ERR_NOMEM;
+    return r->work_block != nullptr;
+  };
+  if (!alloc()) {
+    ask_back(S);
+    if (!alloc()) {
+      refuse(S, r);
+      return SGN_ERR_NOMEM;
+    }
   }
   place(r->res_block, res);
   place(r->work_block, work);
