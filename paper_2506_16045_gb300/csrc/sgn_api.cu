@@ -697,6 +697,12 @@ extern "C" sgn_status sgn_layout_create(sgn_ctx* ctx, int count, const sgn_grid*
   return SGN_OK;
 }
 
+// Internal (serving): building a 2d layout's solve graph failed once, so its solves are
+// host-driven.
+namespace sgn {
+bool layout_graph_refused(const sgn_layout* lay) { return lay->dim == 2 && lay->l2.solve_graph_off; }
+}  // namespace sgn
+
 extern "C" void sgn_layout_destroy(sgn_layout* lay) {
   if (!lay) return;
   DeviceGuard g(lay->device);

@@ -45,6 +45,7 @@
 #include "sgn_internal.h"
 
 namespace sgn {
+bool layout_graph_refused(const sgn_layout* lay);
 sgn_status state_attach(sgn_state* st, cudaStream_t s);
 double* state_rk4_prev(sgn_state* st);
 double* state_rk4_last(sgn_state* st);
@@ -220,7 +221,8 @@ size_t place(void* block, Arrays v) {
 // When the server's streams have finished with the request.
 void free_req_work(sgn_server* S, Req* r) {
   if (r->st) sgn_state_free(r->st);
-  if (r->lay && r->d == 2 && r->footprint <= S->idle_cap) {
+  // a layout whose solve graph could not be built solves host-driven from then on: not kept
+  if (r->lay && r->d == 2 && r->footprint <= S->idle_cap && !sgn::layout_graph_refused(r->lay)) {
     S->idle.push_back({r->q.grid, r->lay, r->footprint});
     S->idle_bytes += r->footprint;
     drop_idle(S, S->idle_cap);

@@ -322,6 +322,14 @@ int main(int argc, char** argv) {
     limit_bytes = used() + 1000000;
     layout_bytes = 40000;
     st = serve(S, SGN_REQ_SOLVE, 2, 64, 5.0, SGN_SCHEME_RK4, &it);
+  } else if (what == "graph") {              // a solve graph that could not be built, once
+    refuse_graph = true;
+    if (serve(S, SGN_REQ_SOLVE, 2, 64, 10.0, SGN_SCHEME_RK4, &it) || it != 2) return 3;
+    std::this_thread::sleep_for(std::chrono::milliseconds(100));
+    st = serve(S, SGN_REQ_SOLVE, 2, 64, 10.0, SGN_SCHEME_RK4, &it);
+    const int n = layouts;                   // and the next request takes the kept layout
+    std::this_thread::sleep_for(std::chrono::milliseconds(100));
+    if (serve(S, SGN_REQ_SOLVE, 2, 64, 10.0, SGN_SCHEME_RK4, nullptr) || layouts != n) st = 6;
   } else if (what == "idle") {               // nothing to do: the memory goes back by itself
     const size_t before = used();
     fill();

@@ -36,3 +36,8 @@ def test_what_does_not_fit_is_still_refused(fake):
 def test_an_idle_server_gives_its_memory_back(fake):
     out = fake("idle")
     assert out[0] == "status 0 iters 0" and out[1] == "left 0 blocks"
+
+
+def test_a_layout_without_a_solve_graph_is_not_kept(fake):
+    """Its solves are host-driven (report 2 here): later requests must not inherit that."""
+    assert fake("graph")[0] == "status 0 iters 1"
