@@ -64,29 +64,17 @@ extern template cudaError_t split_linimp_launch<14>(const sp::LinArgs&, int, int
 extern template cudaError_t split_field_launch<14>(const sp::FieldArgs&, int, int, int,
                                                    cudaStream_t);
 
-// log2 of the CTAs per instance of class l.  At least 2048 points per CTA stay together; from
-// there the classes are halved, the one with the largest share per CTA first, while every CTA
-// still has an SM of its own (one instance: up to 8 CTAs).  Splitting further than the SMs
-// would only add exchanges: two CTAs on an SM share its issue slots and its float64 pipe.
-int split_lcl(const Layout1d& lay, int l) {
-  int lcl[16], total = 0;
-  for (int c = 0; c < 16; ++c) {
-    const int num = lay.class_end[c] - lay.class_begin[c];
-    lcl[c] = c > 11 ? c - 11 : 0;
-    total += num << lcl[c];
+// log2 of the CTAs per instance that class l's split kernel takes beside the layout's other
+// classes; ctas(c) is 2 where class c runs on the two-CTA kernels.
+static_assert(kSplitMinLog == kSplitLog1d && kSplitMaxLog == kMaxLog1d, "the split classes");
+template <typename Ctas>
+static int split_lcl(const Layout1d& lay, int l, bool mixed, Ctas ctas) {
+  int num[kSplitClasses], two[kSplitClasses], lcl[kSplitClasses];
+  for (int c = 0; c < kSplitClasses; ++c) {
+    num[c] = lay.class_end[c] - lay.class_begin[c];
+    two[c] = c >= kClusterLog1d && c <= kSmemLog1d && ctas(c) == 2 ? 2 : 1;
   }
-  for (;;) {
-    int best = -1;
-    for (int c = kSplitLog1d; c <= kMaxLog1d; ++c)
-      if (lay.class_end[c] > lay.class_begin[c] && lcl[c] < 3 &&
-          (best < 0 || c - lcl[c] >= best - lcl[best]))
-        best = c;
-    if (best < 0) break;
-    const int num = lay.class_end[best] - lay.class_begin[best];
-    if (total + (num << lcl[best]) > kSMs) break;
-    total += num << lcl[best];
-    lcl[best] += 1;
-  }
+  split_plan(num, two, mixed, kSMs, lcl);
   return lcl[l];
 }
 
@@ -126,7 +114,10 @@ cudaError_t launch_form(const Layout1d& lay, const Args& a, int first, int num, 
   if constexpr (LG >= kSplitLog1d) {
     if constexpr (LG >= kClusterLog1d && LG <= kSmemLog1d)
       if (K::ctas(lay, LG) == 2) return K::template go<LG, 2>(a, first, num, s);
-    return K::template split<LG>(a, first, num, split_lcl(lay, LG), s);
+    return K::template split<LG>(a, first, num,
+                                 split_lcl(lay, LG, a.precision == SGN_PREC_MIXED,
+                                           [&](int c) { return K::ctas(lay, c); }),
+                                 s);
   } else {
     return K::template go<LG, 1>(a, first, num, s);
   }
@@ -263,7 +254,7 @@ cudaError_t launch_linimp_split(const Layout1d& lay, int l, int first, int num, 
   a.ux = ux_out;
   a.precision = precision;
   a.solve = solve;
-  const int lcl = split_lcl(lay, l);
+  const int lcl = split_lcl(lay, l, precision == SGN_PREC_MIXED, [](int) { return 1; });
   switch (l) {
     case 8: return split_linimp_launch<8>(a, first, num, lcl, s);
     case 9: return split_linimp_launch<9>(a, first, num, lcl, s);
@@ -281,7 +272,7 @@ cudaError_t launch_field_split(const Layout1d& lay, int l, int first, int num, c
                                cudaStream_t s) {
   const sp::FieldArgs a{lay.d_inst, lay.d_ids, static_cast<const cplx<double>*>(tw64), f, eta, hx,
                         out};
-  const int lcl = split_lcl(lay, l);
+  const int lcl = split_lcl(lay, l, false, [](int) { return 1; });
   switch (l) {
     case 8: return split_field_launch<8>(a, first, num, lcl, s);
     case 9: return split_field_launch<9>(a, first, num, lcl, s);

@@ -85,9 +85,6 @@ struct Layout1d {
   cudaEvent_t join[16] = {nullptr};
 };
 
-// log2 of the CTAs per instance that class l's split kernels take (sgn_1d_launch.cu)
-int split_lcl(const Layout1d& lay, int l);
-
 // Launchers (all asynchronous on `stream`; return cudaError_t of the launch).
 cudaError_t twiddles_init(void* tw64, void* tw32, cudaStream_t s);
 

@@ -24,11 +24,10 @@ namespace sp {
 
 using d1::kPi;
 
-// Elements per thread: float64 2 up to n = 1024 and 4 above, mixed 4
 template <int L>
-using Plan64 = Plan<L, (L <= 10 ? 2 : 4)>;
+using Plan64 = Plan<L, 1 << split_log_e(L, false)>;
 template <int L>
-using PlanMx = Plan<L, 4>;
+using PlanMx = Plan<L, 1 << split_log_e(L, true)>;
 // CTAs of 256 threads per SM that the registers leave room for.  3 (80 registers) for the mixed
 // solve and the double-float right-hand side: a batch that fills the GPU hides more latency
 // (ensemble of 256, 4 RK4 steps: 11.15 ms with 2, 10.25 with 3, 10.50 with 4, which spills),
@@ -1146,9 +1145,11 @@ __global__ void SGN_SPLIT_BOUNDS(PL, 2)
 }
 
 // ---- launches -----------------------------------------------------------------------------
-template <typename K, typename Args>
-cudaError_t launch_split(K kernel, int num, int lcl, int threads, size_t smem, cudaStream_t s,
-                         const Args& a, int first) {
+template <typename PL, typename K, typename Args>
+cudaError_t launch_split(K kernel, int num, int lcl, size_t smem, cudaStream_t s, const Args& a,
+                         int first) {
+  if (lcl < PL::kMinLcl || lcl > PL::kMaxLcl) return cudaErrorInvalidConfiguration;
+  const int threads = 1 << (PL::LNTA - lcl);
   cudaError_t e = raise_smem(kernel, smem);
   if (e) return e;
   cudaLaunchConfig_t cfg = {};
@@ -1166,31 +1167,25 @@ cudaError_t launch_split(K kernel, int num, int lcl, int threads, size_t smem, c
   return cudaLaunchKernelEx(&cfg, kernel, a, first, lcl);
 }
 
-inline int clamp_lcl(int lcl, int lo, int hi) { return lcl < lo ? lo : (lcl > hi ? hi : lcl); }
-
 }  // namespace sp
 
-// lcl: log2 of the CTAs per instance that the load asks for, brought into the kernel's range
+// lcl: log2 of the CTAs per instance (split_lcl)
 template <int L>
 cudaError_t split_pcg_launch(const PcgArgs& a, int first, int num, int lcl, cudaStream_t s) {
   if (a.precision == SGN_PREC_MIXED) {
     using PL = sp::PlanMx<L>;
-    lcl = sp::clamp_lcl(lcl, PL::kMinLcl, PL::kMaxLcl);
-    return sp::launch_split(sp::k_solve_mixed<PL>, num, lcl, 1 << (PL::LNTA - lcl),
-                            sp::SmemMixed<PL>::bytes(lcl), s, a, first);
+    return sp::launch_split<PL>(sp::k_solve_mixed<PL>, num, lcl, sp::SmemMixed<PL>::bytes(lcl), s,
+                                a, first);
   }
   using PL = sp::Plan64<L>;
-  lcl = sp::clamp_lcl(lcl, PL::kMinLcl, PL::kMaxLcl);
-  return sp::launch_split(sp::k_solve64<PL>, num, lcl, 1 << (PL::LNTA - lcl),
-                          sp::Smem64<PL>::bytes(lcl), s, a, first);
+  return sp::launch_split<PL>(sp::k_solve64<PL>, num, lcl, sp::Smem64<PL>::bytes(lcl), s, a, first);
 }
 
 template <int L>
 cudaError_t split_rhs_launch(const RhsArgs& a, int first, int num, int lcl, cudaStream_t s) {
   auto go = [&](auto k, auto pl) {
     using PL = decltype(pl);
-    const int c = sp::clamp_lcl(lcl, PL::kMinLcl, PL::kMaxLcl);
-    return sp::launch_split(k, num, c, 1 << (PL::LNTA - c), sp::SmemRhs<PL>::bytes(c), s, a, first);
+    return sp::launch_split<PL>(k, num, lcl, sp::SmemRhs<PL>::bytes(lcl), s, a, first);
   };
   using PM = sp::PlanMx<L>;
   using PD = sp::Plan64<L>;
@@ -1203,8 +1198,7 @@ template <int L>
 cudaError_t split_linimp_launch(const sp::LinArgs& a, int first, int num, int lcl, cudaStream_t s) {
   auto go = [&](auto k, auto pl) {
     using PL = decltype(pl);
-    const int c = sp::clamp_lcl(lcl, PL::kMinLcl, PL::kMaxLcl);
-    return sp::launch_split(k, num, c, 1 << (PL::LNTA - c), sp::SmemLin<PL>::bytes(c), s, a, first);
+    return sp::launch_split<PL>(k, num, lcl, sp::SmemLin<PL>::bytes(lcl), s, a, first);
   };
   if (a.precision == SGN_PREC_MIXED) return go(sp::k_linimp<sp::PlanMx<L>, df>, sp::PlanMx<L>{});
   return go(sp::k_linimp<sp::Plan64<L>, double>, sp::Plan64<L>{});
@@ -1214,9 +1208,7 @@ template <int L>
 cudaError_t split_field_launch(const sp::FieldArgs& a, int first, int num, int lcl,
                                cudaStream_t s) {
   using PL = sp::Plan64<L>;
-  lcl = sp::clamp_lcl(lcl, PL::kMinLcl, PL::kMaxLcl);
-  return sp::launch_split(sp::k_field<PL>, num, lcl, 1 << (PL::LNTA - lcl),
-                          sp::SmemLin<PL>::bytes(lcl), s, a, first);
+  return sp::launch_split<PL>(sp::k_field<PL>, num, lcl, sp::SmemLin<PL>::bytes(lcl), s, a, first);
 }
 
 }  // namespace sgn

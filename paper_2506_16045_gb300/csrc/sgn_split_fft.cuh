@@ -31,6 +31,7 @@
 // owner's use.
 #pragma once
 #include "sgn_fft1d.cuh"
+#include "sgn_split_plan.h"
 
 namespace sgn {
 namespace sp {
@@ -45,8 +46,7 @@ struct Plan {
   static constexpr int LP = LE - 1, RP = 1 << LP;
   static constexpr int HS = RP > 1 ? RP / 2 : 1;             // half-spectrum slots per butterfly
   static constexpr int NYQ = RP > 1 ? HS : 1;                // thread 0's register of mode n/2
-  // N1 = 64 from n = 2048 (N1 / 2 >= 8 CTAs' rows and N2 / CL >= 8 columns), 32 and 16 below
-  static constexpr int L1 = L >= 11 ? 6 : (L >= 9 ? 5 : 4), L2 = L - L1;
+  static constexpr int L1 = split_log_n1(L), L2 = L - L1;
   static constexpr int N1 = 1 << L1, N2 = 1 << L2;
   // phase A: a stage of radix E, then the rest as evenly as possible; phase B: plain stages
   // as evenly as possible, then the paired one of radix RP
@@ -72,12 +72,8 @@ struct Plan {
   static constexpr int sB(int q) { return L2 - cumB(q) - bitsB(q); }
   static constexpr int LNTA = L - LE;                        // log2 threads of an instance
   static constexpr int W = LNTA > 5 ? 1 << (LNTA - 5) : 1;   // their warps
-  // A CTA has at most 256 threads (512 for float64 at n = 16384), which leaves 128 registers
-  // for each; the largest split keeps 32 threads, 8 columns and a pair of rows per CTA.
-  static constexpr int kMinLcl = LNTA - 8 < 0 ? 0 : (LNTA - 8 > 3 ? 3 : LNTA - 8);
+  static constexpr int kMinLcl = split_min_lcl(L, LE), kMaxLcl = split_max_lcl(L, LE);
   static constexpr int kMaxNT = LNTA - kMinLcl > 8 ? 1 << (LNTA - kMinLcl) : 256;
-  static constexpr int kMax0 = L2 - 3 < LNTA - 5 ? L2 - 3 : LNTA - 5;
-  static constexpr int kMaxLcl = kMax0 < 3 ? kMax0 : 3;
 };
 
 __host__ __device__ constexpr int swz(int a) {
