@@ -81,14 +81,19 @@ typedef enum {
 
 typedef enum {
   SGN_PREC_FP64 = 0,              /* every operation in float64 */
-  SGN_PREC_MIXED = 1              /* float32 inner PCG (matvecs, FFTs, vectors) with float64
-                                     dot accumulation, inside float64 iterative refinement */
+  SGN_PREC_MIXED = 1              /* float32 inner PCG (matvecs, FFTs, vectors), inside iterative
+                                     refinement whose residual and solution are double-float (48
+                                     bits; 2d sizes that are not powers of two: float64).  Dot
+                                     products are of float32 terms, summed per thread in float32
+                                     (double-float on sizes that are not powers of two) and over
+                                     the threads in double-float or float64 */
 } sgn_precision;
 
 typedef struct {
   int iters;                      /* PCG iterations (summed over refinements when mixed) */
   int refinements;                /* float32 inner solves (mixed), 0 for FP64 */
-  double rel_resid_Ainv;          /* sqrt(r.A^{-1}r)/sqrt(b.A^{-1}b) at exit (float64 residual) */
+  double rel_resid_Ainv;          /* sqrt(r.A^{-1}r)/sqrt(b.A^{-1}b) at exit (float64 residual;
+                                     mixed: see SGN_PREC_MIXED) */
   int status;                     /* sgn_status of this instance */
 } sgn_pcg_info;
 
@@ -115,9 +120,9 @@ const char* sgn_status_string(sgn_status s);
  * 6 <= n <= 1024 (such as 384 x 240).  A 2d grid with a side that is not a power of two
  * runs on generic kernels (full complex spectra, mixed-radix row and column passes) for
  * the same calls as the 1d generic sizes, with device-driven solves (one cached graph per
- * precision) and float64 right-hand sides; it takes no batches, no
- * inner-solve forms (sgn_layout_set_form2d, sgn_profile_inner2d) and the same power-of-two
- * options as 1d.  Other sizes: SGN_ERR_UNSUPPORTED_SIZE.  A 2d layout of
+ * precision; the float32 inner solves are persistent launches of one fixed form) and float64
+ * right-hand sides; it takes no batches, no choice of inner-solve form
+ * (sgn_layout_set_form2d, sgn_profile_inner2d) and the same power-of-two options as 1d.  Other sizes: SGN_ERR_UNSUPPORTED_SIZE.  A 2d layout of
  * count > 1 (at most 32) is a batch of instances on one grid (every sgn_grid equal); it
  * serves sgn_spectral_grad, sgn_precond_coeffs, sgn_apply_operator, sgn_precond_solve,
  * sgn_pcg and sgn_pcg_async, whose mixed-precision solves advance the float32 inner PCG of
@@ -496,7 +501,8 @@ sgn_status sgn_profile_read(sgn_ctx* ctx, double* pcg_ms, long long* pcg_calls, 
  * or stops (on = 0) recording.  While recording, mixed solves on the layout take the
  * host-driven refinement loop (a stream synchronisation per pass) so that every persistent
  * launch is bracketed by CUDA events on the solve's stream; results are unchanged.
- * SGN_ERR_INVALID_ARG on a 1d layout. */
+ * SGN_ERR_INVALID_ARG on a 1d layout, SGN_ERR_UNSUPPORTED_SIZE on a grid with a side that is
+ * not a power of two. */
 sgn_status sgn_profile_inner2d(sgn_layout* lay, int on, double* ms, long long* launches,
                                long long* iterations);
 

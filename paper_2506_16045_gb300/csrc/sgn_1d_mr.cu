@@ -1,8 +1,9 @@
-// 1d instances whose n is not a power of two: n = 2^a 3^b 5^c (a >= 1, 6 <= n <= 6144), the
-// grids of §6.1 at sizes the register-blocked power-of-two kernels do not take.  One CTA of
-// kMrNT threads per instance, with a mixed-radix Stockham FFT in shared memory (radices 8,
-// 4, 2 for the power of two, then 5 and 3), two buffers used in turn, and per-size twiddle
-// tables built when the layout is created.  Every spectral operation follows the same
+// 1d instances whose n is not a power of two: n = 2^a 3^b 5^c (a >= 1, 6 <= n <= 16384), the
+// grids of §6.1 at sizes the register-blocked power-of-two kernels do not take.  One CTA per
+// instance (kMrNT threads, 256 for float64 solves up to kMrSmall64), with a mixed-radix Stockham
+// FFT (radices 8, 4, 2 for the power of two, then 5 and 3) in shared memory up to kMrSmemN and in
+// global memory above, two buffers used in turn, and per-size twiddle tables built when the
+// layout is created.  Every spectral operation follows the same
 // formulas as the power-of-two kernels (D = F^{-1}(iK)F with the n/2 wavenumber set to 0,
 // Def:G in its weak form, A^{-1} per mode, PCG with the stopping rule R7, the right-hand
 // side of Eq:DAE_DSWE with Def:bigF):

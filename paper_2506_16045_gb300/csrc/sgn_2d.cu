@@ -338,7 +338,7 @@ __global__ void __launch_bounds__(kMatvecNT, 2) k2_rows_matvec(Modes2d M, int lo
 }
 
 // R2C row pass of K/2 packed pairs of real planes (double storage): pair q packs
-// (src[2q], src[2q+1]); half rows go to dst[2q], dst[2q+1].  `scale` multiplies the input.
+// (src[2q], src[2q+1], null: zero); half rows go to dst[2q], dst[2q+1].
 template <typename T>
 __global__ void __launch_bounds__(kRowNT, 3) k2_rows_r2c(Modes2d M, int log2nx, long long P,
                                                          const void* t64, const void* t32,
@@ -1167,7 +1167,7 @@ void layout2d_destroy(Layout2d& L) {
 }
 
 cudaError_t layout2d_set_inner_form(Layout2d& L, int form, int tile_width) {
-  if (L.mr) return cudaErrorNotSupported;            // no persistent form
+  if (L.mr) return cudaErrorNotSupported;            // one persistent form, and no other
   if (form == L.inner_form && tile_width == L.p_tw) return cudaSuccess;
   drop_solve_graphs(L);
   L.inner_form = form;

@@ -59,8 +59,9 @@ struct Layout2d {
   // non-null while profiling: mixed solves take the host-driven path and bracket each
   // persistent launch with events
   Prof2d* prof = nullptr;
-  // Grids whose nx or ny is not a power of two (sgn_2d_mr.cu): full complex spectra,
-  // host-driven solves.  Of the buffers above only parts and sc are allocated.
+  // Grids whose nx or ny is not a power of two (sgn_2d_mr.cu): full complex spectra, solves by
+  // one cached graph, their float32 inner solves persistent.  Of the buffers above parts, sc,
+  // the staging and the persistent solve's are allocated.
   bool mr = false;
   void* mr_twx = nullptr;      // twiddles of nx: float64, float32, double-float tables
   void* mr_twy = nullptr;      // of ny

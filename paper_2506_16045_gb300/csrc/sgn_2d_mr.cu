@@ -17,8 +17,10 @@
 //                          float64, or float32 inner solves inside float64 refinement)
 //   right-hand side       (Eq:DAE_DSWE with Def:bigF in 2d, float64)
 // A solve runs as one cached graph whose loops are while nodes driven by device-side
-// decisions (build_mr_graph), the float32 inner solves as one persistent launch each; under
-// stream capture the method runs host-driven, a kernel at a time.
+// decisions (build_mr_graph), the float32 inner solves as one persistent launch each on half
+// spectra.  Under stream capture, and where the graph cannot be built, the method runs
+// host-driven, a kernel at a time, its float32 vectors in real space: the same iteration up to
+// rounding.
 #include <cuda_runtime.h>
 
 #include <cmath>

@@ -440,7 +440,8 @@ extern "C" sgn_status sgn_profile_enable(sgn_ctx* ctx, int on) {
 extern "C" sgn_status sgn_profile_inner2d(sgn_layout* lay, int on, double* ms,
                                           long long* launches, long long* iterations) {
   if (check_layout(lay) || lay->dim != 2) return SGN_ERR_INVALID_ARG;
-  if (lay->l2.mr) return SGN_ERR_UNSUPPORTED_SIZE;    // no persistent inner solve
+  // grids with other sides: their persistent inner solves run inside a graph only
+  if (lay->l2.mr) return SGN_ERR_UNSUPPORTED_SIZE;
   DeviceGuard g(lay->device);
   sgn::Layout2d& L = lay->l2;
   double t = 0.0;
@@ -771,7 +772,7 @@ extern "C" sgn_status sgn_layout_set_form2d(sgn_layout* lay, int inner, int tile
       (tile_width != 0 && tile_width != 1 && tile_width != 2 && tile_width != 4))
     return fail(lay ? lay->ctx : nullptr, SGN_ERR_INVALID_ARG, "set_form2d args");
   sgn::Layout2d& L = lay->l2;
-  if (L.mr) return fail(lay->ctx, SGN_ERR_UNSUPPORTED_SIZE, "no inner-solve forms on this grid");
+  if (L.mr) return fail(lay->ctx, SGN_ERR_UNSUPPORTED_SIZE, "one inner-solve form on this grid");
   const int tw = tile_width ? tile_width : sgn::persist2d_tile_width(L.nx, L.ny, 1, L.p_grid);
   if (!sgn::persist2d_tile_ok(L.nx, L.ny, tw))
     return fail(lay->ctx, SGN_ERR_UNSUPPORTED_SIZE, "tile width too wide for this grid");
@@ -790,7 +791,7 @@ extern "C" sgn_status sgn_layout_set_radix2d(sgn_layout* lay, int max_radix) {
 extern "C" sgn_status sgn_layout_set_unit_threads2d(sgn_layout* lay, int threads) {
   if (check_layout(lay) || lay->dim != 2 || (threads != 0 && threads != 128 && threads != 256))
     return fail(lay ? lay->ctx : nullptr, SGN_ERR_INVALID_ARG, "set_unit_threads2d args");
-  if (lay->l2.mr) return fail(lay->ctx, SGN_ERR_UNSUPPORTED_SIZE, "no persistent solve on this grid");
+  if (lay->l2.mr) return fail(lay->ctx, SGN_ERR_UNSUPPORTED_SIZE, "the persistent solve of this grid is fixed");
   SGN_CUDA(lay->ctx, sgn::layout2d_set_unit_threads(lay->l2, threads));
   return SGN_OK;
 }
