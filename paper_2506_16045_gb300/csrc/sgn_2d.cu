@@ -71,6 +71,12 @@ __device__ __forceinline__ void grid_finish(double s, double* parts, Scal2d* sc,
   }
 }
 
+// A norm of b or of a residual that is NaN or infinite ends the solve (the comparisons that follow
+// take it as zero).
+__device__ __forceinline__ void check_finite(Scal2d* sc, double s) {
+  if (!isfinite(s) && sc->status == SGN_OK) sc->status = SGN_ERR_BREAKDOWN;
+}
+
 // =======================================================================================
 // Column pass: tiles of TW columns of K half planes, transposed into shared memory
 // (column c of plane q at buf + (q TW + c) * stride), transformed along y.  In spectral space
@@ -226,7 +232,10 @@ __global__ void __launch_bounds__(NT, NT < 512 ? 2 : 1) k2_cols(Modes2d M, int l
       st_c<T>(a.vout[1], gi, g2);
     }
     if (a.residual) {
-      grid_reduce<NT>(part, a.parts, a.sc, [&](double s) { a.sc->rz64 = s / sigma; });
+      grid_reduce<NT>(part, a.parts, a.sc, [&](double s) {
+        a.sc->rz64 = s / sigma;
+        check_finite(a.sc, s);
+      });
     } else if (a.vdot[0]) {
       grid_reduce<NT>(partw, a.parts, a.sc, [&](double s) {
         Scal2d* sc = a.sc;
@@ -555,7 +564,10 @@ __global__ void __launch_bounds__(256) k2_bnorm(Modes2d M, const void* b1, const
     part += M.weight(c) * ((r1x * r1x + r1y * r1y + r2x * r2x + r2y * r2y) -
                            f * (krx * krx + kry * kry));
   }
-  grid_reduce<256>(part, parts, sc, [&](double s) { sc->bb = s / sigma; });
+  grid_reduce<256>(part, parts, sc, [&](double s) {
+    sc->bb = s / sigma;
+    check_finite(sc, s);
+  });
 }
 
 // v as a double-float: by integer operations where its exponent lets both parts be normal
@@ -1475,7 +1487,8 @@ __global__ void k2_setup_fp64(Scal2d* sc) {
   sc->done = 0;
 }
 
-// A zero (or non-finite) right-hand side gives x = 0, as in the host-driven solve.
+// A zero (or non-finite: status BREAKDOWN) right-hand side gives x = 0, as in the host-driven
+// solve.
 __global__ void k2_finalize(const Scal2d* sc, double* x, long long n) {
   if (sc->bb > 0.0) return;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
@@ -1946,10 +1959,11 @@ cudaError_t launch_pcg2d_batch(Layout2d& first, Batch2d& Bt, const void* tw64, c
   std::vector<double> bnorm(B, 0.0), rn(B, 0.0);
   for (int i = 0; i < B; ++i) {
     bnorm[i] = sqrt(fmax(h[i].bb, 0.0));
-    if (h[i].status != SGN_OK) {
-      fin[i] = 1;
-    } else if (!(bnorm[i] > 0.0)) {
+    const bool breakdown = h[i].status == SGN_ERR_BREAKDOWN;    // b is not finite
+    if ((h[i].status == SGN_OK || breakdown) && !(bnorm[i] > 0.0)) {
       if ((e = cudaMemsetAsync(st_of(i) + 5 * P, 0, sizeof(double) * 2 * P, s))) return e;
+      fin[i] = 1;
+    } else if (h[i].status != SGN_OK) {
       fin[i] = 1;
     }
   }
