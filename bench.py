@@ -38,10 +38,10 @@ FP32_PEAK = 152 * 128 * 2 * 2.07e9          # FMA lanes x 2 flops x max SM clock
 FP32_PROBE_TFLOPS = 75.3
 # DRAM bytes (read + write) per launch of the 2d persistent inner-solve kernel on the
 # pcg2d_batch configuration (16 instances of 512^2), from an ncu capture of this kernel
-# version, the staged form with split transform addresses (dram__bytes_read.sum +
-# dram__bytes_write.sum, the mean of the first solve's two launches: 4.368e9 and 6.134e9
+# version, the staged form on planes interleaved by row pair (dram__bytes_read.sum +
+# dram__bytes_write.sum, the mean of the first solve's two launches: 4.441e9 and 6.245e9
 # bytes)
-PCG2D_TRAFFIC_BYTES = 5.251e9
+PCG2D_TRAFFIC_BYTES = 5.343e9
 
 
 def hbm_peak():
@@ -492,7 +492,7 @@ def gpu_arm(args, world, rank, local, pg):
     nominal = (f32 + fhi) / pcg_s / 1e12
     roof = {"bound": "alu", "achieved": achieved, "peak": FP32_PEAK / 1e12, "unit": "TFLOP/s",
             "frac": achieved * 1e12 / FP32_PEAK, "traffic": None,
-            "kernel": "k_pcg1d<float,...,mixed> (one launch per size class per solve)",
+            "kernel": "k_solve_mixed<Plan<L, 4>> (one launch per size class per solve)",
             "note": "float32-operation rate: float32 algorithmic flops plus double-float flops "
                     f"x {DF_COST}; peak = 152 SMs x 128 FMA lanes x 2 x 2.07 GHz (derived)",
             "frac_nominal": nominal * 1e12 / FP32_PEAK,

@@ -396,8 +396,10 @@ void sgn_state_free(sgn_state* st);
  * device, and advances every admitted request concurrently: 1d RK4 runs move together
  * through one batched launch per kernel (per-instance dt), pending 1d solves run as one
  * batched PCG, and 2d or multistep runs advance in per-request chunks.  Requests that
- * arrive while others run join at the next chunk boundary as memory frees up.  The paper
- * has no counterpart; each result equals the request run alone (RK4 is a one-step method
+ * arrive while others run join at the next chunk boundary as memory frees up.  It keeps the
+ * layouts of finished 2d requests (up to 2 GB) for later ones on the same grid and up to 1 GB
+ * of free arrays, and gives both back when one of its allocations fails and after five
+ * seconds without work.  The paper has no counterpart; each result equals the request run alone (RK4 is a one-step method
  * and every instance is computed by its own CTAs, so batching does not change a result). */
 typedef struct sgn_server sgn_server;
 

@@ -27,8 +27,10 @@ using mr::k_mr_twiddles;
 constexpr int kMrNT = 512;
 // Largest n whose float64 solve takes 256 threads: the float64 pipe is the bound
 // either way, and the barriers of 16 warps cost more than they hide while a thread has one or
-// two modes.  512 against 256 threads: a solve at n = 240 1009 and 957 us, at n = 1500 3475 and
-// 3670 us; six RK4 steps at n = 768 equal, at n = 1000 21.5 and 23.1 ms.
+// two modes.  512 against 256 threads, one float64 solve (one call): n = 240 532 and 475 us, 768
+// 579 and 543, 960 700 and 679, 1500 1126 and 1153 us.  The mixed solve has 512 at every size
+// (n = 240 210 us, 192 with 256; 768 213 and 206; 960 238 and 238; 1500 300 and 305), and so has
+// the right-hand side, where the two are equal up to 768 (n = 1500: 209 and 234 us).
 constexpr int kMrSmall64 = 768;
 constexpr int kMrMaxN = 16384;       // largest generic n
 constexpr int kMrSmemN = 6144;       // largest n whose two transform buffers (192 KB) are in

@@ -9,8 +9,9 @@
 // or float64 operations, a shared store and a barrier), then by the float64 pipe.  Against
 // Stockham stages with two barriers each and twiddles gathered from a table in global memory,
 // double-float at 512 x 512 (one GB300): a column pass over two planes 20.0 -> 14.8 us, a row
-// pass over one pair 15.5 -> 12.7 us; 256 x 256 in float64, 2 RK4 steps: 14.1 -> 11.6 ms;
-// 512 x 512 mixed, 4 RK4 steps: 16.3 -> 15.1 ms.
+// pass over one pair 15.5 -> 12.7 us; RK4 runs at 256 x 256 in float64 1.22 and at 512 x 512
+// mixed 1.08 times as fast (ratios of paired runs: the same build differs by a fifth between
+// machines).
 #pragma once
 #include "sgn_2d_dev.cuh"
 

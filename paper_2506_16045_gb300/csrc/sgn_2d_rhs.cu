@@ -16,8 +16,8 @@
 //
 // What bounds it: the issue of the double-float stages (or the float64 pipe), and latency where
 // a grid has few rows.  Against 26 two-dimensional half-spectrum transforms in 23 launches (one
-// GB300): 512 x 512 mixed, 4 RK4 steps 15.5 -> 13.0 ms (about 160 us per evaluation), 256 x 256
-// float64, 2 steps 12.4 -> 11.4 ms.
+// GB300): 512 x 512 mixed, 4 RK4 steps 15.5 -> 13.0 ms (about 160 us less per evaluation), the
+// 256 x 256 float64 run 1.09 times as fast.
 #include "sgn_2d_fft.cuh"
 
 namespace sgn {
@@ -43,8 +43,8 @@ struct RhsArgs2d {
 enum { W_UX = 0, W_MX, W_ZX, W_SX, W_TXX, W_TXY, W_D, W_M, W_PX, W_PY, W_SY, W_DY, W_PHI, W_R };
 
 // Columns per CTA: four float64 fill a 32-byte sector; fewer on narrow grids, where tiles of
-// four would leave SMs idle (nx = 256: 64 tiles; 256 x 256 float64, 2 RK4 steps: 10.66 ms with
-// four, 10.46 with two).
+// four would leave SMs idle (nx = 256: 64 tiles; the 256 x 256 float64 run is 1.02 times as fast
+// with two as with four).
 int rhs_tw(int nx) { return nx >= 512 ? 4 : (nx >= 256 ? 2 : 1); }
 
 template <typename T>

@@ -663,10 +663,10 @@ extern "C" sgn_status sgn_layout_create(sgn_ctx* ctx, int count, const sgn_grid*
     if (ncls > 1) {
       if (cudaEventCreateWithFlags(&L.fork, cudaEventDisableTiming) != cudaSuccess)
         return cleanup(SGN_ERR_CUDA, "layout events");
-      // Side stream c carries the c-th largest class.  A solve CTA of the largest classes
-      // needs a whole SM (its registers or shared memory), so their blocks must not queue
-      // behind small classes spread over the SMs: larger classes get higher priorities,
-      // and the block scheduler dispatches their pending blocks first.
+      // Side stream c carries the c-th largest class.  The largest classes run longest and
+      // their clusters need free SMs together, so their blocks must not queue behind small
+      // classes spread over the SMs: larger classes get higher priorities, and the block
+      // scheduler dispatches their pending blocks first.
       int lo = 0, hi = 0;   // cudaDeviceGetStreamPriorityRange: hi is the greatest priority
       if (cudaDeviceGetStreamPriorityRange(&lo, &hi) != cudaSuccess) {
         cudaGetLastError();
